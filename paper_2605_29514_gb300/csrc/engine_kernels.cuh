@@ -142,6 +142,15 @@ static __device__ __forceinline__ double philox_uniform(uint64_t seed, uint64_t 
 // CTA-wide helpers
 static __device__ __forceinline__ int tid() { return threadIdx.x; }
 
+// A pointer into dynamic shared memory that the compiler knows to be one: the
+// larger routines are called, not inlined, and would use generic loads.
+template <typename E>
+__device__ __forceinline__ E *in_smem(const void *p) {
+  extern __shared__ __align__(16) char smem_raw[];
+  return reinterpret_cast<E *>(smem_raw + (static_cast<uint32_t>(__cvta_generic_to_shared(p)) -
+                                           static_cast<uint32_t>(__cvta_generic_to_shared(smem_raw))));
+}
+
 // Sum of one double per thread over the CTA: a shuffle reduction per warp,
 // then every thread adds the warps' partial sums (red: kThreads doubles of
 // smem, of which the first kThreads / 32 are used).  Two barriers.
@@ -477,12 +486,147 @@ static __device__ __noinline__ void cgemm_tc(int M, int N, int K, cplx<float> al
   __syncthreads();
 }
 
+// Contractions of small bonds, straight from global memory (the L1 holds the
+// operands): thread t owns column t % N of U output rows t / N + u (kThreads
+// / N), so a row of B is read once for U products and nothing is padded.  The
+// shared-memory tiles below round every product up to 64 x 64 x 16.  For an
+// 8 x 8 x 8 complex128 product that is 128 times its arithmetic, on a pipe of
+// two FP64 FMAs a clock: 68 us in tiles, 8 us here (of which 8 the launch);
+// 200^3 takes 13.4 ms in tiles and 8.3 ms here, so complex128 always comes
+// here (N <= 512 in a sweep; a wider product runs in tiles).  In complex64 the
+// tiles' arithmetic is cheap but their barriers are not: up to 2^16 products
+// the direct form is faster (one d = 5 round at cap 32: 439 ms in tiles, 406
+// ms), beyond that the operands' reuse in shared memory wins (64^3: 15 us in
+// tiles, 22 us).
+template <typename T>
+static __device__ __forceinline__ bool gemm_direct(int M, int N, int K) {
+  if (N > kThreads) return false;
+  return sizeof(T) == 8 || static_cast<int64_t>(M) * N * K <= 65536;
+}
+
+template <typename T, int TA, int TB, int U>
+static __device__ __forceinline__ void cgemm_rows(int M, int N, int K, cplx<T> alpha, const cplx<T> *A, int lda,
+                                                  const cplx<T> *B, int ldb, cplx<T> beta, cplx<T> *C, int ldc) {
+  const int rp = kThreads / N, j = threadIdx.x % N, ty = threadIdx.x / N;
+  if (ty < rp) {
+    for (int i0 = ty; i0 < M; i0 += rp * U) {
+      cplx<T> acc[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) acc[u] = cmake<T>(0, 0);
+#pragma unroll 4
+      for (int k = 0; k < K; ++k) {
+        const cplx<T> b = TB == 0 ? B[static_cast<int64_t>(k) * ldb + j] : cconj(B[static_cast<int64_t>(j) * ldb + k]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = min(i0 + u * rp, M - 1);  // a row past the end repeats the last one, unused
+          const cplx<T> a = TA == 0 ? A[static_cast<int64_t>(i) * lda + k] : cconj(A[static_cast<int64_t>(k) * lda + i]);
+          cfma(acc[u], a, b);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * rp;
+        if (i >= M) break;
+        cplx<T> *c = &C[static_cast<int64_t>(i) * ldc + j];
+        cplx<T> v = cmul(alpha, acc[u]);
+        if (beta.re != T(0) || beta.im != T(0)) v = cadd(v, cmul(beta, *c));
+        *c = v;
+      }
+    }
+  }
+  __syncthreads();
+}
+
+// Larger products in shared-memory tiles of 32 MR x 64 outputs, a slice of
+// kTileK of the k range at a time: thread (ty, tx) of a 32 x 16 grid owns rows
+// ty + 32 a and columns tx + 16 b, so a k step reads MR + 4 elements, which the
+// lanes of a warp read without conflicts, for 4 MR products.  The next slice is fetched from global memory into
+// registers while the present one is multiplied.
+constexpr int kTileK = 8;
+
+template <typename T, int TA, int TB, int MR>
+static __device__ __forceinline__ void cgemm_tiles(int M, int N, int K, cplx<T> alpha, const cplx<T> *A, int lda,
+                                                   const cplx<T> *B, int ldb, cplx<T> beta, cplx<T> *C, int ldc,
+                                                   cplx<T> *tile) {
+  constexpr int RM = 32 * MR, RN = 64, LA = RM + 2, LB = RN + 2;  // padded rows of a slice
+  constexpr int NA = RM * kTileK / kThreads, NB = RN * kTileK / kThreads;
+  static_assert(NA * kThreads == RM * kTileK && NB == 1 && kTileK * (LA + LB) <= kBK * (kBM + kPad + kBN + kPad), "tile");
+  cplx<T> *As = in_smem<cplx<T>>(tile), *Bs = As + kTileK * LA;
+  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+  for (int i0 = 0; i0 < M; i0 += RM)
+    for (int j0 = 0; j0 < N; j0 += RN) {
+      cplx<T> acc[MR][4], pa[NA], pb;
+#pragma unroll
+      for (int a = 0; a < MR; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) acc[a][b] = cmake<T>(0, 0);
+      auto fetch = [&](int k0) {
+#pragma unroll
+        for (int r = 0; r < NA; ++r) {
+          const int e = threadIdx.x + r * kThreads;
+          const int k = TA == 0 ? e % kTileK : e / RM, i = TA == 0 ? e / kTileK : e % RM;
+          const int gi = i0 + i, gk = k0 + k;
+          pa[r] = cmake<T>(0, 0);
+          if (gi < M && gk < K)
+            pa[r] = TA == 0 ? A[static_cast<int64_t>(gi) * lda + gk] : cconj(A[static_cast<int64_t>(gk) * lda + gi]);
+        }
+        const int k = TB == 0 ? threadIdx.x / RN : threadIdx.x % kTileK;
+        const int j = TB == 0 ? threadIdx.x % RN : threadIdx.x / kTileK;
+        const int gj = j0 + j, gk = k0 + k;
+        pb = cmake<T>(0, 0);
+        if (gj < N && gk < K)
+          pb = TB == 0 ? B[static_cast<int64_t>(gk) * ldb + gj] : cconj(B[static_cast<int64_t>(gj) * ldb + gk]);
+      };
+      fetch(0);
+      for (int k0 = 0; k0 < K; k0 += kTileK) {
+#pragma unroll
+        for (int r = 0; r < NA; ++r) {
+          const int e = threadIdx.x + r * kThreads;
+          if (TA == 0) As[(e % kTileK) * LA + e / kTileK] = pa[r];
+          else As[(e / RM) * LA + e % RM] = pa[r];
+        }
+        if (TB == 0) Bs[(threadIdx.x / RN) * LB + threadIdx.x % RN] = pb;
+        else Bs[(threadIdx.x % kTileK) * LB + threadIdx.x / kTileK] = pb;
+        __syncthreads();
+        if (k0 + kTileK < K) fetch(k0 + kTileK);
+#pragma unroll
+        for (int k = 0; k < kTileK; ++k) {
+          cplx<T> av[MR], bv[4];
+#pragma unroll
+          for (int a = 0; a < MR; ++a) av[a] = As[k * LA + ty + 32 * a];
+#pragma unroll
+          for (int b = 0; b < 4; ++b) bv[b] = Bs[k * LB + tx + 16 * b];
+#pragma unroll
+          for (int a = 0; a < MR; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) cfma(acc[a][b], av[a], bv[b]);
+        }
+        __syncthreads();
+      }
+#pragma unroll
+      for (int a = 0; a < MR; ++a) {
+        const int gi = i0 + ty + 32 * a;
+        if (gi >= M) continue;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+          const int gj = j0 + tx + 16 * b;
+          if (gj >= N) continue;
+          cplx<T> *c = &C[static_cast<int64_t>(gi) * ldc + gj];
+          cplx<T> v = cmul(alpha, acc[a][b]);
+          if (beta.re != T(0) || beta.im != T(0)) v = cadd(v, cmul(beta, *c));
+          *c = v;
+        }
+      }
+    }
+  __syncthreads();
+}
+
 // C = alpha * op(A) op(B) + beta * C, all row-major, op = identity (0) or
 // conjugate transpose (1).  op(A) is M x K, op(B) is K x N.  Complex64
 // products large enough to fill the tensor-core tiles run cgemm_tc when the
 // kernel enabled it; the rest (and complex128) run on the CUDA cores below.
 template <typename T, int TA, int TB>
-static __device__ void cgemm(int M, int N, int K, cplx<T> alpha, const cplx<T> *A, int lda,
+static __device__ __noinline__ void cgemm(int M, int N, int K, cplx<T> alpha, const cplx<T> *A, int lda,
                       const cplx<T> *B, int ldb, cplx<T> beta, cplx<T> *C, int ldc,
                       cplx<T> *tile) {
   if constexpr (sizeof(T) == 4) {
@@ -491,76 +635,15 @@ static __device__ void cgemm(int M, int N, int K, cplx<T> alpha, const cplx<T> *
       return;
     }
   }
-  // thread (ty, tx) of a kTY x 16 grid owns rows ty + kTY a (a < kMR) and
-  // columns tx + 16 b (b < 4) of the 64 x 64 output tile
-  constexpr int kTY = kThreads / 16, kMR = kBM / kTY;
-  static_assert(kMR * kTY == kBM && (kBM * kBK) % kThreads == 0, "tile shape");
-  cplx<T> *As = tile;                    // [kBK][kBM + kPad]
-  cplx<T> *Bs = tile + kBK * (kBM + kPad);  // [kBK][kBN + kPad]
-  const int ty = tid() / 16, tx = tid() % 16;
-  const int tilesM = (M + kBM - 1) / kBM, tilesN = (N + kBN - 1) / kBN;
-  for (int t = 0; t < tilesM * tilesN; ++t) {
-    const int i0 = (t / tilesN) * kBM, j0 = (t % tilesN) * kBN;
-    cplx<T> acc[kMR][4];
-#pragma unroll
-    for (int a = 0; a < kMR; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = cmake<T>(0, 0);
-    for (int k0 = 0; k0 < K; k0 += kBK) {
-      // A tile: element (i, k) of op(A)
-#pragma unroll
-      for (int r = 0; r < (kBM * kBK) / kThreads; ++r) {
-        int e = tid() + r * kThreads;
-        int i, k;
-        if (TA == 0) { k = e % kBK; i = e / kBK; } else { i = e % kBM; k = e / kBM; }
-        int gi = i0 + i, gk = k0 + k;
-        cplx<T> v = cmake<T>(0, 0);
-        if (gi < M && gk < K) v = TA == 0 ? A[static_cast<int64_t>(gi) * lda + gk]
-                                          : cconj(A[static_cast<int64_t>(gk) * lda + gi]);
-        As[k * (kBM + kPad) + i] = v;
-      }
-#pragma unroll
-      for (int r = 0; r < (kBN * kBK) / kThreads; ++r) {
-        int e = tid() + r * kThreads;
-        int j, k;
-        if (TB == 0) { j = e % kBN; k = e / kBN; } else { k = e % kBK; j = e / kBK; }
-        int gj = j0 + j, gk = k0 + k;
-        cplx<T> v = cmake<T>(0, 0);
-        if (gj < N && gk < K) v = TB == 0 ? B[static_cast<int64_t>(gk) * ldb + gj]
-                                          : cconj(B[static_cast<int64_t>(gj) * ldb + gk]);
-        Bs[k * (kBN + kPad) + j] = v;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int k = 0; k < kBK; ++k) {
-        cplx<T> av[kMR], bv[4];
-#pragma unroll
-        for (int a = 0; a < kMR; ++a) av[a] = As[k * (kBM + kPad) + ty + kTY * a];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) bv[b] = Bs[k * (kBN + kPad) + tx + 16 * b];
-#pragma unroll
-        for (int a = 0; a < kMR; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) cfma(acc[a][b], av[a], bv[b]);
-      }
-      __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < kMR; ++a) {
-      int gi = i0 + ty + kTY * a;
-      if (gi >= M) continue;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        int gj = j0 + tx + 16 * b;
-        if (gj >= N) continue;
-        cplx<T> *c = &C[static_cast<int64_t>(gi) * ldc + gj];
-        cplx<T> v = cmul(alpha, acc[a][b]);
-        if (beta.re != T(0) || beta.im != T(0)) v = cadd(v, cmul(beta, *c));
-        *c = v;
-      }
-    }
+  if (gemm_direct<T>(M, N, K)) {
+    const int rp = kThreads / N;
+    if (M <= rp) cgemm_rows<T, TA, TB, 1>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    else if (M <= 2 * rp) cgemm_rows<T, TA, TB, 2>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    else cgemm_rows<T, TA, TB, 4>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+    return;
   }
-  __syncthreads();
+  if (M <= 64) cgemm_tiles<T, TA, TB, 2>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, tile);
+  else cgemm_tiles<T, TA, TB, 4>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, tile);
 }
 
 static __device__ __forceinline__ int warp_id() { return threadIdx.x >> 5; }
@@ -629,8 +712,10 @@ static __device__ void wy_t_factor(int mr, int jb, int nb, int ldv, const cplx<T
 // (column j holds u_j in rows j..m-1; rows above are not written) so that
 // form_q can build Q explicitly.
 template <typename T>
-static __device__ void qr_r_inplace(int m, int n, cplx<T> *B, int ld, cplx<T> *pbuf, int pbuf_elems, double *red,
-                             double *dm, cplx<T> *vstore = nullptr) {
+static __device__ __noinline__ void qr_r_inplace(int m, int n, cplx<T> *B, int ld, cplx<T> *pbuf_, int pbuf_elems,
+                                                 double *red_, double *dm_, cplx<T> *vstore = nullptr) {
+  cplx<T> *pbuf = in_smem<cplx<T>>(pbuf_);
+  double *red = in_smem<double>(red_), *dm = in_smem<double>(dm_);
   const int steps = min(m, n);
   const int nb = qr_panel_width(m, pbuf_elems);
   // rows of the panel padded to an odd number of elements, so that a column
@@ -807,7 +892,9 @@ static __device__ void qr_r_inplace(int m, int n, cplx<T> *B, int ld, cplx<T> *p
 // or right of it (the columns left of panel p are unit vectors its
 // reflectors do not touch).  Same shared-memory needs as qr_r_inplace.
 template <typename T>
-static __device__ void form_q(int m, int steps, const cplx<T> *vstore, cplx<T> *Q, cplx<T> *pbuf, int pbuf_elems) {
+static __device__ __noinline__ void form_q(int m, int steps, const cplx<T> *vstore, cplx<T> *Q, cplx<T> *pbuf_,
+                                           int pbuf_elems) {
+  cplx<T> *pbuf = in_smem<cplx<T>>(pbuf_);
   const int nb = qr_panel_width(m, pbuf_elems);
   const int ldv = nb + 1;
   cplx<T> *Vp = pbuf;
@@ -974,7 +1061,7 @@ constexpr int kMaxBlockedSweepsF = 30, kMaxBlockedSweepsD = 40;
 
 // Unblocked: C and V wherever they are (shared memory for small problems).
 template <typename T>
-static __device__ int svd_onesided(int m, int n, cplx<T> *C, cplx<T> *V, T *sig2, int *flag, double *red) {
+static __device__ __noinline__ int svd_onesided(int m, int n, cplx<T> *C, cplx<T> *V, T *sig2, int *flag, double *red) {
   const T negligible = onesided_prologue<T>(m, n, C, V, red);
   const T tol = onesided_tol<T>(m);
   const int max_sweeps = sizeof(T) == 4 ? kMaxSweepsF : kMaxSweepsD;
@@ -1251,7 +1338,7 @@ static __device__ bool cross_visit_dispatch(int m, cplx<T> *C, int c0, int wI, i
 // with cross_visit_regs (blocks of 16 columns); the blocks alone are still
 // staged in shared memory.
 template <typename T>
-static __device__ int svd_onesided_blocked(int m, int n, cplx<T> *C, cplx<T> *V, T *sig2, int *flag,
+static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C, cplx<T> *V, T *sig2, int *flag,
                                      double *red, cplx<T> *sbuf, int sbuf_elems, float *rv_wrk = nullptr) {
   const T negligible = onesided_prologue<T>(m, n, C, V, red);
   const T tol = onesided_tol<T>(m);
@@ -1414,7 +1501,7 @@ static __device__ int svd_onesided_blocked(int m, int n, cplx<T> *C, cplx<T> *V,
 // leave X orthonormal only to about sqrt(#rotations) eps; this brings it back
 // to the rounding level of one product.  G and Y are k x k and n x k scratch.
 template <typename T>
-static __device__ void reorthonormalize(int n, int k, cplx<T> *X, cplx<T> *G, cplx<T> *Y, cplx<T> *tile) {
+static __device__ __noinline__ void reorthonormalize(int n, int k, cplx<T> *X, cplx<T> *G, cplx<T> *Y, cplx<T> *tile) {
   const cplx<T> one = cmake<T>(1, 0), zero = cmake<T>(0, 0);
   cgemm<T, 1, 0>(k, k, n, one, X, k, X, k, zero, G, k, tile);
   for (int e = tid(); e < k * k; e += kThreads) {
@@ -1637,7 +1724,7 @@ __device__ __forceinline__ cplx<T> *site_ptr(const EngineParams &P, int64_t shot
 // doubled when dl, right bond doubled when dr; the (alpha, l) index is
 // alpha * chl + l.
 template <typename T>
-static __device__ void materialize(const MpoSpec<T> &sp, const uint64_t *ppx, const uint64_t *ppz, int k,
+static __device__ __noinline__ void materialize(const MpoSpec<T> &sp, const uint64_t *ppx, const uint64_t *ppz, int k,
                             const cplx<T> *A, int chl, int chr, bool dl, bool dr, cplx<T> *out) {
   if (sp.kind == MPO_PROJ_Z) {
     // (I + s Z_S)/2 written without its two cancelling branches: the bond
@@ -1647,11 +1734,11 @@ static __device__ void materialize(const MpoSpec<T> &sp, const uint64_t *ppx, co
     // of two numbers of order one.
     const bool in_s = (ppz[k >> 6] >> (k & 63)) & 1;
     const int Dl = dl ? 2 * chl : chl, Dr = dr ? 2 * chr : chr;
-    const int64_t total = static_cast<int64_t>(Dl) * 2 * Dr;
-    for (int64_t e = tid(); e < total; e += kThreads) {
-      const int R = static_cast<int>(e % Dr);
-      const int sb = static_cast<int>((e / Dr) % 2);
-      const int L = static_cast<int>(e / (2 * Dr));
+    const int total = Dl * 2 * Dr;
+    for (int e = tid(); e < total; e += kThreads) {
+      const int R = e % Dr;
+      const int sb = (e / Dr) & 1;
+      const int L = e / (2 * Dr);
       const int al = dl ? L / chl : 0, l = dl ? L % chl : L;
       const int be = dr ? R / chr : sp.par, r = dr ? R % chr : R;
       const bool keep = in_s ? ((al ^ sb) == be) : (al == be);
@@ -1663,11 +1750,11 @@ static __device__ void materialize(const MpoSpec<T> &sp, const uint64_t *ppx, co
   site_op(sp, ppx, ppz, k, 0, op0);
   site_op(sp, ppx, ppz, k, 1, op1);
   const int Dl = dl ? 2 * chl : chl, Dr = dr ? 2 * chr : chr;
-  const int64_t total = static_cast<int64_t>(Dl) * 2 * Dr;
-  for (int64_t e = tid(); e < total; e += kThreads) {
-    int R = static_cast<int>(e % Dr);
-    int s = static_cast<int>((e / Dr) % 2);
-    int L = static_cast<int>(e / (2 * Dr));
+  const int total = Dl * 2 * Dr;
+  for (int e = tid(); e < total; e += kThreads) {
+    int R = e % Dr;
+    int s = (e / Dr) & 1;
+    int L = e / (2 * Dr);
     int al = dl ? L / chl : -1, l = dl ? L % chl : L;
     int be = dr ? R / chr : -1, r = dr ? R % chr : R;
     cplx<T> val = cmake<T>(0, 0);
@@ -1688,21 +1775,25 @@ static __device__ void materialize(const MpoSpec<T> &sp, const uint64_t *ppx, co
   }
 }
 
-// Keep count at one bond from eigenvalues sorted in decreasing order.
+// Keep count at one bond from eigenvalues sorted in decreasing order, by one
+// warp (a lane's square roots are independent; one thread would do them in a
+// chain).
 template <typename T>
 static __device__ int keep_count(const T *lam_sorted, int n, int cap, double cutoff, double delta) {
-  double s1 = sqrt(fmax(static_cast<double>(lam_sorted[0]), 0.0));
+  auto sigma = [&](int i) { return sqrt(fmax(static_cast<double>(lam_sorted[i]), 0.0)); };
+  auto above = [&](int m, double thr) {
+    int k = 0;
+    for (int i = 0; i < m; i += 32)
+      k += __popc(__ballot_sync(0xffffffffu, i + lane_id() < m && sigma(min(i + lane_id(), m - 1)) > thr));
+    return k;
+  };
+  const double s1 = sigma(0);
   if (!(s1 > 0.0)) return 1;
-  int k = 0;
-  for (int i = 0; i < n; ++i)
-    if (sqrt(fmax(static_cast<double>(lam_sorted[i]), 0.0)) > cutoff * s1) ++k;
+  int k = above(n, cutoff * s1);
   if (k < 1) k = 1;
   if (k > cap) {
-    double thr = sqrt(fmax(static_cast<double>(lam_sorted[cap]), 0.0)) + delta * s1;
-    int kk = 0;
-    for (int i = 0; i < cap; ++i)
-      if (sqrt(fmax(static_cast<double>(lam_sorted[i]), 0.0)) > thr) ++kk;
-    k = kk < 1 ? 1 : kk;
+    k = above(cap, sigma(cap) + delta * s1);
+    if (k < 1) k = 1;
   }
   return k;
 }
@@ -1717,7 +1808,7 @@ static __device__ int keep_count(const T *lam_sorted, int n, int cap, double cut
 //   Left across site k: A_k^dag as a (2 chi_{k+1}) x chi_k matrix = Q R;
 //   site k becomes Q^dag and A_{k-1} <- A_{k-1} R^dag.
 template <typename T>
-static __device__ void mps_move_center(const EngineParams &P, const Smem<T> &S, int64_t shot, const Scratch<T> &X,
+static __device__ __noinline__ void mps_move_center(const EngineParams &P, const Smem<T> &S, int64_t shot, const Scratch<T> &X,
                                 int target) {
   int *chi = S.chi;
   const cplx<T> one = cmake<T>(1, 0), zero = cmake<T>(0, 0);
@@ -1792,14 +1883,15 @@ static __device__ void mps_move_center(const EngineParams &P, const Smem<T> &S, 
 // mps_finish then runs the truncating right sweep; the centre ends at a and the
 // state is renormalised.
 template <typename T>
-static __device__ double mps_prepare(const EngineParams &P, const Smem<T> &S, int64_t shot,
-                              const Scratch<T> &X, int a, int b) {
+static __device__ __noinline__ double mps_prepare(const EngineParams &P, const Smem<T> &S, int64_t shot,
+                              const Scratch<T> &X, int a, int b, bool want_norm) {
   const MpoSpec<T> &sp = *S.spec;
   int *chi = S.chi;
   if (a == b) {
     cplx<T> *A = site_ptr<T>(P, shot, a);
     materialize(sp, S.ppx, S.ppz, a, A, chi[a], chi[a + 1], false, false, X.t);
     __syncthreads();
+    if (!want_norm) return 0.0;
     const int64_t tot = static_cast<int64_t>(chi[a]) * 2 * chi[a + 1];
     double nrm = 0;
     for (int64_t e = tid(); e < tot; e += kThreads) nrm += cabs2d(X.t[e]);
@@ -1838,19 +1930,16 @@ static __device__ double mps_prepare(const EngineParams &P, const Smem<T> &S, in
   }
   __syncthreads();
   const cplx<T> one = cmake<T>(1, 0), zero = cmake<T>(0, 0);
-  const int cap = P.chi_cap;
-  (void)cap;
   // left sweep: R factor of the left part through site k, for k = a..b-1
   // (R at bond a is the identity: sites left of a are left-canonical).
   for (int k = a; k < b; ++k) {
     const int Dl = Dbond(k), Dr = Dbond(k + 1);
     const cplx<T> *Ak = X.ap + S.off[k - a];
     int m;
+    const cplx<T> *src = X.t;
     if (k == a) {
       m = 2 * Dl;
-      const int64_t tot = static_cast<int64_t>(m) * Dr;
-      for (int64_t e = tid(); e < tot; e += kThreads) X.t[e] = Ak[e];
-      __syncthreads();
+      src = Ak;
     } else {
       const int r = S.rdim[k - a];
       const cplx<T> *Rk = X.g + S.goff[k - a];
@@ -1863,18 +1952,25 @@ static __device__ double mps_prepare(const EngineParams &P, const Smem<T> &S, in
       __syncthreads();
       return 0.0;
     }
-    qr_r_inplace<T>(m, Dr, X.t, Dr, S.jbuf, P.svd_elems, S.red, S.dmisc + 4);
     if (tid() == 0) S.dmisc[D_FLOPS] += qr_flops(m, Dr);
     const int rn = min(m, Dr);
     cplx<T> *Rout = X.g + S.goff[k + 1 - a];
+    if (src != X.t) {
+      for (int e = tid(); e < m * Dr; e += kThreads) X.t[e] = src[e];
+      __syncthreads();
+    }
+    qr_r_inplace<T>(m, Dr, X.t, Dr, S.jbuf, P.svd_elems, S.red, S.dmisc + 4);
     for (int e = tid(); e < rn * Dr; e += kThreads) Rout[e] = X.t[e];
     if (tid() == 0) S.rdim[k + 1 - a] = rn;
     __syncthreads();
   }
-  // squared norm: || R_b A'_b ||_F^2 (the right part beyond b is right-canonical)
+  // R_b A'_b, the first matrix of the right sweep, stays in X.y for mps_finish;
+  // squared norm of the state: its Frobenius norm (the right part beyond b is
+  // right-canonical)
   {
     const int Dl = Dbond(b), n2 = 2 * Dbond(b + 1), r = S.rdim[b - a];
     cgemm<T, 0, 0>(r, n2, Dl, one, X.g + S.goff[b - a], Dl, X.ap + S.off[b - a], n2, zero, X.y, n2, S.tile);
+    if (!want_norm) return 0.0;
     double nrm = 0;
     for (int e = tid(); e < r * n2; e += kThreads) nrm += cabs2d(X.y[e]);
     return block_sum(nrm, S.red);
@@ -1882,7 +1978,7 @@ static __device__ double mps_prepare(const EngineParams &P, const Smem<T> &S, in
 }
 
 template <typename T>
-static __device__ void mps_finish(const EngineParams &P, const Smem<T> &S, int64_t shot, const Scratch<T> &X,
+static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem<T> &S, int64_t shot, const Scratch<T> &X,
                            int a, int b) {
   const MpoSpec<T> &sp = *S.spec;
   int *chi = S.chi;
@@ -1914,8 +2010,8 @@ static __device__ void mps_finish(const EngineParams &P, const Smem<T> &S, int64
     const int n2 = 2 * kappa;
     const int r = S.rdim[k - a];
     const cplx<T> *Rk = X.g + S.goff[k - a];
-    // C = R_k M (r x n2), then its SVD
-    cgemm<T, 0, 0>(r, n2, Dl, one, Rk, Dl, M, n2, zero, X.y, n2, S.tile);
+    // C = R_k M (r x n2; mps_prepare left the first one in X.y), then its SVD
+    if (k < b) cgemm<T, 0, 0>(r, n2, Dl, one, Rk, Dl, M, n2, zero, X.y, n2, S.tile);
     prof_mark(S.dmisc, PROF_RIGHT, tp);
     const bool in_smem = r * n2 + n2 * n2 <= P.svd_elems;
     cplx<T> *Cc = in_smem ? S.jbuf : X.h;
@@ -2044,18 +2140,21 @@ static __device__ void mps_finish(const EngineParams &P, const Smem<T> &S, int64
     sort_desc<T>(n2, X.lam, S.perm);
     for (int i = tid(); i < n2; i += kThreads) S.lam[i] = X.lam[S.perm[i]];
     __syncthreads();
-    if (tid() == 0) {
-      int kmax = min(cap, P.chimax[k]);
-      int keep = keep_count<T>(S.lam, n2, kmax, P.cutoff, P.delta);
-      if (keep > kmax) keep = kmax;
+    if (warp_id() == 0) {
+      const int kmax = min(cap, P.chimax[k]);
+      const int keep = min(keep_count<T>(S.lam, n2, kmax, P.cutoff, P.delta), kmax);
       double tot = 0, drop = 0;
-      for (int i = 0; i < n2; ++i) {
-        double l = fmax(static_cast<double>(S.lam[i]), 0.0);
+      for (int i = lane_id(); i < n2; i += 32) {
+        const double l = fmax(static_cast<double>(S.lam[i]), 0.0);
         tot += l;
         if (i >= keep) drop += l;
       }
-      if (tot > 0) S.dmisc[D_DISC] += drop / tot;
-      S.misc[M_KEEP] = keep;
+      tot = warp_sum(tot);
+      drop = warp_sum(drop);
+      if (tid() == 0) {
+        if (tot > 0) S.dmisc[D_DISC] += drop / tot;
+        S.misc[M_KEEP] = keep;
+      }
     }
     __syncthreads();
     const int keep = S.misc[M_KEEP];
@@ -2114,7 +2213,7 @@ static __device__ void mps_finish(const EngineParams &P, const Smem<T> &S, int64
 // <phi| i^m X^x Z^z |phi> over sites [a, b] (centre inside, so the rest of
 // the chain contracts to the identity).  Returns the real part.
 template <typename T>
-static __device__ double mps_expect(const EngineParams &P, const Smem<T> &S, int64_t shot,
+static __device__ __noinline__ double mps_expect(const EngineParams &P, const Smem<T> &S, int64_t shot,
                              const Scratch<T> &X, int a, int b, int m) {
   const int *chi = S.chi;
   const cplx<T> one = cmake<T>(1, 0), zero = cmake<T>(0, 0);
@@ -2401,18 +2500,19 @@ __global__ void __launch_bounds__(kThreads, 1) round_kernel(EngineParams P) {
             if (meas) m = conj_rows(S.tx, S.tz, S.tm, W, n + op.a, -1, S.ppx, S.ppz);
             else if (op.pauli == 0) m = conj_rows(S.tx, S.tz, S.tm, W, n + op.a, n + op.b, S.ppx, S.ppz);
             else m = conj_rows(S.tx, S.tz, S.tm, W, op.a, op.b, S.ppx, S.ppz);
-            int lo = n, hi = -1, j = -1, xany = 0, xz = 0;
-            for (int q = 0; q < n; ++q) {
-              bool x = (S.ppx[q >> 6] >> (q & 63)) & 1, z = (S.ppz[q >> 6] >> (q & 63)) & 1;
-              if (x || z) { lo = min(lo, q); hi = max(hi, q); }
-              if (x && j < 0) j = q;
-              xany |= x;
-              xz += x && z;
+            int lo = n, hi = -1, j = -1, xz = 0;
+            for (int w = 0; w < W; ++w) {
+              const uint64_t x = S.ppx[w], any = x | S.ppz[w];
+              if (any) {
+                if (hi < 0) lo = 64 * w + __ffsll(any) - 1;
+                hi = 64 * w + 63 - __clzll(any);
+              }
+              if (x && j < 0) j = 64 * w + __ffsll(x) - 1;
+              xz += popc64(x & S.ppz[w]);
             }
-            int c = S.misc[M_CENTER];
+            const int xany = j >= 0;
             S.misc[M_LO] = lo;
             S.misc[M_HI] = hi;
-            (void)c;
             S.misc[M_A] = lo;
             S.misc[M_B] = hi;
             S.misc[M_J] = j;
@@ -2421,10 +2521,11 @@ __global__ void __launch_bounds__(kThreads, 1) round_kernel(EngineParams P) {
             MpoSpec<T> &sp = *S.spec;
             sp.lo = lo; sp.hi = hi; sp.j = j;
             if (!meas) {
-              double th = P.theta[op.idx];
-              cplx<T> w1 = cmul(cmake<T>(0, static_cast<T>(-sin(th))), ipow<T>(m));
+              double sn, cs;
+              sincos(P.theta[op.idx], &sn, &cs);
+              cplx<T> w1 = cmul(cmake<T>(0, static_cast<T>(-sn)), ipow<T>(m));
               sp.kind = MPO_ROT;
-              sp.w0 = cmake<T>(static_cast<T>(cos(th)), 0);
+              sp.w0 = cmake<T>(static_cast<T>(cs), 0);
               sp.w1 = w1;
             }
             if (lo > hi) S.misc[M_FAIL] = STN_ENUMERIC;  // identity Pauli cannot occur
@@ -2470,7 +2571,7 @@ __global__ void __launch_bounds__(kThreads, 1) round_kernel(EngineParams P) {
             if (tid() == 0) set_meas_spec<T>(S, small);
             __syncthreads();
             prof_mark(S.dmisc, PROF_EXPECT, tq);
-            const double ps = fmin(1.0, fmax(0.0, mps_prepare<T>(P, S, shot, X, a, b)));
+            const double ps = fmin(1.0, fmax(0.0, mps_prepare<T>(P, S, shot, X, a, b, true)));
             prof_mark(S.dmisc, PROF_LEFT, tq);
             if (tid() == 0) {
               double p0 = small == 0 ? ps : 1.0 - ps;
@@ -2498,13 +2599,13 @@ __global__ void __launch_bounds__(kThreads, 1) round_kernel(EngineParams P) {
             lidx = S.misc[M_LIDX];
             outcome = S.misc[M_OUTCOME];
             tq = clock64();
-            if (outcome != small) mps_prepare<T>(P, S, shot, X, a, b);
+            if (outcome != small) mps_prepare<T>(P, S, shot, X, a, b, false);
             __syncthreads();
             prof_mark(S.dmisc, PROF_LEFT, tq);
             mps_finish<T>(P, S, shot, X, a, b);
           } else {
             long long tq = clock64();
-            mps_prepare<T>(P, S, shot, X, a, b);
+            mps_prepare<T>(P, S, shot, X, a, b, false);
             __syncthreads();
             prof_mark(S.dmisc, PROF_LEFT, tq);
             mps_finish<T>(P, S, shot, X, a, b);
@@ -2589,6 +2690,34 @@ __global__ void init_kernel(EngineParams P) {
 }
 
 // ---------------------------------------------------------------------------
+// The truncation sweep's SVD on its own: right singular vectors V (n x n,
+// column-major; columns from min(m, n) on, or beyond, are zero) and
+// squared singular values of the row-major m x n matrix A, on the copy in
+// `work` (work may be A): R factor, Jacobi on X = R^dag (n x k), V = normalised
+// columns of X.
+template <typename T>
+static __device__ void svd_bond(int m, int n, const cplx<T> *A, cplx<T> *work, cplx<T> *V, T *sig2, cplx<T> *buf,
+                                cplx<T> *uv, double *red, double *dm, int *flag, float *rv_wrk) {
+  if (work != A)
+    for (int e = tid(); e < m * n; e += kThreads) work[e] = A[e];
+  __syncthreads();
+  qr_r_inplace<T>(m, n, work, n, buf, SvdSmem<T>::elems, red, dm);
+  const int k = min(m, n);
+  const bool regs = sizeof(T) == 4 && k > 16 && n <= kThreads;
+  const bool x_smem = !regs && n * k <= SvdSmem<T>::elems;
+  cplx<T> *Xc = x_smem ? buf : work;
+  for (int e = tid(); e < n * k; e += kThreads) Xc[e] = cconj(work[e]);
+  __syncthreads();
+  if (x_smem) svd_onesided<T>(n, k, Xc, nullptr, sig2, flag, red);
+  else svd_onesided_blocked<T>(n, k, Xc, nullptr, sig2, flag, red, buf, SvdSmem<T>::elems, regs ? rv_wrk : nullptr);
+  for (int e = tid(); e < n * n; e += kThreads) {
+    const int c = e / n;
+    const T l = c < k ? sig2[c] : T(0);
+    V[e] = l > T(0) ? cscale(Xc[e], T(1) / sqrt(l)) : cmake<T>(0, 0);
+  }
+  for (int c = k + tid(); c < n; c += kThreads) sig2[c] = T(0);
+}
+
 // Kernel-level checks of the dense routines on one CTA (complex elements of
 // precision T, column-major C/V for the SVD, row-major B for the QR).
 template <typename T>
@@ -2610,24 +2739,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
     qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, red, dm, vstore);
     form_q<T>(m, min(m, n), vstore, V, buf, SvdSmem<T>::elems);
   } else if (use_smem == 3) {
-    // the large-bond path of the truncation sweep: A row-major (m x n),
-    // R factor, Jacobi on X = R^dag (n x k), V = normalised columns of X
-    qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, red, dm);
-    const int k = min(m, n);
-    const bool regs = sizeof(T) == 4 && k > 16 && n <= kThreads;
-    const bool x_smem = !regs && n * k <= SvdSmem<T>::elems;
-    cplx<T> *Xc = x_smem ? buf : A;
-    for (int e = tid(); e < n * k; e += kThreads) Xc[e] = cconj(A[e]);
-    __syncthreads();
-    if (x_smem) svd_onesided<T>(n, k, Xc, nullptr, sig2, flag, red);
-    else svd_onesided_blocked<T>(n, k, Xc, nullptr, sig2, flag, red, buf, SvdSmem<T>::elems,
-                                 regs ? rv_wrk : nullptr);
-    for (int e = tid(); e < n * n; e += kThreads) {
-      const int c = e / n;
-      const T l = c < k ? sig2[c] : T(0);
-      V[e] = l > T(0) ? cscale(Xc[e], T(1) / sqrt(l)) : cmake<T>(0, 0);
-    }
-    for (int c = k + tid(); c < n; c += kThreads) sig2[c] = T(0);
+    svd_bond<T>(m, n, A, A, V, sig2, buf, uv, red, dm, flag, rv_wrk);
   } else {
     cplx<T> *C = A, *VV = V;
     if (use_smem == 1) {
@@ -2955,7 +3067,7 @@ __global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(EngineParams P, do
       const int tgt = c0 < lo ? lo : (c0 > hi ? hi : c0);
       if (tgt != c0) mps_move_center<T>(P, S, shot, X, tgt);
       if (S.misc[M_FAIL]) break;
-      mps_prepare<T>(P, S, shot, X, lo, hi);
+      mps_prepare<T>(P, S, shot, X, lo, hi, false);
       __syncthreads();
       mps_finish<T>(P, S, shot, X, lo, hi);
       __syncthreads();

@@ -1,0 +1,46 @@
+"""The untiled contraction of small bonds at the sizes where it can go wrong:
+one column, one row, row counts around the rows in flight, the widest output.
+References are numpy in float64; bounds are rounding levels."""
+
+import numpy as np
+import pytest
+
+import paper_2605_29514_gb300 as stn
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+CDT = {0: torch.complex128, 1: torch.complex64}
+RDT = {0: torch.float64, 1: torch.float32}
+EPS = {0: 2.2e-16, 1: 1.2e-7}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    stn.build()
+
+
+def cmat(rng, m, n, precision):
+    return (rng.normal(size=(m, n)) + 1j * rng.normal(size=(m, n))).astype([np.complex128, np.complex64][precision])
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("op_a,op_b", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("m,n,k", [(1, 1, 1), (1, 511, 3), (2, 512, 5), (3, 513, 2), (512, 1, 7), (513, 1, 2),
+                                   (9, 257, 4), (17, 31, 33), (32, 64, 32), (32, 64, 33)])
+def test_untiled_contraction(precision, op_a, op_b, m, n, k):
+    rng = np.random.default_rng(m + 100 * n + 7 * k)
+    a = cmat(rng, *((k, m) if op_a else (m, k)), precision)
+    b = cmat(rng, *((n, k) if op_b else (k, n)), precision)
+    c0 = cmat(rng, m, n, precision)
+    da, db, dc = (torch.tensor(x, device="cuda") for x in (a, b, c0))
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    stn.dense_cgemm(precision, op_a, op_b, m, n, k, da.data_ptr(), a.shape[1], db.data_ptr(), b.shape[1],
+                    dc.data_ptr(), n, st.data_ptr(), alpha=0.5 - 0.25j, beta=-2.0)
+    oa, ob = (x.astype(np.complex128) for x in (a, b))
+    oa, ob = (oa.conj().T if op_a else oa), (ob.conj().T if op_b else ob)
+    ref = (0.5 - 0.25j) * (oa @ ob) - 2.0 * c0
+    scale = np.abs(oa) @ np.abs(ob) + 2.0 * np.abs(c0)
+    assert (np.abs(dc.cpu().numpy() - ref) / scale).max() < 4 * (k + 4) * EPS[precision]
