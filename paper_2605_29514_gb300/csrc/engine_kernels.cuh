@@ -1059,6 +1059,10 @@ static __device__ void onesided_epilogue(int m, int n, const cplx<T> *C, T *sig2
 constexpr int kMaxSweepsF = 15, kMaxSweepsD = 20;
 constexpr int kMaxBlockedSweepsF = 30, kMaxBlockedSweepsD = 40;
 
+}  // namespace stn
+#include "small_bond.cuh"
+namespace stn {
+
 // Unblocked: C and V wherever they are (shared memory for small problems).
 template <typename T>
 static __device__ __noinline__ int svd_onesided(int m, int n, cplx<T> *C, cplx<T> *V, T *sig2, int *flag, double *red) {
@@ -1822,12 +1826,17 @@ static __device__ __noinline__ void mps_move_center(const EngineParams &P, const
       return;
     }
     cplx<T> *A = site_ptr<T>(P, shot, c), *Bn = site_ptr<T>(P, shot, c + 1);
-    for (int e = tid(); e < m * r; e += kThreads) X.t[e] = A[e];
-    __syncthreads();
-    qr_r_inplace<T>(m, r, X.t, r, S.jbuf, P.svd_elems, S.red, S.dmisc + 4, X.h);
-    form_q<T>(m, steps, X.h, X.y, S.jbuf, P.svd_elems);
-    cgemm<T, 0, 0>(steps, 2 * r2, r, one, X.t, r, Bn, 2 * r2, zero, X.w, 2 * r2, S.tile);
-    for (int e = tid(); e < m * steps; e += kThreads) A[e] = X.y[e];
+    if (qr_small_elems(m, r, true) <= P.svd_elems) {
+      qr_small<T>(m, r, A, r, false, X.t, steps, A, S.jbuf);
+      cgemm<T, 0, 0>(steps, 2 * r2, r, one, X.t, r, Bn, 2 * r2, zero, X.w, 2 * r2, S.tile);
+    } else {
+      for (int e = tid(); e < m * r; e += kThreads) X.t[e] = A[e];
+      __syncthreads();
+      qr_r_inplace<T>(m, r, X.t, r, S.jbuf, P.svd_elems, S.red, S.dmisc + 4, X.h);
+      form_q<T>(m, steps, X.h, X.y, S.jbuf, P.svd_elems);
+      cgemm<T, 0, 0>(steps, 2 * r2, r, one, X.t, r, Bn, 2 * r2, zero, X.w, 2 * r2, S.tile);
+      for (int e = tid(); e < m * steps; e += kThreads) A[e] = X.y[e];
+    }
     for (int e = tid(); e < steps * 2 * r2; e += kThreads) Bn[e] = X.w[e];
     if (tid() == 0) {
       chi[c + 1] = steps;
@@ -1846,17 +1855,22 @@ static __device__ __noinline__ void mps_move_center(const EngineParams &P, const
       return;
     }
     cplx<T> *A = site_ptr<T>(P, shot, c), *Am = site_ptr<T>(P, shot, c - 1);
-    for (int e = tid(); e < m * l; e += kThreads) {
-      const int j = e / l, i = e % l;  // X.t[j][i] = conj(A[i][j]), A as l x 2r
-      X.t[e] = cconj(A[static_cast<int64_t>(i) * m + j]);
-    }
-    __syncthreads();
-    qr_r_inplace<T>(m, l, X.t, l, S.jbuf, P.svd_elems, S.red, S.dmisc + 4, X.h);
-    form_q<T>(m, steps, X.h, X.y, S.jbuf, P.svd_elems);
-    cgemm<T, 0, 1>(2 * ll, steps, l, one, Am, l, X.t, l, zero, X.w, steps, S.tile);
-    for (int e = tid(); e < steps * m; e += kThreads) {
-      const int k = e / m, j = e % m;
-      A[e] = cconj(X.y[static_cast<int64_t>(j) * steps + k]);
+    if (qr_small_elems(m, l, true) <= P.svd_elems) {
+      qr_small<T>(m, l, A, m, true, X.t, steps, A, S.jbuf);
+      cgemm<T, 0, 1>(2 * ll, steps, l, one, Am, l, X.t, l, zero, X.w, steps, S.tile);
+    } else {
+      for (int e = tid(); e < m * l; e += kThreads) {
+        const int j = e / l, i = e % l;  // X.t[j][i] = conj(A[i][j]), A as l x 2r
+        X.t[e] = cconj(A[static_cast<int64_t>(i) * m + j]);
+      }
+      __syncthreads();
+      qr_r_inplace<T>(m, l, X.t, l, S.jbuf, P.svd_elems, S.red, S.dmisc + 4, X.h);
+      form_q<T>(m, steps, X.h, X.y, S.jbuf, P.svd_elems);
+      cgemm<T, 0, 1>(2 * ll, steps, l, one, Am, l, X.t, l, zero, X.w, steps, S.tile);
+      for (int e = tid(); e < steps * m; e += kThreads) {
+        const int k = e / m, j = e % m;
+        A[e] = cconj(X.y[static_cast<int64_t>(j) * steps + k]);
+      }
     }
     for (int e = tid(); e < 2 * ll * steps; e += kThreads) Am[e] = X.w[e];
     if (tid() == 0) {
@@ -1955,12 +1969,16 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
     if (tid() == 0) S.dmisc[D_FLOPS] += qr_flops(m, Dr);
     const int rn = min(m, Dr);
     cplx<T> *Rout = X.g + S.goff[k + 1 - a];
-    if (src != X.t) {
-      for (int e = tid(); e < m * Dr; e += kThreads) X.t[e] = src[e];
-      __syncthreads();
+    if (qr_small_elems(m, Dr, false) <= P.svd_elems) {
+      qr_small<T>(m, Dr, src, Dr, false, Rout, rn, nullptr, S.jbuf);
+    } else {
+      if (src != X.t) {
+        for (int e = tid(); e < m * Dr; e += kThreads) X.t[e] = src[e];
+        __syncthreads();
+      }
+      qr_r_inplace<T>(m, Dr, X.t, Dr, S.jbuf, P.svd_elems, S.red, S.dmisc + 4);
+      for (int e = tid(); e < rn * Dr; e += kThreads) Rout[e] = X.t[e];
     }
-    qr_r_inplace<T>(m, Dr, X.t, Dr, S.jbuf, P.svd_elems, S.red, S.dmisc + 4);
-    for (int e = tid(); e < rn * Dr; e += kThreads) Rout[e] = X.t[e];
     if (tid() == 0) S.rdim[k + 1 - a] = rn;
     __syncthreads();
   }
@@ -2732,12 +2750,21 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
   cplx<T> *buf = uv + kMaxVec;
   float *rv_wrk = reinterpret_cast<float *>(buf + SvdSmem<T>::elems);
   if (what == 0) {
-    qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, red, dm);
+    if (qr_small_elems(m, n, false) <= SvdSmem<T>::elems) qr_small<T>(m, n, A, n, false, A, m, nullptr, buf);
+    else qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, red, dm);
   } else if (what == 2) {
     // explicit Q of the gauge steps: reflectors kept in sig2's buffer
     cplx<T> *vstore = reinterpret_cast<cplx<T> *>(sig2);
-    qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, red, dm, vstore);
-    form_q<T>(m, min(m, n), vstore, V, buf, SvdSmem<T>::elems);
+    if (qr_small_elems(m, n, true) <= SvdSmem<T>::elems) {
+      qr_small<T>(m, n, A, n, false, A, m, V, buf);
+      const int ld = m | 1, steps = min(m, n);
+      const cplx<T> *U = buf + n * ld;
+      for (int e = tid(); e < m * steps; e += kThreads)
+        if (e / steps >= e % steps) vstore[e] = U[(e % steps) * ld + e / steps];
+    } else {
+      qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, red, dm, vstore);
+      form_q<T>(m, min(m, n), vstore, V, buf, SvdSmem<T>::elems);
+    }
   } else if (use_smem == 3) {
     svd_bond<T>(m, n, A, A, V, sig2, buf, uv, red, dm, flag, rv_wrk);
   } else {

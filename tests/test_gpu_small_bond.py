@@ -1,6 +1,9 @@
-"""The untiled contraction of small bonds at the sizes where it can go wrong:
-one column, one row, row counts around the rows in flight, the widest output.
-References are numpy in float64; bounds are rounding levels."""
+"""The routines of bonds that fit shared memory, at the sizes where they can go
+wrong: the untiled contraction (one column, one row, row counts around the
+rows in flight, the widest output) and the shared-memory QR (columns around a
+warp's four and the CTA's 64 groups, both sides of its capacity).  References
+are numpy in float64; bounds are rounding levels: 64 eps sqrt(size) of the
+matrix norm."""
 
 import numpy as np
 import pytest
@@ -44,3 +47,27 @@ def test_untiled_contraction(precision, op_a, op_b, m, n, k):
     ref = (0.5 - 0.25j) * (oa @ ob) - 2.0 * c0
     scale = np.abs(oa) @ np.abs(ob) + 2.0 * np.abs(c0)
     assert (np.abs(dc.cpu().numpy() - ref) / scale).max() < 4 * (k + 4) * EPS[precision]
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("m,n", [(1, 1), (1, 5), (5, 1), (2, 3), (3, 4), (4, 5), (16, 63), (70, 64), (70, 65), (66, 129),
+                                 (91, 85), (91, 95), (200, 110)])
+def test_shared_memory_qr(precision, m, n):
+    """R^dag R = A^dag A with R upper trapezoidal, A = Q R with orthonormal Q."""
+    rng = np.random.default_rng(31 * m + n)
+    a = cmat(rng, m, n, precision)
+    a[:, n // 2] = 0  # a zero column gets no reflector
+    k = min(m, n)
+    r = torch.tensor(a, device="cuda")
+    stn.dense_qr(precision, m, n, r.data_ptr())
+    b, q, work = torch.tensor(a, device="cuda"), torch.zeros(m, k, dtype=CDT[precision], device="cuda"), None
+    work = torch.zeros(m, k, dtype=CDT[precision], device="cuda")
+    stn.dense_qr_q(precision, m, n, b.data_ptr(), q.data_ptr(), work.data_ptr())
+    a = a.astype(np.complex128)
+    bound = 64 * EPS[precision] * np.sqrt(m * n) * np.linalg.norm(a)
+    r, b, q = (x.cpu().numpy().astype(np.complex128) for x in (r, b, q))
+    for x in (r, b):
+        assert np.all(x[k:] == 0) and np.all(np.tril(x[:k, :k], -1) == 0)
+        assert np.abs(x.conj().T @ x - a.conj().T @ a).max() <= bound * np.linalg.norm(a)
+    assert np.abs(q @ b[:k] - a).max() <= bound
+    assert np.abs(q.conj().T @ q - np.eye(k)).max() < 64 * EPS[precision] * np.sqrt(m * n)
