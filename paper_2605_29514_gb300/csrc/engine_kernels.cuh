@@ -2034,26 +2034,18 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
     const bool in_smem = r * n2 + n2 * n2 <= P.svd_elems;
     cplx<T> *Cc = in_smem ? S.jbuf : X.h;
     cplx<T> *Vc = in_smem ? S.jbuf + r * n2 : X.v;
-    // In the complex64 path a bond whose SVD fits shared memory in complex128
-    // is decomposed in double precision: FP32 Jacobi rotations leave the small
-    // singular directions with an absolute error of about sqrt(#rotations)
-    // eps sigma_1, which would be dropped or kept wrongly at every sweep.
-    bool svd64 = false, vec_from_columns = false;
-    if constexpr (sizeof(T) == 4) svd64 = 2 * (r * n2 + n2 * n2) <= P.svd_elems;
+    // In the complex64 path a bond whose SVD (with V) fits shared memory in
+    // complex128 is decomposed in double precision: FP32 Jacobi rotations leave
+    // the small singular directions with an absolute error of about
+    // sqrt(#rotations) eps sigma_1, which would be dropped or kept wrongly at
+    // every sweep.  In complex128, every bond whose matrix fits takes this path.
+    bool vec_from_columns = false;
+    const int dscale = static_cast<int>(sizeof(double) / sizeof(T));
+    const bool svd64 = n2 <= kSmallSvdCols && n2 * (r | 1) * dscale <= P.svd_elems && r * dscale <= kMaxVec &&
+                       (sizeof(T) == 8 || 2 * (r * n2 + n2 * n2) <= P.svd_elems);
     if (svd64) {
-      cplx<double> *Cd = reinterpret_cast<cplx<double> *>(S.jbuf), *Vd = Cd + r * n2;
-      double *sd = reinterpret_cast<double *>(X.te);
-      for (int e = tid(); e < r * n2; e += kThreads) {
-        int i = e / n2, j = e % n2;
-        cplx<T> v = X.y[e];
-        Cd[j * r + i] = cmake<double>(static_cast<double>(v.re), static_cast<double>(v.im));
-      }
-      __syncthreads();
-      svd_onesided<double>(r, n2, Cd, Vd, sd, &S.misc[M_JFLAG], S.red);
-      for (int e = tid(); e < n2 * n2; e += kThreads)
-        X.v[e] = cmake<T>(static_cast<T>(Vd[e].re), static_cast<T>(Vd[e].im));
-      for (int i = tid(); i < n2; i += kThreads) X.lam[i] = static_cast<T>(sd[i]);
-      __syncthreads();
+      svd_small<T>(r, n2, X.y, X.v, X.lam, P.cutoff, reinterpret_cast<cplx<double> *>(S.jbuf),
+                   reinterpret_cast<cplx<double> *>(S.uvec), S.red);
       Vc = X.v;
     } else if (sizeof(T) == 4 && P.svd64_all) {
       // Complex64 contractions with every SVD in double precision: the large
@@ -2188,7 +2180,8 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       X.vs[i * keep + c] = v;
     }
     __syncthreads();
-    reorthonormalize<T>(n2, keep, X.vs, X.e, X.y, S.tile);
+    // vectors rounded from double precision to float are orthonormal to rounding
+    if (sizeof(T) == 8 || !svd64) reorthonormalize<T>(n2, keep, X.vs, X.e, X.y, S.tile);
     // new right-canonical site k: B[c][s][r] = conj(Vs[(s*kappa + r)][c])
     cplx<T> *Bk = site_ptr<T>(P, shot, k);
     for (int e = tid(); e < keep * n2; e += kThreads) {
@@ -2709,13 +2702,21 @@ __global__ void init_kernel(EngineParams P) {
 
 // ---------------------------------------------------------------------------
 // The truncation sweep's SVD on its own: right singular vectors V (n x n,
-// column-major; columns from min(m, n) on, or beyond, are zero) and
-// squared singular values of the row-major m x n matrix A, on the copy in
-// `work` (work may be A): R factor, Jacobi on X = R^dag (n x k), V = normalised
+// column-major; columns from min(m, n) on, or beyond the rank, are zero) and
+// squared singular values of the row-major m x n matrix A.  complex128 whose
+// matrix fits shared memory: svd_small on A.  Else, on the copy in `work`
+// (work may be A): R factor, Jacobi on X = R^dag (n x k), V = normalised
 // columns of X.
 template <typename T>
 static __device__ void svd_bond(int m, int n, const cplx<T> *A, cplx<T> *work, cplx<T> *V, T *sig2, cplx<T> *buf,
                                 cplx<T> *uv, double *red, double *dm, int *flag, float *rv_wrk) {
+  if constexpr (sizeof(T) == 8) {
+    if (n <= kSmallSvdCols && n * (m | 1) <= SvdSmem<T>::elems) {
+      const int rank = svd_small<T>(m, n, A, V, sig2, 0.0, buf, uv, red);
+      for (int e = tid() + rank * n; e < n * n; e += kThreads) V[e] = cmake<T>(0, 0);
+      return;
+    }
+  }
   if (work != A)
     for (int e = tid(); e < m * n; e += kThreads) work[e] = A[e];
   __syncthreads();

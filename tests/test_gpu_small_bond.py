@@ -1,9 +1,10 @@
 """The routines of bonds that fit shared memory, at the sizes where they can go
 wrong: the untiled contraction (one column, one row, row counts around the
-rows in flight, the widest output) and the shared-memory QR (columns around a
-warp's four and the CTA's 64 groups, both sides of its capacity).  References
-are numpy in float64; bounds are rounding levels: 64 eps sqrt(size) of the
-matrix norm."""
+rows in flight, the widest output), the shared-memory QR (columns around a
+warp's four and the CTA's 64 groups, both sides of its capacity) and the
+pivoted double-precision SVD (rank-deficient, zero and badly scaled matrices,
+the column limit).  References are numpy in float64; bounds are rounding
+levels: 64 eps sqrt(size) of the matrix norm."""
 
 import numpy as np
 import pytest
@@ -71,3 +72,46 @@ def test_shared_memory_qr(precision, m, n):
         assert np.abs(x.conj().T @ x - a.conj().T @ a).max() <= bound * np.linalg.norm(a)
     assert np.abs(q @ b[:k] - a).max() <= bound
     assert np.abs(q.conj().T @ q - np.eye(k)).max() < 64 * EPS[precision] * np.sqrt(m * n)
+
+
+@pytest.mark.parametrize("m,n,rank", [(1, 1, 1), (1, 9, 1), (9, 1, 1), (4, 4, 2), (7, 5, 5), (33, 64, 20), (64, 64, 64),
+                                      (65, 64, 31), (40, 65, 40), (20, 128, 20), (20, 129, 20), (90, 90, 3)])
+@pytest.mark.parametrize("scale", [1.0, 1e-60])
+def test_pivoted_svd(m, n, rank, scale):
+    """complex128: singular values and right vectors of matrices of full and
+    deficient rank, with values over ten decades, and of a badly scaled one (not
+    beyond 128 columns: the general path's QR takes columns below 1e-30 as zero)."""
+    if n > 128 and scale != 1.0:
+        pytest.skip("the general path treats columns below 1e-30 as zero")
+    rng = np.random.default_rng(5 * m + n)
+    u, _ = np.linalg.qr(cmat(rng, m, rank, 0))
+    v, _ = np.linalg.qr(cmat(rng, n, rank, 0))
+    s = scale * 10.0 ** (-10.0 * np.arange(rank) / rank)
+    a = (u * s) @ v.conj().T
+    da = torch.tensor(a, device="cuda")
+    dv = torch.full((n, n), np.nan, dtype=torch.complex128, device="cuda")
+    ds = torch.full((n,), np.nan, dtype=torch.float64, device="cuda")
+    stn.dense_svd_noalloc(0, m, n, da.data_ptr(), dv.data_ptr(), ds.data_ptr())
+    sig = np.sqrt(ds.cpu().numpy())
+    vecs = dv.cpu().numpy()  # rows: columns of V
+    order = np.argsort(-sig)
+    bound = 64 * EPS[0] * np.sqrt(m * n)
+    assert np.abs(sig[order[:rank]] - s).max() < bound * scale
+    assert np.all(sig[order[rank:]] < bound * scale)
+    vk = vecs[order[:rank]].T
+    assert np.abs(vk.conj().T @ vk - np.eye(rank)).max() < bound
+    assert np.abs(a @ vk @ vk.conj().T - a).max() < bound * scale
+    assert np.all(np.isfinite(vecs))
+
+
+def test_pivoted_svd_zero_and_non_finite():
+    for value in (0.0, np.nan, np.inf):
+        a = torch.zeros(6, 5, dtype=torch.complex128, device="cuda")
+        a[3, 2] = value
+        dv = torch.full((5, 5), 7.0, dtype=torch.complex128, device="cuda")
+        ds = torch.full((5,), 7.0, dtype=torch.float64, device="cuda")
+        stn.dense_svd_noalloc(0, 6, 5, a.data_ptr(), dv.data_ptr(), ds.data_ptr())
+        if value == 0.0:
+            assert torch.all(ds == 0) and torch.all(dv == 0)
+        else:
+            assert not torch.any(torch.isfinite(ds))
