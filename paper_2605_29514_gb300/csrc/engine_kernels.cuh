@@ -26,6 +26,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <type_traits>
+
 #include "../../include/stn.h"
 #include "engine.h"
 
@@ -2035,7 +2037,7 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
     cplx<T> *Cc = in_smem ? S.jbuf : X.h;
     cplx<T> *Vc = in_smem ? S.jbuf + r * n2 : X.v;
     // In the complex64 path a bond whose SVD (with V) fits shared memory in
-    // complex128 is decomposed in double precision: FP32 Jacobi rotations leave
+    // 16-byte numbers is decomposed in pairs of floats: FP32 Jacobi rotations leave
     // the small singular directions with an absolute error of about
     // sqrt(#rotations) eps sigma_1, which would be dropped or kept wrongly at
     // every sweep.  In complex128, every bond whose matrix fits takes this path.
@@ -2044,8 +2046,7 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
     const bool svd64 = n2 <= kSmallSvdCols && n2 * (r | 1) * dscale <= P.svd_elems && r * dscale <= kMaxVec &&
                        (sizeof(T) == 8 || 2 * (r * n2 + n2 * n2) <= P.svd_elems);
     if (svd64) {
-      svd_small<T>(r, n2, X.y, X.v, X.lam, P.cutoff, reinterpret_cast<cplx<double> *>(S.jbuf),
-                   reinterpret_cast<cplx<double> *>(S.uvec), S.red);
+      svd_small<T>(r, n2, X.y, X.v, X.lam, P.cutoff, S.jbuf, S.uvec, S.red);
       Vc = X.v;
     } else if (sizeof(T) == 4 && P.svd64_all) {
       // Complex64 contractions with every SVD in double precision: the large
@@ -2180,7 +2181,7 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       X.vs[i * keep + c] = v;
     }
     __syncthreads();
-    // vectors rounded from double precision to float are orthonormal to rounding
+    // vectors rounded from pairs of floats to float are orthonormal to rounding
     if (sizeof(T) == 8 || !svd64) reorthonormalize<T>(n2, keep, X.vs, X.e, X.y, S.tile);
     // new right-canonical site k: B[c][s][r] = conj(Vs[(s*kappa + r)][c])
     cplx<T> *Bk = site_ptr<T>(P, shot, k);

@@ -4,13 +4,15 @@
 // Included by engine_kernels.cuh, after its complex and warp helpers.
 //
 // At these sizes (a few to about a hundred columns) nothing is bound by a
-// rate: a step is a chain of a reduction, a square root and a barrier, and on
-// the FP64 side of the number of instructions, since a warp's FP64
-// instruction takes 16 cycles of the SM's FP64 pipe (two FMAs a clock).  So a
-// column belongs to a group of 8 lanes (three shuffle levels instead of
-// five, and 8 rows per lane at 64 rows), only the warps that hold columns
-// take part in a step's barrier, and square roots start from the hardware's
-// approximation.
+// rate: a step is a chain of a reduction, a square root and a barrier.  A
+// column belongs to a group of 8 lanes (three shuffle levels instead of five),
+// only the warps that hold columns take part in a step's barrier, and square
+// roots start from the hardware's approximation.
+//
+// An FP64 instruction of a warp holds its quarter of the SM for 64 cycles
+// (measured; a dependent FP32 FMA takes 4), so the complex64 path computes what
+// has to be better than single precision in pairs of floats (ff, 48 bits): the
+// SVD it used to run in double, and the norms and scalars of its reflectors.
 
 namespace stn {
 
@@ -53,34 +55,213 @@ __device__ __forceinline__ double rsqrt64(double x) {
   return fma(r * e, fma(0.375, e, 0.5), r);
 }
 
+// ---------------------------------------------------------------------------
+// Pairs of floats, value h + l with |l| <= ulp(h) / 2: the error-free sum and
+// product of Knuth and Dekker (the product's error by FMA), about 2^-46
+// relative per operation.  The intrinsics keep a product from being contracted
+// into the sum that follows it.
+struct ff {
+  float h, l;
+};
+__device__ __forceinline__ ff ff_of(float x) { return ff{x, 0.f}; }
+__device__ __forceinline__ ff ff_neg(ff a) { return ff{-a.h, -a.l}; }
+// renormalises h + l with |l| well below |h|
+__device__ __forceinline__ ff ff_norm(ff a) {
+  const float s = __fadd_rn(a.h, a.l);
+  return ff{s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
+}
+// acc.h + x exactly into acc.h and (added to) acc.l; acc is renormalised later
+__device__ __forceinline__ void ff_push(ff &acc, float x, float low) {
+  const float s = __fadd_rn(acc.h, x), b = __fsub_rn(s, acc.h);
+  const float e = __fadd_rn(__fsub_rn(acc.h, __fsub_rn(s, b)), __fsub_rn(x, b));
+  acc.h = s;
+  acc.l = __fadd_rn(acc.l, __fadd_rn(e, low));
+}
+// acc += a b
+__device__ __forceinline__ void ff_fma(ff &acc, ff a, ff b) {
+  const float p = __fmul_rn(a.h, b.h);
+  ff_push(acc, p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p))));
+}
+// a + b, to the last bit the same as b + a: the lanes of a butterfly sum must
+// agree, since they rotate their rows by what they compute from it.
+__device__ __forceinline__ ff ff_add(ff a, ff b) {
+  ff v = ff{a.h, 0.f};
+  ff_push(v, b.h, __fadd_rn(a.l, b.l));
+  return ff_norm(v);
+}
+__device__ __forceinline__ ff ff_mul(ff a, ff b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return ff_norm(ff{p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)))});
+}
+// f (1 + d)^(-1/2) for |d| of the order of single rounding
+__device__ __forceinline__ ff ff_corrected(float f, float d) {
+  return ff_norm(ff{f, f * (d * fmaf(0.375f, d, -0.5f))});
+}
+// 1 / sqrt(x), x a normal positive number: the same third-order step as rsqrt64
+__device__ __forceinline__ ff ff_rsqrt(ff x) {
+  const float r = rsqrtf(x.h), p = __fmul_rn(r, r);
+  ff d = ff_of(-1.f);
+  ff_fma(d, x, ff{p, fmaf(r, r, -p)});
+  return ff_corrected(r, d.h + d.l);
+}
+
+template <>
+struct alignas(16) cplx<ff> {
+  ff re, im;
+};
+
+// Arithmetic of the working precision S (double or ff).
 template <typename S>
-__device__ __forceinline__ S group_sum(S v) {
+struct Work;
+template <>
+struct Work<double> {
+  static constexpr double eps = 1.11e-16;
+  static __device__ __forceinline__ double scale(double x, float) { return x; }
+  static __device__ __forceinline__ int key(double x, int c) {  // column in the low bits, order of the high words
+    const int hi = __double2hiint(x);
+    return hi < 0 ? -1 : ((hi & ~127) | c);
+  }
+  static constexpr int key_infinite = 0x7ff00000;
+  static __device__ __forceinline__ double infinite() { return __longlong_as_double(0x7ff0000000000000ll); }
+  static __device__ __forceinline__ double value(double x) { return x; }
+  static __device__ __forceinline__ bool finite(double x) { return x <= 1.7e308; }
+  static __device__ __forceinline__ double add(double a, double b) { return a + b; }
+  static __device__ __forceinline__ double norm(double a) { return a; }
+  static __device__ __forceinline__ double of(double x) { return x; }
+  static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
+  static __device__ __forceinline__ double rsqrt(double x) { return rsqrt64(x); }
+  // w += conj(a) b, b += u w, s += |x|^2
+  static __device__ __forceinline__ void dot(cplx<double> &w, cplx<double> a, cplx<double> b) { cfma(w, cconj(a), b); }
+  static __device__ __forceinline__ void axpy(cplx<double> &b, cplx<double> u, cplx<double> w) { cfma(b, u, w); }
+  static __device__ __forceinline__ void sq(double &s, cplx<double> x) { s = fma(x.re, x.re, fma(x.im, x.im, s)); }
+  static __device__ __forceinline__ double shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+};
+template <>
+struct Work<ff> {
+  static constexpr float eps = 1.42e-14f;  // 2^-46
+  static __device__ __forceinline__ ff scale(float x, float sc) { return ff_of(x * sc); }
+  static __device__ __forceinline__ int key(ff x, int c) {
+    const int b = __float_as_int(x.h);
+    return b < 0 ? -1 : ((b & ~127) | c);
+  }
+  static constexpr int key_infinite = 0x7f800000;
+  static __device__ __forceinline__ ff infinite() { return ff_of(__int_as_float(0x7f800000)); }
+  static __device__ __forceinline__ float value(ff x) { return x.h; }
+  static __device__ __forceinline__ bool finite(ff x) { return x.h <= 3e38f; }
+  static __device__ __forceinline__ ff add(ff a, ff b) { return ff_add(a, b); }
+  static __device__ __forceinline__ ff norm(ff a) { return ff_norm(a); }
+  static __device__ __forceinline__ ff of(float x) { return ff_of(x); }
+  static __device__ __forceinline__ ff mul(ff a, ff b) { return ff_mul(a, b); }
+  static __device__ __forceinline__ ff rsqrt(ff x) { return ff_rsqrt(x); }
+  static __device__ __forceinline__ void dot(cplx<ff> &w, cplx<ff> a, cplx<ff> b) {
+    ff_fma(w.re, a.re, b.re);
+    ff_fma(w.re, a.im, b.im);
+    ff_fma(w.im, a.re, b.im);
+    ff_fma(w.im, ff_neg(a.im), b.re);
+  }
+  static __device__ __forceinline__ void axpy(cplx<ff> &b, cplx<ff> u, cplx<ff> w) {
+    ff_fma(b.re, u.re, w.re);
+    ff_fma(b.re, ff_neg(u.im), w.im);
+    ff_fma(b.im, u.re, w.im);
+    ff_fma(b.im, u.im, w.re);
+    b.re = ff_norm(b.re);
+    b.im = ff_norm(b.im);
+  }
+  static __device__ __forceinline__ void sq(ff &s, cplx<ff> x) {
+    ff_fma(s, x.re, x.re);
+    ff_fma(s, x.im, x.im);
+  }
+  static __device__ __forceinline__ ff shfl(ff v, int o) {
+    return ff{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
+  }
+};
+
+// Sum over the lanes of a group (from = kGroup / 2) or a warp (from = 16).
+template <typename S>
+__device__ __forceinline__ S lane_sum(S v, int from) {
+  v = Work<S>::norm(v);
+#pragma unroll
+  for (int o = from; o > 0; o >>= 1) v = Work<S>::add(v, Work<S>::shfl(v, o));
+  return v;
+}
+__device__ __forceinline__ float group_sum(float v) {
 #pragma unroll
   for (int o = kGroup / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+__device__ __forceinline__ double group_sum(double v) { return lane_sum<double>(v, kGroup / 2); }
+__device__ __forceinline__ ff group_sum(ff v) { return lane_sum<ff>(v, kGroup / 2); }
 
-// Reflector of x = col[j..m-1] with squared norm nx2 (P = I - 2 u u^dag, P x =
-// gamma e_1, gamma = -(x_0 / |x_0|) ||x||) into u[j..m-1]; returns gamma.  One
-// warp.
-template <typename T>
-__device__ __forceinline__ cplx<T> make_reflector(const cplx<T> *col, cplx<T> *u, int j, int m, double nx2) {
-  const cplx<T> al = col[j];
-  const double are = static_cast<double>(al.re), aim = static_cast<double>(al.im);
-  const double a2 = are * are + aim * aim;
-  const double nx = nx2 * rsqrt64(nx2);
-  const bool zero = !(a2 > 1e-290);
-  const double ra = rsqrt64(zero ? 1.0 : a2);
-  const double pr = zero ? 1.0 : are * ra, pi = zero ? 0.0 : aim * ra;
-  const double aa = zero ? 0.0 : a2 * ra;
-  const cplx<T> gam = cmake<T>(static_cast<T>(-pr * nx), static_cast<T>(-pi * nx));
-  const T sc = static_cast<T>(rsqrt64(2.0 * nx * (nx + aa)));
+// Scalars of the Hermitian reflector P = I - 2 u u^dag of a column x with
+// squared norm nx2 > 0 and first element al: P x = gamma e_1, gamma = -(al /
+// |al|) ||x||, u = (x - gamma e_1) sc.  With a = al / ||x||: sc = 1 / (||x||
+// sqrt(2 (1 + |a|))); an |a| below rounding takes the phase 1.
+template <typename S>
+__device__ __forceinline__ void reflector_scalars(cplx<S> al, S nx2, cplx<S> &gam, S &sc) {
+  using K = Work<S>;
+  const S r = K::rsqrt(nx2), nx = K::mul(nx2, r);
+  const S ar = K::mul(al.re, r), ai = K::mul(al.im, r);
+  S a2 = K::of(0);
+  K::sq(a2, cmake<S>(ar, ai));
+  a2 = K::norm(a2);
+  const bool tiny = !(K::value(a2) > 1e-32f);
+  const S ra = K::rsqrt(tiny ? K::of(1) : a2);
+  const S pr = tiny ? K::of(1) : K::mul(ar, ra), pi = tiny ? K::of(0) : K::mul(ai, ra);
+  const S one_a = K::add(K::of(1), tiny ? K::of(0) : K::mul(a2, ra));
+  const S m1 = K::of(-1);
+  gam = cmake<S>(K::mul(m1, K::mul(pr, nx)), K::mul(m1, K::mul(pi, nx)));
+  sc = K::mul(r, K::rsqrt(K::add(one_a, one_a)));
+}
+
+// Reflector j of the column col[j..m-1] in the storage precision T into
+// u[j..m-1]; col[j] becomes gamma.  A column of norm up to 1e-30 gets none
+// (u = 0).  Norm and scalars in double, or for float in ff on the column scaled
+// by a power of two: single-precision squares of entries near 1e-20 would be
+// denormal, and a reflector built from such a norm not unitary.  One warp.
+__device__ __forceinline__ void reflect_column(cplx<double> *col, cplx<double> *u, int j, int m) {
+  double s = 0;
+  for (int i = j + lane_id(); i < m; i += 32) Work<double>::sq(s, col[i]);
+  s = lane_sum<double>(s, 16);
+  cplx<double> gam = cmake<double>(0, 0);
+  double sc = 0;
+  if (s > 1e-60) reflector_scalars<double>(col[j], s, gam, sc);
   for (int i = j + lane_id(); i < m; i += 32) {
-    cplx<T> x = col[i];
-    if (i == j) x = cmake<T>(x.re - gam.re, x.im - gam.im);
-    u[i] = cscale(x, sc);
+    cplx<double> x = col[i];
+    if (i == j) x = cmake<double>(x.re - gam.re, x.im - gam.im);
+    u[i] = sc > 0 ? cscale(x, sc) : cmake<double>(0, 0);
   }
-  return gam;
+  __syncwarp();
+  if (lane_id() == 0) col[j] = gam;
+}
+__device__ __forceinline__ void reflect_column(cplx<float> *col, cplx<float> *u, int j, int m) {
+  float mx = 0.f;
+  for (int i = j + lane_id(); i < m; i += 32) mx = fmaxf(mx, fmaxf(fabsf(col[i].re), fabsf(col[i].im)));
+  const int bits = __reduce_max_sync(0xffffffffu, __float_as_int(mx));
+  const int ex = min(253, max(1, bits >> 23));
+  const float down = __int_as_float((254 - ex) << 23), up = __int_as_float(ex << 23);  // 2^-(ex - 127) and its inverse
+  ff s = ff_of(0.f);
+  for (int i = j + lane_id(); i < m; i += 32) {
+    const float re = col[i].re * down, im = col[i].im * down;
+    ff_fma(s, ff_of(re), ff_of(re));
+    ff_fma(s, ff_of(im), ff_of(im));
+  }
+  s = lane_sum<ff>(s, 16);
+  cplx<float> gam = cmake<float>(0.f, 0.f);
+  float sc = 0.f;
+  if (sqrtf(s.h) * up > 1e-30f) {
+    cplx<ff> g;
+    ff c;
+    reflector_scalars<ff>(cmake<ff>(ff_of(col[j].re * down), ff_of(col[j].im * down)), s, g, c);
+    gam = cmake<float>(g.re.h, g.im.h);
+    sc = c.h;
+  }
+  for (int i = j + lane_id(); i < m; i += 32) {
+    cplx<float> x = cmake<float>(col[i].re * down, col[i].im * down);
+    if (i == j) x = cmake<float>(x.re - gam.re, x.im - gam.im);
+    u[i] = sc > 0.f ? cscale(x, sc) : cmake<float>(0.f, 0.f);
+  }
+  __syncwarp();
+  if (lane_id() == 0) col[j] = cmake<float>(gam.re * up, gam.im * up);
 }
 
 // Householder QR in shared memory.  A is m x n: row-major with leading
@@ -119,18 +300,7 @@ static __device__ __noinline__ void qr_small(int m, int n, const cplx<T> *A, int
   __syncthreads();
   const int nthr = team_threads(n);
   const int gl = lane_id() & (kGroup - 1), g = tid() / kGroup;
-  auto reflect = [&](int j) {
-    cplx<T> *col = Bm + j * ld, *u = U + (keep ? j : (j & 1)) * ld;
-    double s = 0;
-    for (int i = j + lane_id(); i < m; i += 32) s += cabs2d(col[i]);
-    s = warp_sum(s);
-    cplx<T> gam = cmake<T>(0, 0);
-    if (s > 1e-60) gam = make_reflector<T>(col, u, j, m, s);
-    else  // (numerically) zero column: no reflector
-      for (int i = j + lane_id(); i < m; i += 32) u[i] = cmake<T>(0, 0);
-    __syncwarp();
-    if (lane_id() == 0) col[j] = gam;
-  };
+  auto reflect = [&](int j) { reflect_column(Bm + j * ld, U + (keep ? j : (j & 1)) * ld, j, m); };
   if (tid() < nthr) {
     if (warp_id() == 0) reflect(0);
     team_sync(nthr);
@@ -216,114 +386,237 @@ static __device__ __noinline__ void qr_small(int m, int n, const cplx<T> *A, int
   __syncthreads();
 }
 
-// SVD of a bond in double precision, in shared memory: Householder QR with
-// column pivoting, then one-sided (Hestenes) Jacobi on the rows of R, the
-// preconditioning of Drmac and Veselic (SIAM J. Matrix Anal. Appl. 29, 2008).
-// A (m x n, row-major, leading dimension n) = Q R, R in the original column
-// order; rotating the rows of R until they are orthogonal gives the rows
-// sigma_i v_i^dag, so no rotation is accumulated.  lam[i] = sigma_i^2 (unsorted,
-// zero beyond the numerical rank, which is returned) and column i of V (n x n,
-// column-major; columns beyond the rank are not written, except column 0 of a
-// zero matrix) = v_i.  Values that are not finite give lam = NaN.
+// The rotation of a pair of rows with squared norms al, be and inner product
+// g: x <- cs x - sn uc y, y <- sn x + cs uc y makes them orthogonal.  Its angle
+// is found in single precision from numbers scaled by a power of two; cosine,
+// sine and the phase uc = conj(g / |g|) are then brought to the working
+// precision by a third-order correction, so the rotation is unitary to rounding
+// and only its angle is approximate (which costs no sweep: an angle good to
+// 1e-7 leaves 1e-7 of the product).  tg: what |x|^2 loses and |y|^2 gains.
+template <typename S>
+struct Rotation {
+  S cs, sn, tg;
+  cplx<S> uc;
+};
+
+__device__ __forceinline__ void rotation_angle(float diff, float gr, float gi, float &t, float &ur, float &ui,
+                                               float &absg) {
+  const float mx = fmaxf(fmaxf(fabsf(gr), fabsf(gi)), 1e-37f), imx = 1.f / mx;
+  const float a = gr * imx, b = gi * imx, n2 = a * a + b * b, rn = rsqrtf(n2);
+  absg = mx * (n2 * rn);
+  const float zeta = diff / (2.f * absg), az = fabsf(zeta);
+  t = az > 1e10f ? 0.5f / az : 1.f / (az + sqrtf(1.f + az * az));
+  if (zeta < 0.f) t = -t;
+  ur = a * rn;
+  ui = -b * rn;
+}
+
+__device__ __forceinline__ bool make_rotation(double al, double be, cplx<double> g, double tol2, Rotation<double> &r) {
+  if (!(cabs2(g) > tol2 * al * be)) return false;
+  const int ex = min(2045, max(1, __double2hiint(fmax(al, be)) >> 20));  // the larger norm is scaled to [1, 2)
+  const double sc = __hiloint2double((2046 - ex) << 20, 0);
+  float tf, urf, uif, absg;
+  rotation_angle(static_cast<float>((be - al) * sc), static_cast<float>(g.re * sc), static_cast<float>(g.im * sc), tf,
+                 urf, uif, absg);
+  const double t = static_cast<double>(tf), w = fma(t, t, 1.0);
+  const double c0 = static_cast<double>(rsqrtf(fmaf(tf, tf, 1.f)));
+  double d = fma(-w * c0, c0, 1.0);
+  r.cs = fma(c0 * d, fma(0.375, d, 0.5), c0);
+  r.sn = t * r.cs;
+  const double ur = static_cast<double>(urf), ui = static_cast<double>(uif);
+  d = fma(-ur, ur, fma(-ui, ui, 1.0));
+  d = fma(d, fma(0.375, d, 0.5), 1.0);
+  r.uc = cmake<double>(ur * d, ui * d);
+  r.tg = static_cast<double>(tf * absg) * __hiloint2double(ex << 20, 0);
+  return true;
+}
+__device__ __forceinline__ bool make_rotation(ff al, ff be, cplx<ff> g, float tol, Rotation<ff> &r) {
+  const float gr = g.re.h, gi = g.im.h;
+  const float lim = tol * sqrtf(al.h) * sqrtf(be.h);
+  if (!(fmaxf(fabsf(gr), fabsf(gi)) > 0.70711f * lim)) return false;  // max(|re|, |im|) >= |g| / sqrt(2)
+  float tf, ur, ui, absg;
+  rotation_angle(ff_add(be, ff_neg(al)).h, gr, gi, tf, ur, ui, absg);
+  if (!(absg > lim)) return false;
+  const ff t = ff_of(tf);
+  ff w = ff_of(1.f);
+  ff_fma(w, t, t);
+  r.cs = ff_rsqrt(ff_norm(w));
+  r.sn = ff_mul(t, r.cs);
+  ff d = ff_of(-1.f);
+  ff_fma(d, ff_of(ur), ff_of(ur));
+  ff_fma(d, ff_of(ui), ff_of(ui));
+  r.uc = cmake<ff>(ff_corrected(ur, d.h + d.l), ff_corrected(ui, d.h + d.l));
+  r.tg = ff_of(tf * absg);
+  return true;
+}
+
+__device__ __forceinline__ void rotate_pair(cplx<double> &x, cplx<double> &y, const Rotation<double> &r) {
+  const cplx<double> a = x, b = cmul(r.uc, y);
+  x = cmake<double>(fma(r.cs, a.re, -r.sn * b.re), fma(r.cs, a.im, -r.sn * b.im));
+  y = cmake<double>(fma(r.sn, a.re, r.cs * b.re), fma(r.sn, a.im, r.cs * b.im));
+}
+// a b + c d
+__device__ __forceinline__ ff ff_two(ff a, ff b, ff c, ff d) {
+  const float p = __fmul_rn(a.h, b.h);
+  ff v = ff{p, fmaf(a.l, b.h, fmaf(a.h, b.l, fmaf(a.h, b.h, -p)))};
+  ff_fma(v, c, d);
+  return ff_norm(v);
+}
+__device__ __forceinline__ void rotate_pair(cplx<ff> &x, cplx<ff> &y, const Rotation<ff> &r) {
+  const cplx<ff> a = x;
+  const cplx<ff> b = cmake<ff>(ff_two(r.uc.re, y.re, ff_neg(r.uc.im), y.im), ff_two(r.uc.re, y.im, r.uc.im, y.re));
+  const ff ns = ff_neg(r.sn);
+  x = cmake<ff>(ff_two(r.cs, a.re, ns, b.re), ff_two(r.cs, a.im, ns, b.im));
+  y = cmake<ff>(ff_two(r.sn, a.re, r.cs, b.re), ff_two(r.sn, a.im, r.cs, b.im));
+}
+
+// SVD of a bond in shared memory, in double precision (T = double) or in
+// pairs of floats (T = float): Householder QR with column pivoting, then
+// one-sided (Hestenes) Jacobi on the rows of R, the preconditioning of Drmac
+// and Veselic (SIAM J. Matrix Anal. Appl. 29, 2008).  A (m x n, row-major,
+// leading dimension n) = Q R, R in the original column order; rotating the rows
+// of R until they are orthogonal gives the rows sigma_i v_i^dag, so no rotation
+// is accumulated.  lam[i] = sigma_i^2 (unsorted, zero beyond the numerical rank,
+// which is returned; but see cutoff) and column i of V (n x n, column-major; columns beyond the
+// rank are not written, except column 0 of a zero matrix) = v_i.  Values that
+// are not finite give lam = NaN.
 //
-// Against Jacobi on A's columns with accumulated V (what bonds that fit
-// shared memory ran before) this takes about half the sweeps and a quarter of
-// the rotations on the matrices of a d = 3 and a d = 5 run, and rotates one
-// matrix instead of two.  A group of 8 lanes rotates a pair; the angle is
-// found in single precision from exponent-scaled numbers, and the cosine,
-// sine and phase are brought to double precision by a third-order correction,
-// so the rotation is unitary to rounding and only its angle is approximate
-// (which costs no sweep: an angle good to 1e-7 leaves 1e-7 of the product).
+// Against Jacobi on A's columns with accumulated V this takes about half the
+// sweeps and a quarter of the rotations on the matrices of a d = 3 and a d = 5
+// run, and rotates one matrix instead of two.
 //
-// cutoff > 0 (the truncation's): two rows whose norms are both so small that
-// all such rows together stay below half of cutoff sigma_1 are not rotated
-// against each other.  They are dropped whatever their mutual angles are, and
-// the sum of their squares, the discarded weight, does not change.
+// Pairs of floats against double, on the complex64 path whose input and output
+// are single precision: 32 x 32 bonds of a d = 5 round take 259 us against 960
+// us, 52 x 52 ones of an X-memory 0.84 ms against 3.1 ms, with the same errors
+// of the singular values, vectors and truncated matrix.
 //
-// buf: n (m | 1) complex doubles; u: m of them; nr: n doubles (all shared
-// memory); n <= kSmallSvdCols.  CTA-wide.
+// cutoff > 0 (the truncation's): the QR stops once the norm of all that is left
+// is at most d sigma_1, d = min(cutoff / 16, sqrt(eps_T cutoff)) with eps_T the
+// rounding of T; lam[rank] is then what is left (its squared norm, for the
+// discarded weight).  A value below cutoff sigma_1 is dropped by the caller, and
+// leaving such a remainder out turns a kept vector of value s by at most (d
+// sigma_1 / s)^2, that is the decomposed matrix by d^2 sigma_1 / cutoff <= eps_T
+// sigma_1.  In complex64 the remainder is the rounding noise of A, about a third
+// of the rows of a bond, and the most expensive ones.  (Keeping them but not
+// rotating them against each other was slower: it leaves the sweeps converging
+// linearly.)
+//
+// buf: n (m | 1) 16-byte complex numbers; u: m of them; nr: n doubles (all
+// shared memory); n <= kSmallSvdCols.  CTA-wide.
 template <typename T>
-static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cplx<T> *V, T *lam, double cutoff,
-                                             cplx<double> *buf_, cplx<double> *u_, double *nr_) {
+static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cplx<T> *V, T *lam, double cutoff_,
+                                             void *buf_, void *u_, void *nr_) {
+  using S = std::conditional_t<sizeof(T) == 8, double, ff>;
+  using K = Work<S>;
+  using R = decltype(K::value(S()));  // double or float
   const int ld = m | 1, steps = min(m, n);
-  cplx<double> *Bm = in_smem<cplx<double>>(buf_), *u = in_smem<cplx<double>>(u_);
-  double *nr = in_smem<double>(nr_);
+  cplx<S> *Bm = in_smem<cplx<S>>(buf_), *u = in_smem<cplx<S>>(u_);
+  S *nr = in_smem<S>(nr_);
+  const int gl = lane_id() & (kGroup - 1), g = tid() / kGroup;
+  float down = 1.f, up = 1.f;  // ff: the matrix scaled by a power of two to entries up to 1
+  if constexpr (sizeof(T) == 4) {
+    int *top = reinterpret_cast<int *>(u);
+    if (tid() == 0) *top = 0;
+    __syncthreads();
+    int bits = 0;
+    for (int e = tid(); e < m * n; e += kThreads)
+      bits = max(bits, max(__float_as_int(fabsf(A[e].re)), __float_as_int(fabsf(A[e].im))));
+    bits = __reduce_max_sync(0xffffffffu, bits);
+    if (lane_id() == 0) atomicMax(top, bits);
+    __syncthreads();
+    const int ex = min(253, max(1, *top >> 23));
+    down = __int_as_float((254 - ex) << 23);
+    up = __int_as_float(ex << 23);
+    __syncthreads();
+  }
   for (int e = tid(); e < m * n; e += kThreads) {
     const int i = e / n, c = e % n;
     const cplx<T> x = A[e];
-    Bm[c * ld + i] = cmake<double>(static_cast<double>(x.re), static_cast<double>(x.im));
+    Bm[c * ld + i] = cmake<S>(K::scale(x.re, down), K::scale(x.im, down));
   }
   __syncthreads();
-  const int gl = lane_id() & (kGroup - 1), g = tid() / kGroup;
-  constexpr double eps2 = 1.11e-16 * 1.11e-16;
-  // largest of k numbers >= 0 (or -1) by their high words, column in the low
-  // bits; every warp finds it by itself
+  // largest of k numbers >= 0 (or -1), column in the low bits; every warp finds
+  // it by itself
   auto top_key = [&](int k) {
     int key = -1;
-    for (int c = lane_id(); c < k; c += 32) {
-      const int hi = __double2hiint(nr[c]);
-      key = max(key, hi < 0 ? -1 : ((hi & ~127) | c));
-    }
+    for (int c = lane_id(); c < k; c += 32) key = max(key, K::key(nr[c], c));
     return __reduce_max_sync(0xffffffffu, key);
   };
+  const R cutoff = static_cast<R>(cutoff_), eps_t = sizeof(T) == 8 ? R(1.11e-16) : R(5.96e-8);
   int rank = 0;
-  double neg = 0.0;  // squared norm of a negligible row
+  R neg = 0;    // squared norm of a negligible row
+  R rest = 0;   // squared norm of the remainder that may be left out
+  R left = 0;   // bound on the squared norm of the remainder that was
   bool finite = true;
   {
     const int nthr = team_threads(n);
     if (tid() < nthr) {
       for (int c = g; (c & ~3) < n; c += kGroups) {
-        double s = 0;
+        S s = K::of(0);
         if (c < n)
-          for (int i = gl; i < m; i += kGroup) s += cabs2(Bm[c * ld + i]);
+          for (int i = gl; i < m; i += kGroup) K::sq(s, Bm[c * ld + i]);
         s = group_sum(s);
-        if (gl == 0 && c < n) nr[c] = s <= 1.7e308 ? s : __longlong_as_double(0x7ff0000000000000ll);
+        if (gl == 0 && c < n) nr[c] = K::finite(s) ? s : K::infinite();
       }
     }
     __syncthreads();
     const int k0 = top_key(n);
-    finite = k0 < 0x7ff00000;
-    neg = eps2 * nr[k0 & 127];
+    finite = k0 < K::key_infinite;
+    neg = K::eps * K::eps * K::value(nr[k0 & 127]);
+    rest = min(cutoff * cutoff / 256, eps_t * cutoff) * K::value(nr[k0 & 127]);
     __syncthreads();
     if (tid() < nthr && finite) {
       for (int j = 0; j < steps; ++j) {
         const int key = top_key(n);
         const int p = key & 127;
-        const double nx2 = key < 0 ? 0.0 : nr[p];
-        if (!(nx2 > neg)) break;  // the rest is below rounding (also: a zero matrix)
+        const S nx2 = key < 0 ? K::of(0) : nr[p];
+        left = K::value(nx2) * (n - j);
+        if (!(K::value(nx2) > neg) || left <= rest) break;  // what is left is dropped or below rounding
+        left = 0;
         if (warp_id() == (p & (kGroups - 1)) / 4) {
-          cplx<double> *col = Bm + p * ld;
-          const cplx<double> gam = make_reflector<double>(col, u, j, m, nx2);
+          cplx<S> *col = Bm + p * ld;
+          cplx<S> gam;
+          S sc;
+          reflector_scalars<S>(col[j], nx2, gam, sc);
+          for (int i = j + lane_id(); i < m; i += 32) {
+            cplx<S> x = col[i];
+            if (i == j) {
+              x.re = K::add(x.re, K::mul(K::of(-1), gam.re));
+              x.im = K::add(x.im, K::mul(K::of(-1), gam.im));
+            }
+            u[i] = cmake<S>(K::mul(x.re, sc), K::mul(x.im, sc));
+          }
           __syncwarp();
-          for (int i = j + lane_id(); i < m; i += 32) col[i] = i == j ? gam : cmake<double>(0, 0);
+          for (int i = j + lane_id(); i < m; i += 32) col[i] = i == j ? gam : cmake<S>(K::of(0), K::of(0));
         }
         team_sync(nthr);
         const int i0 = j + ((gl - j) & (kGroup - 1));
         for (int c = g; (c & ~3) < n; c += kGroups) {
-          const bool on = c < n && c != p && nr[min(c, n - 1)] >= 0.0;
-          cplx<double> *b = Bm + min(c, n - 1) * ld;
-          cplx<double> w = cmake<double>(0, 0);
-          if (on)
+          const bool on = c < n && c != p && K::value(nr[min(c, n - 1)]) >= 0;
+          if (__any_sync(0xffffffffu, on)) {
+            cplx<S> *b = Bm + min(c, n - 1) * ld;
+            cplx<S> w = cmake<S>(K::of(0), K::of(0));
+            if (on)
 #pragma unroll 4
-            for (int i = i0; i < m; i += kGroup) cfma(w, cconj(u[i]), b[i]);
-          w.re = group_sum(w.re);
-          w.im = group_sum(w.im);
-          double s = 0;
-          if (on) {
-            w = cmake<double>(-2.0 * w.re, -2.0 * w.im);
+              for (int i = i0; i < m; i += kGroup) K::dot(w, u[i], b[i]);
+            w.re = group_sum(w.re);
+            w.im = group_sum(w.im);
+            S s = K::of(0);
+            if (on) {
+              w = cmake<S>(K::mul(K::of(-2), w.re), K::mul(K::of(-2), w.im));
 #pragma unroll 4
-            for (int i = i0; i < m; i += kGroup) {
-              cplx<double> x = b[i];
-              cfma(x, u[i], w);
-              b[i] = x;
-              if (i > j) s = fma(x.re, x.re, fma(x.im, x.im, s));
+              for (int i = i0; i < m; i += kGroup) {
+                cplx<S> x = b[i];
+                K::axpy(x, u[i], w);
+                b[i] = x;
+                if (i > j) K::sq(s, x);
+              }
             }
+            s = group_sum(s);
+            if (gl == 0 && on) nr[c] = s;
           }
-          s = group_sum(s);
-          if (gl == 0 && c < n) {
-            if (on) nr[c] = s;
-            else if (c == p) nr[c] = -1.0;
-          }
+          __syncwarp();
+          if (gl == 0 && c == p) nr[c] = K::of(-1);
         }
         team_sync(nthr);
         rank = j + 1;
@@ -331,20 +624,25 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
     }
   }
   // the rank is known to the team's threads
-  if (tid() == 0) reinterpret_cast<int *>(u)[0] = rank;
+  if (tid() == 0) {
+    reinterpret_cast<int *>(u)[0] = rank;
+    reinterpret_cast<R *>(u)[2] = left;
+  }
   __syncthreads();
   rank = reinterpret_cast<int *>(u)[0];
+  left = reinterpret_cast<R *>(u)[2];
   __syncthreads();
 
   // rows of R: row i at Bm[c ld + i], ld odd, so 8 lanes over c meet no bank twice
   const int kk = rank + (rank & 1), half = kk / 2;
   const int nthr = team_threads(max(1, half));
-  const double tol = 4.0 * 1.11e-16 * sqrt(static_cast<double>(n)), tol2 = tol * tol;
+  const R tol = R(4) * K::eps * sqrt(static_cast<R>(n));
+  const R limit = sizeof(T) == 8 ? tol * tol : tol;  // make_rotation takes tol^2 in double
   auto norms = [&]() {
     for (int i = g; (i & ~3) < kk; i += nthr / kGroup) {
-      double s = 0;
+      S s = K::of(0);
       if (i < rank)
-        for (int c = gl; c < n; c += kGroup) s += cabs2(Bm[c * ld + i]);
+        for (int c = gl; c < n; c += kGroup) K::sq(s, Bm[c * ld + i]);
       s = group_sum(s);
       if (gl == 0 && i < rank) nr[i] = s;
     }
@@ -352,8 +650,6 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   if (tid() < nthr && finite) {
     for (int sweep = 0; sweep < kMaxSweepsD && rank > 1; ++sweep) {
       norms();
-      team_sync(nthr);
-      const double noise = cutoff * cutoff * nr[top_key(rank) & 127] / (4.0 * rank);
       team_sync(nthr);
       bool rotated = false;
       for (int round = 0; round < kk - 1; ++round) {
@@ -364,48 +660,30 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
           if (p > q) { const int t = p; p = q; q = t; }
           bool on = pi < half && q < rank;
           if (!on) p = q = 0;
-          const double al = nr[p], be = nr[q];
-          on = on && al > neg && be > neg && (al > noise || be > noise);
-          cplx<double> dot = cmake<double>(0, 0);
+          const S al = nr[p], be = nr[q];
+          const R av = K::value(al), bv = K::value(be);
+          on = on && av > neg && bv > neg;
+          if (!__any_sync(0xffffffffu, on)) continue;
+          cplx<S> dot = cmake<S>(K::of(0), K::of(0));
           if (on)
 #pragma unroll 4
-            for (int c = gl; c < n; c += kGroup) cfma(dot, cconj(Bm[c * ld + p]), Bm[c * ld + q]);
-          if (!__any_sync(0xffffffffu, on)) continue;
+            for (int c = gl; c < n; c += kGroup) K::dot(dot, Bm[c * ld + p], Bm[c * ld + q]);
           dot.re = group_sum(dot.re);
           dot.im = group_sum(dot.im);
-          if (!(cabs2(dot) > tol2 * al * be)) on = false;
-          if (on) {
+          Rotation<S> rot;
+          if (on && make_rotation(al, be, dot, limit, rot)) {
             rotated = true;
-            // numbers scaled by a power of two so that the larger norm is in [1, 2)
-            const int ex = max(1, __double2hiint(fmax(al, be)) >> 20);
-            const double sc = __hiloint2double((2046 - min(2045, ex)) << 20, 0);
-            const float df = static_cast<float>((be - al) * sc);
-            const float gr = static_cast<float>(dot.re * sc), gi = static_cast<float>(dot.im * sc);
-            const float mx = fmaxf(fmaxf(fabsf(gr), fabsf(gi)), 1e-37f), imx = 1.f / mx;
-            const float ga = gr * imx, gb = gi * imx, g2 = ga * ga + gb * gb, gl2 = rsqrtf(g2);
-            const float absg = mx * (g2 * gl2);
-            const float zeta = df / (2.f * absg), az = fabsf(zeta);
-            float tf = az > 1e10f ? 0.5f / az : 1.f / (az + sqrtf(1.f + az * az));
-            if (zeta < 0.f) tf = -tf;
-            const double t = static_cast<double>(tf), w = fma(t, t, 1.0);
-            double cs = static_cast<double>(rsqrtf(fmaf(tf, tf, 1.f)));
-            double d = fma(-w * cs, cs, 1.0);
-            cs = fma(cs * d, fma(0.375, d, 0.5), cs);
-            const double sn = t * cs;
-            double ur = static_cast<double>(ga * gl2), ui = -static_cast<double>(gb * gl2);
-            d = fma(-ur, ur, fma(-ui, ui, 1.0));
-            d = fma(d, fma(0.375, d, 0.5), 1.0);
-            const cplx<double> uc = cmake<double>(ur * d, ui * d);  // conj(g / |g|)
 #pragma unroll 2
             for (int c = gl; c < n; c += kGroup) {
-              const cplx<double> x = Bm[c * ld + p], y = cmul(uc, Bm[c * ld + q]);
-              Bm[c * ld + p] = cmake<double>(fma(cs, x.re, -sn * y.re), fma(cs, x.im, -sn * y.im));
-              Bm[c * ld + q] = cmake<double>(fma(sn, x.re, cs * y.re), fma(sn, x.im, cs * y.im));
+              cplx<S> x = Bm[c * ld + p], y = Bm[c * ld + q];
+              rotate_pair(x, y, rot);
+              Bm[c * ld + p] = x;
+              Bm[c * ld + q] = y;
             }
             if (gl == 0) {
-              const double tg = t * static_cast<double>(absg) * __hiloint2double(min(2045, ex) << 20, 0);
-              nr[p] = fmax(al - tg, 0.0);
-              nr[q] = fmax(be + tg, 0.0);
+              const S a1 = K::add(al, K::mul(K::of(-1), rot.tg)), b1 = K::add(be, rot.tg);
+              nr[p] = K::value(a1) > 0 ? a1 : K::of(0);
+              nr[q] = K::value(b1) > 0 ? b1 : K::of(0);
             }
           }
         }
@@ -418,15 +696,17 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   __syncthreads();
   for (int e = tid(); e < n * rank; e += kThreads) {
     const int i = e / n, c = e % n;
-    const double s = nr[i];
-    const cplx<double> x = Bm[c * ld + i];
-    const double inv = s > 0.0 ? rsqrt64(s) : 0.0;
-    V[e] = cmake<T>(static_cast<T>(x.re * inv), static_cast<T>(-x.im * inv));
+    const S s = nr[i];
+    const cplx<S> x = Bm[c * ld + i];
+    const S inv = K::value(s) > 0 ? K::rsqrt(s) : K::of(0);
+    V[e] = cmake<T>(static_cast<T>(K::value(K::mul(x.re, inv))), static_cast<T>(-K::value(K::mul(x.im, inv))));
   }
   if (rank == 0)
     for (int c = tid(); c < n; c += kThreads) V[c] = cmake<T>(c == 0 ? T(1) : T(0), 0);
   for (int i = tid(); i < n; i += kThreads)
-    lam[i] = !finite ? static_cast<T>(__longlong_as_double(0x7ff8000000000000ll)) : i < rank ? static_cast<T>(nr[i]) : T(0);
+    lam[i] = !finite ? static_cast<T>(__longlong_as_double(0x7ff8000000000000ll))
+                     : i < rank ? static_cast<T>(K::value(nr[i])) * up * up
+                     : i == rank && cutoff > 0 ? static_cast<T>(left) * up * up : T(0);
   __syncthreads();
   return rank;
 }
