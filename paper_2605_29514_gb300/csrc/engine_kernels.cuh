@@ -1728,10 +1728,11 @@ __device__ __forceinline__ cplx<T> *site_ptr(const EngineParams &P, int64_t shot
 
 // out = branch-summed MPO tensor of site k (see header comment): left bond
 // doubled when dl, right bond doubled when dr; the (alpha, l) index is
-// alpha * chl + l.
+// alpha * chl + l.  Elements first, first + stride, ... by the calling thread.
 template <typename T>
 static __device__ __noinline__ void materialize(const MpoSpec<T> &sp, const uint64_t *ppx, const uint64_t *ppz, int k,
-                            const cplx<T> *A, int chl, int chr, bool dl, bool dr, cplx<T> *out) {
+                            const cplx<T> *A, int chl, int chr, bool dl, bool dr, cplx<T> *out,
+                            int first, int stride) {
   if (sp.kind == MPO_PROJ_Z) {
     // (I + s Z_S)/2 written without its two cancelling branches: the bond
     // index carries the parity of the S bits to the left, a site in S adds
@@ -1741,7 +1742,7 @@ static __device__ __noinline__ void materialize(const MpoSpec<T> &sp, const uint
     const bool in_s = (ppz[k >> 6] >> (k & 63)) & 1;
     const int Dl = dl ? 2 * chl : chl, Dr = dr ? 2 * chr : chr;
     const int total = Dl * 2 * Dr;
-    for (int e = tid(); e < total; e += kThreads) {
+    for (int e = first; e < total; e += stride) {
       const int R = e % Dr;
       const int sb = (e / Dr) & 1;
       const int L = e / (2 * Dr);
@@ -1757,7 +1758,7 @@ static __device__ __noinline__ void materialize(const MpoSpec<T> &sp, const uint
   site_op(sp, ppx, ppz, k, 1, op1);
   const int Dl = dl ? 2 * chl : chl, Dr = dr ? 2 * chr : chr;
   const int total = Dl * 2 * Dr;
-  for (int e = tid(); e < total; e += kThreads) {
+  for (int e = first; e < total; e += stride) {
     int R = e % Dr;
     int s = (e / Dr) & 1;
     int L = e / (2 * Dr);
@@ -1781,27 +1782,54 @@ static __device__ __noinline__ void materialize(const MpoSpec<T> &sp, const uint
   }
 }
 
-// Keep count at one bond from eigenvalues sorted in decreasing order, by one
-// warp (a lane's square roots are independent; one thread would do them in a
-// chain).
+// Keep count at one bond from its eigenvalues lam (>= 0) in the decreasing order
+// perm, by one warp.  The cutoff is compared in squares, lam_i > cutoff^2 lam_1:
+// square roots (of double, by one thread) were most of the 11,000 cycles the
+// keep decision of a bond took.
 template <typename T>
-static __device__ int keep_count(const T *lam_sorted, int n, int cap, double cutoff, double delta) {
-  auto sigma = [&](int i) { return sqrt(fmax(static_cast<double>(lam_sorted[i]), 0.0)); };
-  auto above = [&](int m, double thr) {
+static __device__ int keep_count(const T *lam, const int *perm, int n, int cap, double cutoff, double delta) {
+  auto at = [&](int i) { return static_cast<double>(lam[perm[i]]); };
+  auto above = [&](int m, double thr2) {
     int k = 0;
     for (int i = 0; i < m; i += 32)
-      k += __popc(__ballot_sync(0xffffffffu, i + lane_id() < m && sigma(min(i + lane_id(), m - 1)) > thr));
+      k += __popc(__ballot_sync(0xffffffffu, i + lane_id() < m && at(min(i + lane_id(), m - 1)) > thr2));
     return k;
   };
-  const double s1 = sigma(0);
-  if (!(s1 > 0.0)) return 1;
-  int k = above(n, cutoff * s1);
-  if (k < 1) k = 1;
+  const double l1 = at(0);
+  if (!(l1 > 0.0)) return 1;
+  int k = max(1, above(n, cutoff * cutoff * l1));
   if (k > cap) {
-    k = above(cap, sigma(cap) + delta * s1);
-    if (k < 1) k = 1;
+    const double thr = sqrt(at(cap)) + delta * sqrt(l1);
+    k = max(1, above(cap, thr * thr));
   }
   return k;
+}
+
+// Discarded over total weight of a bond, by one warp (lane 0's value counts).
+static __device__ __forceinline__ double discarded_weight(const double *lam, const int *perm, int n, int keep) {
+  double tot = 0, drop = 0;
+  for (int i = lane_id(); i < n; i += 32) {
+    const double l = lam[perm[i]];
+    tot += l;
+    if (i >= keep) drop += l;
+  }
+  tot = warp_sum(tot);
+  drop = warp_sum(drop);
+  return tot > 0 ? drop / tot : 0.0;
+}
+static __device__ __forceinline__ double discarded_weight(const float *lam, const int *perm, int n, int keep) {
+  ff tot = ff_of(0.f), drop = ff_of(0.f);
+  for (int i = lane_id(); i < n; i += 32) {
+    const float l = lam[perm[i]];
+    ff_push(tot, l, 0.f);
+    if (i >= keep) ff_push(drop, l, 0.f);
+  }
+  tot = lane_sum<ff>(tot, 16);
+  drop = lane_sum<ff>(drop, 16);
+  if (!(tot.h > 0.f)) return 0.0;
+  const float q = drop.h / tot.h;
+  ff_fma(drop, ff_of(-q), tot);  // the remainder: a second quotient digit of single precision
+  return static_cast<double>(q) + static_cast<double>((drop.h + drop.l) / tot.h);
 }
 
 // Exact gauge steps (no truncation) moving the orthogonality centre of a
@@ -1905,7 +1933,7 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
   int *chi = S.chi;
   if (a == b) {
     cplx<T> *A = site_ptr<T>(P, shot, a);
-    materialize(sp, S.ppx, S.ppz, a, A, chi[a], chi[a + 1], false, false, X.t);
+    materialize(sp, S.ppx, S.ppz, a, A, chi[a], chi[a + 1], false, false, X.t, tid(), kThreads);
     __syncthreads();
     if (!want_norm) return 0.0;
     const int64_t tot = static_cast<int64_t>(chi[a]) * 2 * chi[a + 1];
@@ -1932,16 +1960,19 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
   }
   __syncthreads();
   if (S.misc[M_FAIL]) return 0.0;
-  for (int k = a; k <= b; ++k) {
-    bool in = k >= sp.lo && k <= sp.hi;
-    bool dl = in && k > sp.lo, dr = in && k < sp.hi;
-    cplx<T> *A = site_ptr<T>(P, shot, k);
-    cplx<T> *out = X.ap + S.off[k - a];
-    if (in) {
-      materialize(sp, S.ppx, S.ppz, k, A, chi[k], chi[k + 1], dl, dr, out);
-    } else {
-      const int64_t tot = static_cast<int64_t>(chi[k]) * 2 * chi[k + 1];
-      for (int64_t e = tid(); e < tot; e += kThreads) out[e] = A[e];
+  // Doubled sites: one of up to kWarpSite elements by a warp, the span's sites
+  // in parallel (a site's tensor is a chain of index arithmetic and two loads:
+  // 5000 cycles, which the whole CTA would spend per site); a larger one by
+  // the CTA.  The span is the operator's support, so a <= lo <= hi <= b hold with
+  // equality.
+  constexpr int kWarpSite = 1024;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int k = pass == 0 ? a + warp_id() : a; k <= b; k += pass == 0 ? kWarps : 1) {
+      const bool dl = k > sp.lo, dr = k < sp.hi;
+      const bool by_warp = Dbond(k) * 2 * Dbond(k + 1) <= kWarpSite;
+      if (by_warp != (pass == 0)) continue;
+      materialize(sp, S.ppx, S.ppz, k, site_ptr<T>(P, shot, k), chi[k], chi[k + 1], dl, dr, X.ap + S.off[k - a],
+                  by_warp ? lane_id() : tid(), by_warp ? 32 : kThreads);
     }
   }
   __syncthreads();
@@ -2140,54 +2171,51 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       S.dmisc[D_FLOPS] += gemm_flops(r, n2, Dl) + svd_flops(r, n2);
       S.dmisc[D_PROF + 1 + (vec_from_columns ? PROF_NSVD_LARGE : PROF_NSVD_SMALL)] += 1.0;
     }
+    // S.lam holds the squared values, S.perm their order
     for (int i = tid(); i < n2; i += kThreads) {
-      if (!isfinite(static_cast<double>(X.lam[i]))) {
-        S.misc[M_FAIL] = STN_ENUMERIC;
-        X.lam[i] = T(0);
-      }
+      const T l = X.lam[i];
+      const bool bad = !isfinite(l);
+      if (bad) S.misc[M_FAIL] = STN_ENUMERIC;
+      S.lam[i] = bad ? T(0) : l;
     }
     __syncthreads();
     if (S.misc[M_FAIL]) return;
-    sort_desc<T>(n2, X.lam, S.perm);
-    for (int i = tid(); i < n2; i += kThreads) S.lam[i] = X.lam[S.perm[i]];
-    __syncthreads();
+    sort_desc<T>(n2, S.lam, S.perm);
     if (warp_id() == 0) {
       const int kmax = min(cap, P.chimax[k]);
-      const int keep = min(keep_count<T>(S.lam, n2, kmax, P.cutoff, P.delta), kmax);
-      double tot = 0, drop = 0;
-      for (int i = lane_id(); i < n2; i += 32) {
-        const double l = fmax(static_cast<double>(S.lam[i]), 0.0);
-        tot += l;
-        if (i >= keep) drop += l;
-      }
-      tot = warp_sum(tot);
-      drop = warp_sum(drop);
-      if (tid() == 0) {
-        if (tot > 0) S.dmisc[D_DISC] += drop / tot;
-        S.misc[M_KEEP] = keep;
-      }
+      const int keep = min(keep_count<T>(S.lam, S.perm, n2, kmax, P.cutoff, P.delta), kmax);
+      if (tid() == 0) S.misc[M_KEEP] = keep;
     }
     __syncthreads();
     const int keep = S.misc[M_KEEP];
+    if (warp_id() == kWarps - 1) {  // the others go on meanwhile
+      const double w = discarded_weight(S.lam, S.perm, n2, keep);
+      if (lane_id() == 0) S.dmisc[D_DISC] += w;
+    }
     // sorted, kept right singular vectors: Vs[:, c] = V[:, perm[c]], c < keep
-    // (or the rotated column of X over its norm)
+    // (or the rotated column of X over its norm), and the new right-canonical
+    // site k: B[c][s][r] = conj(Vs[(s*kappa + r)][c]).  Vectors rounded from pairs
+    // of floats to float are orthonormal to rounding; the others take one
+    // Newton-Schulz step in between.
+    cplx<T> *Bk = site_ptr<T>(P, shot, k);
+    const bool orthonormal = sizeof(T) == 4 && svd64;
     for (int e = tid(); e < n2 * keep; e += kThreads) {
       int i = e / keep, c = e % keep;
       cplx<T> v = Vc[static_cast<int64_t>(S.perm[c]) * n2 + i];
       if (vec_from_columns) {
-        T l = S.lam[c];
+        T l = S.lam[S.perm[c]];
         v = l > T(0) ? cscale(v, T(1) / sqrt(l)) : cmake<T>(i == c ? T(1) : T(0), 0);
       }
       X.vs[i * keep + c] = v;
+      if (orthonormal) Bk[c * n2 + i] = cconj(v);
     }
     __syncthreads();
-    // vectors rounded from pairs of floats to float are orthonormal to rounding
-    if (sizeof(T) == 8 || !svd64) reorthonormalize<T>(n2, keep, X.vs, X.e, X.y, S.tile);
-    // new right-canonical site k: B[c][s][r] = conj(Vs[(s*kappa + r)][c])
-    cplx<T> *Bk = site_ptr<T>(P, shot, k);
-    for (int e = tid(); e < keep * n2; e += kThreads) {
-      int c = e / n2, sr = e % n2;
-      Bk[e] = cconj(X.vs[sr * keep + c]);
+    if (!orthonormal) {
+      reorthonormalize<T>(n2, keep, X.vs, X.e, X.y, S.tile);
+      for (int e = tid(); e < keep * n2; e += kThreads) {
+        int c = e / n2, sr = e % n2;
+        Bk[e] = cconj(X.vs[sr * keep + c]);
+      }
     }
     // W = M Vs (Dl x keep)
     cgemm<T, 0, 0>(Dl, keep, n2, one, M, n2, X.vs, keep, zero, X.w, keep, S.tile);
@@ -2762,7 +2790,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
       const int ld = m | 1, steps = min(m, n);
       const cplx<T> *U = buf + n * ld;
       for (int e = tid(); e < m * steps; e += kThreads)
-        if (e / steps >= e % steps) vstore[e] = U[(e % steps) * ld + e / steps];
+        if (e / steps >= e % steps)  // unit vectors there, of length sqrt(2) in U
+          vstore[e] = cscale(U[(e % steps) * ld + e / steps], static_cast<T>(0.70710678118654752440));
     } else {
       qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, red, dm, vstore);
       form_q<T>(m, min(m, n), vstore, V, buf, SvdSmem<T>::elems);

@@ -115,7 +115,8 @@ template <typename S>
 struct Work;
 template <>
 struct Work<double> {
-  static constexpr double eps = 1.11e-16;
+  static constexpr double eps = 1.11e-16, tiny2 = 1e-32;
+  static __device__ __forceinline__ double minus(double x) { return -x; }
   static __device__ __forceinline__ double scale(double x, float) { return x; }
   static __device__ __forceinline__ int key(double x, int c) {  // column in the low bits, order of the high words
     const int hi = __double2hiint(x);
@@ -130,15 +131,24 @@ struct Work<double> {
   static __device__ __forceinline__ double of(double x) { return x; }
   static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
   static __device__ __forceinline__ double rsqrt(double x) { return rsqrt64(x); }
-  // w += conj(a) b, b += u w, s += |x|^2
+  // w += conj(a) b, b -= u w, s += |x|^2
   static __device__ __forceinline__ void dot(cplx<double> &w, cplx<double> a, cplx<double> b) { cfma(w, cconj(a), b); }
-  static __device__ __forceinline__ void axpy(cplx<double> &b, cplx<double> u, cplx<double> w) { cfma(b, u, w); }
+  static __device__ __forceinline__ void axpy(cplx<double> &b, cplx<double> u, cplx<double> w) {
+    cfma(b, cmake<double>(-u.re, -u.im), w);
+  }
   static __device__ __forceinline__ void sq(double &s, cplx<double> x) { s = fma(x.re, x.re, fma(x.im, x.im, s)); }
   static __device__ __forceinline__ double shfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 };
 template <>
+struct Work<float> {
+  static __device__ __forceinline__ float add(float a, float b) { return a + b; }
+  static __device__ __forceinline__ float norm(float a) { return a; }
+  static __device__ __forceinline__ float shfl(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+};
+template <>
 struct Work<ff> {
-  static constexpr float eps = 1.42e-14f;  // 2^-46
+  static constexpr float eps = 1.42e-14f, tiny2 = 1e-28f;  // 2^-46
+  static __device__ __forceinline__ ff minus(ff x) { return ff_neg(x); }
   static __device__ __forceinline__ ff scale(float x, float sc) { return ff_of(x * sc); }
   static __device__ __forceinline__ int key(ff x, int c) {
     const int b = __float_as_int(x.h);
@@ -160,10 +170,11 @@ struct Work<ff> {
     ff_fma(w.im, ff_neg(a.im), b.re);
   }
   static __device__ __forceinline__ void axpy(cplx<ff> &b, cplx<ff> u, cplx<ff> w) {
-    ff_fma(b.re, u.re, w.re);
-    ff_fma(b.re, ff_neg(u.im), w.im);
-    ff_fma(b.im, u.re, w.im);
-    ff_fma(b.im, u.im, w.re);
+    const ff nr = ff_neg(u.re), ni = ff_neg(u.im);
+    ff_fma(b.re, nr, w.re);
+    ff_fma(b.re, u.im, w.im);
+    ff_fma(b.im, nr, w.im);
+    ff_fma(b.im, ni, w.re);
     b.re = ff_norm(b.re);
     b.im = ff_norm(b.im);
   }
@@ -184,47 +195,77 @@ __device__ __forceinline__ S lane_sum(S v, int from) {
   for (int o = from; o > 0; o >>= 1) v = Work<S>::add(v, Work<S>::shfl(v, o));
   return v;
 }
-__device__ __forceinline__ float group_sum(float v) {
-#pragma unroll
-  for (int o = kGroup / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 __device__ __forceinline__ double group_sum(double v) { return lane_sum<double>(v, kGroup / 2); }
 __device__ __forceinline__ ff group_sum(ff v) { return lane_sum<ff>(v, kGroup / 2); }
+// Both parts of a complex number: at the first level half of the lanes take
+// over the real and half the imaginary part, so the sum costs the additions of
+// one number.
+template <typename S>
+__device__ __forceinline__ cplx<S> group_sum(cplx<S> w) {
+  const bool upper = (lane_id() & (kGroup / 2)) != 0;
+  const S re = Work<S>::norm(w.re), im = Work<S>::norm(w.im);
+  S v = Work<S>::add(upper ? im : re, Work<S>::shfl(upper ? re : im, kGroup / 2));
+#pragma unroll
+  for (int o = kGroup / 4; o > 0; o >>= 1) v = Work<S>::add(v, Work<S>::shfl(v, o));
+  const S other = Work<S>::shfl(v, kGroup / 2);
+  return cmake<S>(upper ? other : v, upper ? v : other);
+}
 
-// Scalars of the Hermitian reflector P = I - 2 u u^dag of a column x with
-// squared norm nx2 > 0 and first element al: P x = gamma e_1, gamma = -(al /
-// |al|) ||x||, u = (x - gamma e_1) sc.  With a = al / ||x||: sc = 1 / (||x||
-// sqrt(2 (1 + |a|))); an |a| below rounding takes the phase 1.
+// Scalars of the Hermitian reflector P = I - v v^dag of a column x with squared
+// norm nx2 > 0 and first element al: P x = gamma e_1, gamma = -(al / |al|)
+// ||x||, v = (x - gamma e_1) sc with 1 / sc^2 = ||x|| (||x|| + |al|).  Both
+// follow from q = 1 / (||x|| |al|): two square roots in a chain instead of
+// three.  An |al| below rounding takes the phase 1.
 template <typename S>
 __device__ __forceinline__ void reflector_scalars(cplx<S> al, S nx2, cplx<S> &gam, S &sc) {
   using K = Work<S>;
-  const S r = K::rsqrt(nx2), nx = K::mul(nx2, r);
-  const S ar = K::mul(al.re, r), ai = K::mul(al.im, r);
   S a2 = K::of(0);
-  K::sq(a2, cmake<S>(ar, ai));
+  K::sq(a2, al);
   a2 = K::norm(a2);
-  const bool tiny = !(K::value(a2) > 1e-32f);
-  const S ra = K::rsqrt(tiny ? K::of(1) : a2);
-  const S pr = tiny ? K::of(1) : K::mul(ar, ra), pi = tiny ? K::of(0) : K::mul(ai, ra);
-  const S one_a = K::add(K::of(1), tiny ? K::of(0) : K::mul(a2, ra));
-  const S m1 = K::of(-1);
-  gam = cmake<S>(K::mul(m1, K::mul(pr, nx)), K::mul(m1, K::mul(pi, nx)));
-  sc = K::mul(r, K::rsqrt(K::add(one_a, one_a)));
+  const bool tiny = !(K::value(a2) > K::tiny2 * K::value(nx2));
+  if (tiny) {
+    al = cmake<S>(K::of(1), K::of(0));
+    a2 = K::of(1);
+  }
+  const S p = K::mul(nx2, a2), q = K::rsqrt(p), t = K::mul(nx2, q);  // t = ||x|| / |al|
+  const S mt = K::minus(t);
+  gam = cmake<S>(K::mul(al.re, mt), K::mul(al.im, mt));
+  sc = K::rsqrt(tiny ? nx2 : K::add(nx2, K::mul(p, q)));
+}
+
+// The same for squared norms far from 1, whose products with |al|^2 could leave
+// the range of S.
+__device__ __forceinline__ void reflector_scaled(cplx<double> al, double nx2, cplx<double> &gam, double &sc) {
+  if (nx2 > 1e-130 && nx2 < 1e130) {
+    reflector_scalars<double>(al, nx2, gam, sc);
+  } else {
+    const double r = rsqrt64(nx2);
+    reflector_scalars<double>(cscale(al, r), 1.0, gam, sc);
+    gam = cscale(gam, nx2 * r);
+    sc *= r;
+  }
+}
+__device__ __forceinline__ void reflector_scaled(cplx<ff> al, ff nx2, cplx<ff> &gam, ff &sc) {
+  const int e = (__float_as_int(nx2.h) >> 24) - 63;  // nx2 in [2^(2 e - 1), 2^(2 e + 1))
+  const float f = __int_as_float((127 - e) << 23), g = __int_as_float((127 + e) << 23);
+  reflector_scalars<ff>(cmake<ff>(ff{al.re.h * f, al.re.l * f}, ff{al.im.h * f, al.im.l * f}),
+                        ff{nx2.h * f * f, nx2.l * f * f}, gam, sc);
+  gam = cmake<ff>(ff{gam.re.h * g, gam.re.l * g}, ff{gam.im.h * g, gam.im.l * g});
+  sc = ff{sc.h * f, sc.l * f};
 }
 
 // Reflector j of the column col[j..m-1] in the storage precision T into
 // u[j..m-1]; col[j] becomes gamma.  A column of norm up to 1e-30 gets none
-// (u = 0).  Norm and scalars in double, or for float in ff on the column scaled
-// by a power of two: single-precision squares of entries near 1e-20 would be
-// denormal, and a reflector built from such a norm not unitary.  One warp.
+// (u = 0).  Norm and scalars in double, or for float in ff; always on the column
+// scaled by a power of two: single-precision squares of entries near 1e-20 would
+// be denormal, and a reflector built from such a norm not unitary.  One warp.
 __device__ __forceinline__ void reflect_column(cplx<double> *col, cplx<double> *u, int j, int m) {
   double s = 0;
   for (int i = j + lane_id(); i < m; i += 32) Work<double>::sq(s, col[i]);
   s = lane_sum<double>(s, 16);
   cplx<double> gam = cmake<double>(0, 0);
   double sc = 0;
-  if (s > 1e-60) reflector_scalars<double>(col[j], s, gam, sc);
+  if (s > 1e-60) reflector_scaled(col[j], s, gam, sc);
   for (int i = j + lane_id(); i < m; i += 32) {
     cplx<double> x = col[i];
     if (i == j) x = cmake<double>(x.re - gam.re, x.im - gam.im);
@@ -245,7 +286,20 @@ __device__ __forceinline__ void reflect_column(cplx<float> *col, cplx<float> *u,
     ff_fma(s, ff_of(re), ff_of(re));
     ff_fma(s, ff_of(im), ff_of(im));
   }
-  s = lane_sum<ff>(s, 16);
+  // The sum over the warp in two integers, steps 2^-16 and 2^-40 (the largest
+  // component is in [1, 2), so a lane's sum is at most 8 rows per lane and 512
+  // rows give 2^28 in the first): two integer reductions for five levels of
+  // shuffles, and exact.
+  if (m <= 512) {
+    const int hi = __float2int_rn(s.h * 0x1p16f);
+    const int lo = __float2int_rn((__fadd_rn(s.h, -static_cast<float>(hi) * 0x1p-16f) + s.l) * 0x1p40f);
+    const int th = __reduce_add_sync(0xffffffffu, hi), tl = __reduce_add_sync(0xffffffffu, lo);
+    const float h0 = static_cast<float>(th);
+    s = ff_add(ff{h0 * 0x1p-16f, static_cast<float>(th - __float2int_rn(h0)) * 0x1p-16f},
+               ff_of(static_cast<float>(tl) * 0x1p-40f));
+  } else {
+    s = lane_sum<ff>(s, 16);
+  }
   cplx<float> gam = cmake<float>(0.f, 0.f);
   float sc = 0.f;
   if (sqrtf(s.h) * up > 1e-30f) {
@@ -315,10 +369,9 @@ static __device__ __noinline__ void qr_small(int m, int n, const cplx<T> *A, int
         if (on)
 #pragma unroll 4
           for (int i = i0; i < m; i += kGroup) cfma(w, cconj(u[i]), b[i]);
-        w.re = group_sum(w.re);
-        w.im = group_sum(w.im);
+        w = group_sum(w);
         if (on) {
-          w = cmake<T>(T(-2) * w.re, T(-2) * w.im);
+          w = cmake<T>(-w.re, -w.im);
 #pragma unroll 4
           for (int i = i0; i < m; i += kGroup) {
             cplx<T> x = b[i];
@@ -360,10 +413,9 @@ static __device__ __noinline__ void qr_small(int m, int n, const cplx<T> *A, int
       if (on)
 #pragma unroll 4
         for (int i = i0; i < m; i += kGroup) cfma(w, cconj(u[i]), q[i]);
-      w.re = group_sum(w.re);
-      w.im = group_sum(w.im);
+      w = group_sum(w);
       if (on) {
-        w = cmake<T>(T(-2) * w.re, T(-2) * w.im);
+        w = cmake<T>(-w.re, -w.im);
 #pragma unroll 4
         for (int i = i0; i < m; i += kGroup) {
           cplx<T> x = q[i];
@@ -577,12 +629,12 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
           cplx<S> *col = Bm + p * ld;
           cplx<S> gam;
           S sc;
-          reflector_scalars<S>(col[j], nx2, gam, sc);
+          reflector_scaled(col[j], nx2, gam, sc);
           for (int i = j + lane_id(); i < m; i += 32) {
             cplx<S> x = col[i];
             if (i == j) {
-              x.re = K::add(x.re, K::mul(K::of(-1), gam.re));
-              x.im = K::add(x.im, K::mul(K::of(-1), gam.im));
+              x.re = K::add(x.re, K::minus(gam.re));
+              x.im = K::add(x.im, K::minus(gam.im));
             }
             u[i] = cmake<S>(K::mul(x.re, sc), K::mul(x.im, sc));
           }
@@ -599,11 +651,9 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
             if (on)
 #pragma unroll 4
               for (int i = i0; i < m; i += kGroup) K::dot(w, u[i], b[i]);
-            w.re = group_sum(w.re);
-            w.im = group_sum(w.im);
+            w = group_sum(w);
             S s = K::of(0);
             if (on) {
-              w = cmake<S>(K::mul(K::of(-2), w.re), K::mul(K::of(-2), w.im));
 #pragma unroll 4
               for (int i = i0; i < m; i += kGroup) {
                 cplx<S> x = b[i];
@@ -668,8 +718,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
           if (on)
 #pragma unroll 4
             for (int c = gl; c < n; c += kGroup) K::dot(dot, Bm[c * ld + p], Bm[c * ld + q]);
-          dot.re = group_sum(dot.re);
-          dot.im = group_sum(dot.im);
+          dot = group_sum(dot);
           Rotation<S> rot;
           if (on && make_rotation(al, be, dot, limit, rot)) {
             rotated = true;
@@ -681,7 +730,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
               Bm[c * ld + q] = y;
             }
             if (gl == 0) {
-              const S a1 = K::add(al, K::mul(K::of(-1), rot.tg)), b1 = K::add(be, rot.tg);
+              const S a1 = K::add(al, K::minus(rot.tg)), b1 = K::add(be, rot.tg);
               nr[p] = K::value(a1) > 0 ? a1 : K::of(0);
               nr[q] = K::value(b1) > 0 ? b1 : K::of(0);
             }
