@@ -14,8 +14,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libstn.so")
-SOURCES = ["engine_f32.cu", "engine_f64.cu", "engine.cu", "engine_noalloc.cu", "peaks.cu", "tc_gemm.cu",
-           "program.cpp", "api.cpp"]
+SOURCES = ["engine_f32.cu", "engine_f64.cu", "engine_f32_light.cu", "engine_f64_light.cu", "engine.cu",
+           "engine_noalloc.cu", "peaks.cu", "tc_gemm.cu", "program.cpp", "api.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 

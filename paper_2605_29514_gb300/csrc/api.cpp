@@ -21,6 +21,8 @@ struct stn_ctx {
   int64_t max_shots = 0, shots = 0;
   uint64_t shot_offset = 0;
   int n = 0, W = 0, rec_bytes = 0, K = 0, grid = 1, svd_elems = 0;
+  bool light = false;                 // the round and adjoint kernels of 256 threads
+  int sms = 1, light_grid = 0, light_elems = 0;
   std::vector<int> chimax;
   std::vector<int64_t> site_off;
   int64_t slab_elems = 0;
@@ -119,6 +121,7 @@ stn::EngineParams params(const stn_ctx *c, int op_begin, int op_end, const doubl
   p.g_elems = c->plan.g_elems;
   p.work_c = c->plan.work_c;
   p.svd_elems = c->svd_elems;
+  p.svd_rule = c->svd_elems;
   p.svd64_all = c->cfg.precision == STN_PRECISION_C64_SVD64 ? 1 : 0;
   p.use_tc = c->cfg.precision != STN_PRECISION_C128 && c->cfg.gemm_units == STN_GEMM_TENSOR ? 1 : 0;
   p.err = c->d_err;
@@ -282,6 +285,18 @@ stn_status stn_create(const stn_config *cfg, int64_t max_shots, void *cuda_strea
     return STN_EINVAL;
   }
 
+  // Programs whose bonds stay at kLightBond run 256-thread CTAs, two per SM
+  // when the batch has more shots than SMs.  The choice depends on the
+  // configuration alone, so that a shot's result does not depend on the batch.
+  c->light = c->plan.work_c <= stn::kLightBond && !(cfg->gemm_units == STN_GEMM_TENSOR && cfg->precision != STN_PRECISION_C128) &&
+             cfg->precision != STN_PRECISION_C64_SVD64;
+  if (c->light) {
+    c->light_elems = cfg->precision == STN_PRECISION_C128 ? stn::round_light_elems_f64(n, c->W)
+                                                          : stn::round_light_elems_f32(n, c->W);
+    // the blocked SVD needs two columns, a reflector of the fallback one, the tiles their slice
+    if (c->light_elems < 2 * 4 * c->plan.work_c + 2176) c->light = false;
+  }
+
   int dev = 0, sms = 1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -290,6 +305,8 @@ stn_status stn_create(const stn_config *cfg, int64_t max_shots, void *cuda_strea
     return STN_ECUDA;
   }
   c->grid = static_cast<int>(std::min<int64_t>(max_shots, sms));
+  c->sms = sms;
+  c->light_grid = static_cast<int>(std::min<int64_t>(max_shots, 2 * sms));
 
   const int64_t S = max_shots;
   const size_t nn = static_cast<size_t>(2 * n);
@@ -318,7 +335,15 @@ stn_status stn_create(const stn_config *cfg, int64_t max_shots, void *cuda_strea
   A(dalloc(c, &c->d_obs, static_cast<size_t>(S)));
   A(dalloc(c, &c->d_det_table, sizeof(int32_t) * c->prog.det.size()));
   A(dalloc(c, &c->d_logical, sizeof(int32_t) * c->prog.logical.size()));
-  A(dalloc(c, &c->d_scratch, c->elem * static_cast<size_t>(c->grid) * c->plan.total));
+  {
+    const size_t per_cta = c->elem * static_cast<size_t>(c->plan.total);
+    bool got = c->light && dalloc(c, &c->d_scratch, per_cta * c->light_grid) == cudaSuccess;
+    if (c->light && !got) {  // one CTA per SM where the scratch of two does not fit
+      cudaGetLastError();
+      c->light_grid = c->grid;
+    }
+    if (!got) A(dalloc(c, &c->d_scratch, per_cta * c->grid));
+  }
   A(dalloc(c, &c->d_err, sizeof(int)));
   A(dalloc(c, &c->d_offset, sizeof(uint64_t)));
   A(dalloc(c, &c->d_ticket, sizeof(int)));
@@ -436,17 +461,38 @@ stn_status stn_begin_batch(stn_ctx *c, int64_t shots, uint64_t shot_offset) {
   return STN_OK;
 }
 
+// CTAs of a round or adjoint launch over `shots` shots.
+static int round_grid(const stn_ctx *c, int64_t shots) {
+  return static_cast<int>(std::min<int64_t>(c->light ? c->light_grid : c->grid, shots));
+}
+
+static cudaError_t launch_round(stn_ctx *c, stn::EngineParams p, int grid) {
+  if (!c->light) return stn::launch_round(c->cfg.precision, p, grid, c->stream);
+  p.svd_elems = c->light_elems;
+  return c->cfg.precision == STN_PRECISION_C128 ? stn::launch_round_light_f64(p, grid, c->sms, c->stream)
+                                                : stn::launch_round_light_f32(p, grid, c->sms, c->stream);
+}
+
+static cudaError_t launch_adjoint(stn_ctx *c, stn::EngineParams p, double *grad, int grid) {
+  const bool f64 = c->cfg.precision == STN_PRECISION_C128;
+  if (!c->light)
+    return f64 ? stn::launch_adjoint_f64(p, grad, grid, c->stream) : stn::launch_adjoint_f32(p, grad, grid, c->stream);
+  p.svd_elems = c->light_elems;
+  return f64 ? stn::launch_adjoint_light_f64(p, grad, grid, c->stream)
+             : stn::launch_adjoint_light_f32(p, grad, grid, c->stream);
+}
+
 static stn_status launch_ops(stn_ctx *c, int op_begin, int op_end, const double *d_theta) {
   if (c->shots < 1) return fail(c, STN_EINVAL, "no batch: call stn_begin_batch first");
   if (!d_theta && c->K > 0) return fail(c, STN_EINVAL, "theta is NULL");
   stn::EngineParams p = params(c, op_begin, op_end, d_theta ? d_theta : c->d_theta);
-  int grid = static_cast<int>(std::min<int64_t>(c->grid, c->shots));
+  const int grid = round_grid(c, c->shots);
   cudaError_t e = cudaSuccess;
   if (c->shots > grid) {  // more shots than CTAs: take them from a queue
     e = cudaMemsetAsync(c->d_ticket, 0, sizeof(int), c->stream);
     p.ticket = c->d_ticket;
   }
-  if (e == cudaSuccess) e = stn::launch_round(c->cfg.precision, p, grid, c->stream);
+  if (e == cudaSuccess) e = launch_round(c, p, grid);
   if (e != cudaSuccess) return cuda_fail(c, e, "round kernel");
   return STN_OK;
 }
@@ -668,13 +714,13 @@ stn_status stn_capture_batch(stn_ctx *c, int64_t shots, const double *d_theta) {
   p.shot_offset_dev = c->d_offset;
   cudaError_t le = cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream);
   if (le == cudaSuccess) le = stn::launch_init(c->cfg.precision, p, c->stream);
-  const int grid = static_cast<int>(std::min<int64_t>(c->grid, shots));
+  const int grid = round_grid(c, shots);
   if (shots > grid) p.ticket = c->d_ticket;
   for (size_t st = 0; le == cudaSuccess && st + 1 < c->prog.step_begin.size(); ++st) {
     p.op_begin = c->prog.step_begin[st];
     p.op_end = c->prog.step_begin[st + 1];
     if (p.ticket) le = cudaMemsetAsync(c->d_ticket, 0, sizeof(int), c->stream);
-    if (le == cudaSuccess) le = stn::launch_round(c->cfg.precision, p, grid, c->stream);
+    if (le == cudaSuccess) le = launch_round(c, p, grid);
   }
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(c->stream, &g);
@@ -765,15 +811,14 @@ stn_status stn_logprob_grad(stn_ctx *c, uint64_t shot_offset, int64_t n_rec, con
   p.rot_ord = d_rot;
   p.n_ops_total = n_ops;
   p.n_rot = n_rot;
-  const int grid = static_cast<int>(std::min<int64_t>(c->grid, n_rec));
-  e = stn::launch_round(c->cfg.precision, p, grid, c->stream);
+  const int grid = round_grid(c, n_rec);
+  e = launch_round(c, p, grid);
   if (e != cudaSuccess) return cuda_fail(c, e, "adjoint forward");
   st = stn_sync(c);
   if (st != STN_OK) return st;
   e = cudaMemcpy(h_logp, c->d_logp, sizeof(double) * n_rec, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(c, e, "stn_logprob_grad logp");
-  e = c->cfg.precision == STN_PRECISION_C128 ? stn::launch_adjoint_f64(p, d_grad, grid, c->stream)
-                                             : stn::launch_adjoint_f32(p, d_grad, grid, c->stream);
+  e = launch_adjoint(c, p, d_grad, grid);
   if (e != cudaSuccess) return cuda_fail(c, e, "adjoint backward");
   st = stn_sync(c);
   if (st != STN_OK) return st;

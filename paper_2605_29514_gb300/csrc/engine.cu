@@ -82,17 +82,6 @@ ScratchPlan plan_scratch(int n, const int *chimax, int chi_cap) {
   return p;
 }
 
-// Largest SVD buffer (complex elements, at most SvdSmem) that keeps the round
-// kernel within the 227 KB of shared memory a CTA may use.
-template <typename T>
-static int svd_elems_for(int n, int W) {
-  const size_t limit = 227 * 1024;
-  size_t base = smem_bytes<T>(n, W, 0);
-  if (base + 64 >= limit) return 0;
-  size_t e = (limit - base - 64) / sizeof(cplx<T>);
-  return static_cast<int>(e < static_cast<size_t>(SvdSmem<T>::elems) ? e : SvdSmem<T>::elems);
-}
-
 int round_kernel_svd_elems(int precision, int n, int W) {
   return precision == 0 ? svd_elems_for<double>(n, W) : svd_elems_for<float>(n, W);
 }

@@ -8,7 +8,6 @@
 
 namespace stn {
 
-constexpr int kThreads = 512;   // threads per CTA of the round kernel (16 warps)
 constexpr double kNearThreshold = 1e-5;
 // Phase counters (SM clock cycles of the CTA, summed over ops): left sweep,
 // right-sweep SVDs, the rest of the right sweep, expectation values, the whole
@@ -55,6 +54,7 @@ struct EngineParams {
   int64_t scratch_elems, ap_elems, g_elems;
   int work_c;               // largest bond of the plan (sizes the work area)
   int svd_elems;            // complex elements of the shared-memory SVD buffer
+  int svd_rule;             // ... of the 512-thread kernel: bounds the bonds decomposed in pairs of floats
   int svd64_all;            // complex64 path: every bond SVD in double precision
   int use_tc;               // complex64 and gemm_units = STN_GEMM_TENSOR: large contractions on tcgen05
   int *err;                 // first error code seen on the device
@@ -99,6 +99,17 @@ cudaError_t launch_dense_check_f32(int what, int m, int n, void *A, void *V, voi
 cudaError_t launch_dense_check_f64(int what, int m, int n, void *A, void *V, void *sig2, int use_smem,
                                    cudaStream_t s);
 cudaError_t launch_round(int precision, const EngineParams &p, int grid, cudaStream_t s);
+// The same kernels with 256 threads and at most half of an SM's shared memory
+// a CTA (engine_f32_light.cu, engine_f64_light.cu), for programs whose bonds
+// stay at kLightBond or below; *_elems: their shared SVD buffer, in complex
+// elements.
+constexpr int kLightBond = 64;
+cudaError_t launch_round_light_f32(const EngineParams &p, int grid, int sms, cudaStream_t s);
+cudaError_t launch_round_light_f64(const EngineParams &p, int grid, int sms, cudaStream_t s);
+cudaError_t launch_adjoint_light_f32(const EngineParams &p, double *grad, int grid, cudaStream_t s);
+cudaError_t launch_adjoint_light_f64(const EngineParams &p, double *grad, int grid, cudaStream_t s);
+int round_light_elems_f32(int n, int W);
+int round_light_elems_f64(int n, int W);
 cudaError_t launch_adjoint_f32(const EngineParams &p, double *grad, int grid, cudaStream_t s);
 cudaError_t launch_adjoint_f64(const EngineParams &p, double *grad, int grid, cudaStream_t s);
 cudaError_t launch_diag_f32(const EngineParams &p, int what, int target, int cut, const int32_t *lq, int nl,

@@ -4,7 +4,7 @@
 namespace stn {
 
 cudaError_t launch_round_f32(const EngineParams &p, int grid, cudaStream_t s) {
-  return launch_round_t<float>(p, grid, s);
+  return launch_round_t<float>(p, grid, grid, s);
 }
 
 cudaError_t launch_init_f32(const EngineParams &p, cudaStream_t s) { return launch_init_t<float>(p, s); }

@@ -4,7 +4,7 @@
 namespace stn {
 
 cudaError_t launch_round_f64(const EngineParams &p, int grid, cudaStream_t s) {
-  return launch_round_t<double>(p, grid, s);
+  return launch_round_t<double>(p, grid, grid, s);
 }
 
 cudaError_t launch_init_f64(const EngineParams &p, cudaStream_t s) { return launch_init_t<double>(p, s); }

@@ -1,0 +1,18 @@
+// Complex128 instantiations of the round and adjoint kernels with 256 threads and two
+// CTAs per SM.
+#define STN_CTA_THREADS 256
+#include "engine_kernels.cuh"
+
+namespace stn {
+
+cudaError_t launch_round_light_f64(const EngineParams &p, int grid, int sms, cudaStream_t s) {
+  return launch_round_t<double>(p, grid, sms, s);
+}
+
+cudaError_t launch_adjoint_light_f64(const EngineParams &p, double *grad, int grid, cudaStream_t s) {
+  return launch_adjoint_t<double>(p, grad, grid, s);
+}
+
+int round_light_elems_f64(int n, int W) { return svd_elems_for<double>(n, W); }
+
+}  // namespace stn

@@ -31,7 +31,27 @@
 #include "../../include/stn.h"
 #include "engine.h"
 
-namespace stn {
+// The CTA size is a compile-time constant of the including file: 512 threads
+// (one CTA per SM, all of its shared memory), or 256 for programs whose bonds
+// stay small (kLightBond): barriers and reductions over half the warps are
+// cheaper where a step's work fills neither, and two such CTAs fit an SM.  With
+// one shot per SM, 256 threads took a d = 5 round at theta = 1e-3 from 120 to
+// 107 ms, d = 7 from 194 to 174 ms, one d = 3 shot in complex128 from 23.7 to
+// 20.7 ms; 128 threads were up to 10 % better at bonds of 4 and 10 % worse at 32.
+#ifndef STN_CTA_THREADS
+#define STN_CTA_THREADS 512
+#endif
+#if STN_CTA_THREADS == 512
+#define STN_BEGIN namespace stn { inline namespace cta512 {
+#else
+#define STN_BEGIN namespace stn { inline namespace cta256 {
+#endif
+#define STN_END }}
+
+STN_BEGIN
+
+constexpr int kThreads = STN_CTA_THREADS;
+constexpr bool kLight = kThreads < 512;
 
 // ---------------------------------------------------------------------------
 // complex arithmetic
@@ -114,7 +134,7 @@ struct SvdSmem<double> {
 };
 constexpr int kMaxVec = 1024;  // longest Householder vector (4 * largest bond)
 
-constexpr int kBM = 64, kBN = 64, kBK = 16, kPad = 4;
+constexpr int kTileElems = 2176;  // complex elements of a contraction's shared-memory tiles
 
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): two 32x32->64-bit
@@ -154,8 +174,9 @@ __device__ __forceinline__ E *in_smem(const void *p) {
 }
 
 // Sum of one double per thread over the CTA: a shuffle reduction per warp,
-// then every thread adds the warps' partial sums (red: kThreads doubles of
-// smem, of which the first kThreads / 32 are used).  Two barriers.
+// then every thread adds the warps' partial sums (red: the first kThreads / 32
+// of kRedDoubles doubles of shared memory).  Two barriers.
+constexpr int kRedDoubles = 512;
 static __device__ double block_sum(double v, double *red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -305,7 +326,7 @@ static __device__ __forceinline__ void tc_disable() {
   __syncthreads();
 }
 
-static_assert(kThreads == 512, "the tensor-core staging and epilogue map 512 threads onto the tiles");
+static_assert(kLight || kThreads == 512, "the tensor-core staging and epilogue map 512 threads onto the tiles");
 
 __device__ __forceinline__ void st_f4(float *p, float a, float b, float c, float d) {
   *reinterpret_cast<float4 *>(p) = make_float4(a, b, c, d);
@@ -539,9 +560,9 @@ static __device__ __forceinline__ void cgemm_rows(int M, int N, int K, cplx<T> a
   __syncthreads();
 }
 
-// Larger products in shared-memory tiles of 32 MR x 64 outputs, a slice of
-// kTileK of the k range at a time: thread (ty, tx) of a 32 x 16 grid owns rows
-// ty + 32 a and columns tx + 16 b, so a k step reads MR + 4 elements, which the
+// Larger products in shared-memory tiles of kTY MR x 64 outputs, a slice of
+// kTileK of the k range at a time: thread (ty, tx) of a kTY x 16 grid owns rows
+// ty + kTY a and columns tx + 16 b, so a k step reads MR + 4 elements, which the
 // lanes of a warp read without conflicts, for 4 MR products.  The next slice is fetched from global memory into
 // registers while the present one is multiplied.
 constexpr int kTileK = 8;
@@ -550,14 +571,14 @@ template <typename T, int TA, int TB, int MR>
 static __device__ __forceinline__ void cgemm_tiles(int M, int N, int K, cplx<T> alpha, const cplx<T> *A, int lda,
                                                    const cplx<T> *B, int ldb, cplx<T> beta, cplx<T> *C, int ldc,
                                                    cplx<T> *tile) {
-  constexpr int RM = 32 * MR, RN = 64, LA = RM + 2, LB = RN + 2;  // padded rows of a slice
+  constexpr int kTY = kThreads / 16, RM = kTY * MR, RN = 64, LA = RM + 2, LB = RN + 2;  // padded rows of a slice
   constexpr int NA = RM * kTileK / kThreads, NB = RN * kTileK / kThreads;
-  static_assert(NA * kThreads == RM * kTileK && NB == 1 && kTileK * (LA + LB) <= kBK * (kBM + kPad + kBN + kPad), "tile");
+  static_assert(NA * kThreads == RM * kTileK && NB * kThreads == RN * kTileK && kTileK * (LA + LB) <= kTileElems, "tile");
   cplx<T> *As = in_smem<cplx<T>>(tile), *Bs = As + kTileK * LA;
   const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
   for (int i0 = 0; i0 < M; i0 += RM)
     for (int j0 = 0; j0 < N; j0 += RN) {
-      cplx<T> acc[MR][4], pa[NA], pb;
+      cplx<T> acc[MR][4], pa[NA], pb[NB];
 #pragma unroll
       for (int a = 0; a < MR; ++a)
 #pragma unroll
@@ -572,12 +593,15 @@ static __device__ __forceinline__ void cgemm_tiles(int M, int N, int K, cplx<T> 
           if (gi < M && gk < K)
             pa[r] = TA == 0 ? A[static_cast<int64_t>(gi) * lda + gk] : cconj(A[static_cast<int64_t>(gk) * lda + gi]);
         }
-        const int k = TB == 0 ? threadIdx.x / RN : threadIdx.x % kTileK;
-        const int j = TB == 0 ? threadIdx.x % RN : threadIdx.x / kTileK;
-        const int gj = j0 + j, gk = k0 + k;
-        pb = cmake<T>(0, 0);
-        if (gj < N && gk < K)
-          pb = TB == 0 ? B[static_cast<int64_t>(gk) * ldb + gj] : cconj(B[static_cast<int64_t>(gj) * ldb + gk]);
+#pragma unroll
+        for (int r = 0; r < NB; ++r) {
+          const int e = threadIdx.x + r * kThreads;
+          const int k = TB == 0 ? e / RN : e % kTileK, j = TB == 0 ? e % RN : e / kTileK;
+          const int gj = j0 + j, gk = k0 + k;
+          pb[r] = cmake<T>(0, 0);
+          if (gj < N && gk < K)
+            pb[r] = TB == 0 ? B[static_cast<int64_t>(gk) * ldb + gj] : cconj(B[static_cast<int64_t>(gj) * ldb + gk]);
+        }
       };
       fetch(0);
       for (int k0 = 0; k0 < K; k0 += kTileK) {
@@ -587,15 +611,19 @@ static __device__ __forceinline__ void cgemm_tiles(int M, int N, int K, cplx<T> 
           if (TA == 0) As[(e % kTileK) * LA + e / kTileK] = pa[r];
           else As[(e / RM) * LA + e % RM] = pa[r];
         }
-        if (TB == 0) Bs[(threadIdx.x / RN) * LB + threadIdx.x % RN] = pb;
-        else Bs[(threadIdx.x % kTileK) * LB + threadIdx.x / kTileK] = pb;
+#pragma unroll
+        for (int r = 0; r < NB; ++r) {
+          const int e = threadIdx.x + r * kThreads;
+          if (TB == 0) Bs[(e / RN) * LB + e % RN] = pb[r];
+          else Bs[(e % kTileK) * LB + e / kTileK] = pb[r];
+        }
         __syncthreads();
         if (k0 + kTileK < K) fetch(k0 + kTileK);
 #pragma unroll
         for (int k = 0; k < kTileK; ++k) {
           cplx<T> av[MR], bv[4];
 #pragma unroll
-          for (int a = 0; a < MR; ++a) av[a] = As[k * LA + ty + 32 * a];
+          for (int a = 0; a < MR; ++a) av[a] = As[k * LA + ty + kTY * a];
 #pragma unroll
           for (int b = 0; b < 4; ++b) bv[b] = Bs[k * LB + tx + 16 * b];
 #pragma unroll
@@ -607,7 +635,7 @@ static __device__ __forceinline__ void cgemm_tiles(int M, int N, int K, cplx<T> 
       }
 #pragma unroll
       for (int a = 0; a < MR; ++a) {
-        const int gi = i0 + ty + 32 * a;
+        const int gi = i0 + ty + kTY * a;
         if (gi >= M) continue;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
@@ -631,7 +659,7 @@ template <typename T, int TA, int TB>
 static __device__ __noinline__ void cgemm(int M, int N, int K, cplx<T> alpha, const cplx<T> *A, int lda,
                       const cplx<T> *B, int ldb, cplx<T> beta, cplx<T> *C, int ldc,
                       cplx<T> *tile) {
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 4 && !kLight) {
     if (g_tc.enabled && M >= 64 && N >= 32 && K >= kTcK) {
       cgemm_tc<TA, TB>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
       return;
@@ -1061,9 +1089,9 @@ static __device__ void onesided_epilogue(int m, int n, const cplx<T> *C, T *sig2
 constexpr int kMaxSweepsF = 15, kMaxSweepsD = 20;
 constexpr int kMaxBlockedSweepsF = 30, kMaxBlockedSweepsD = 40;
 
-}  // namespace stn
+STN_END
 #include "small_bond.cuh"
-namespace stn {
+STN_BEGIN
 
 // Unblocked: C and V wherever they are (shared memory for small problems).
 template <typename T>
@@ -1369,7 +1397,7 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
   // between the prologue and the epilogue.
   const int per_sweep = nb + (nbe - 1) * (nbe / 2);
   int *last_mod = reinterpret_cast<int *>(red);
-  const bool skipping = nb <= static_cast<int>(kThreads * sizeof(double) / sizeof(int));
+  const bool skipping = nb <= static_cast<int>(kRedDoubles * sizeof(double) / sizeof(int));
   if (skipping) {
     for (int i = tid(); i < nb; i += kThreads) last_mod[i] = -1;
     __syncthreads();
@@ -1598,7 +1626,7 @@ struct Smem {
   double *red;
   double *dmisc;
   cplx<T> *tile;
-  cplx<T> *jbuf, *uvec;
+  cplx<T> *jbuf;
   int *rdim;
   T *lam;
   MpoSpec<T> *spec;
@@ -1618,15 +1646,26 @@ __host__ __device__ size_t smem_bytes(int n, int W, int svd_elems) {
   add(sizeof(int) * 16);              // misc
   add(sizeof(int64_t) * (n + 2));     // off
   add(sizeof(int64_t) * (n + 2));     // goff
-  add(sizeof(double) * kThreads);     // red
+  add(sizeof(double) * kRedDoubles);  // red
   add(sizeof(double) * 24);           // dmisc
-  add(sizeof(cplx<T>) * kBK * (kBM + kPad + kBN + kPad));  // tile
+  if (!kLight) add(sizeof(cplx<T>) * kTileElems);  // tile
   add(sizeof(cplx<T>) * svd_elems);  // jbuf
-  add(sizeof(cplx<T>) * kMaxVec);     // uvec
   add(sizeof(int) * (n + 2));         // rdim
   add(sizeof(T) * kLamElems);         // lam (also the register-visit reductions)
   add(sizeof(MpoSpec<T>));
   return b;
+}
+
+// Largest SVD buffer (complex elements, at most SvdSmem) that keeps the round
+// kernel within the 227 KB of shared memory a CTA may use, or two CTAs within
+// the 228 KB of an SM (1 KB of which each CTA reserves).
+template <typename T>
+inline int svd_elems_for(int n, int W) {
+  const size_t limit = (kLight ? 112 : 227) * 1024;
+  const size_t base = smem_bytes<T>(n, W, 0);
+  if (base + 64 >= limit) return 0;
+  const size_t e = (limit - base - 64) / sizeof(cplx<T>);
+  return static_cast<int>(e < static_cast<size_t>(SvdSmem<T>::elems) ? e : SvdSmem<T>::elems);
 }
 
 template <typename T>
@@ -1648,11 +1687,11 @@ static __device__ Smem<T> carve(char *base, int n, int W, int svd_elems) {
   s.misc = reinterpret_cast<int *>(take(sizeof(int) * 16));
   s.off = reinterpret_cast<int64_t *>(take(sizeof(int64_t) * (n + 2)));
   s.goff = reinterpret_cast<int64_t *>(take(sizeof(int64_t) * (n + 2)));
-  s.red = reinterpret_cast<double *>(take(sizeof(double) * kThreads));
+  s.red = reinterpret_cast<double *>(take(sizeof(double) * kRedDoubles));
   s.dmisc = reinterpret_cast<double *>(take(sizeof(double) * 24));
-  s.tile = reinterpret_cast<cplx<T> *>(take(sizeof(cplx<T>) * kBK * (kBM + kPad + kBN + kPad)));
+  if (!kLight) s.tile = reinterpret_cast<cplx<T> *>(take(sizeof(cplx<T>) * kTileElems));
   s.jbuf = reinterpret_cast<cplx<T> *>(take(sizeof(cplx<T>) * svd_elems));
-  s.uvec = reinterpret_cast<cplx<T> *>(take(sizeof(cplx<T>) * kMaxVec));
+  if (kLight) s.tile = s.jbuf;  // free whenever a GEMM runs
   s.rdim = reinterpret_cast<int *>(take(sizeof(int) * (n + 2)));
   s.lam = reinterpret_cast<T *>(take(sizeof(T) * kLamElems));
   s.spec = reinterpret_cast<MpoSpec<T> *>(take(sizeof(MpoSpec<T>)));
@@ -2071,13 +2110,17 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
     // 16-byte numbers is decomposed in pairs of floats: FP32 Jacobi rotations leave
     // the small singular directions with an absolute error of about
     // sqrt(#rotations) eps sigma_1, which would be dropped or kept wrongly at
-    // every sweep.  In complex128, every bond whose matrix fits takes this path.
+    // every sweep.  In complex128, every bond of up to
+    // kSmallSvdCols columns takes this path.
     bool vec_from_columns = false;
     const int dscale = static_cast<int>(sizeof(double) / sizeof(T));
-    const bool svd64 = n2 <= kSmallSvdCols && n2 * (r | 1) * dscale <= P.svd_elems && r * dscale <= kMaxVec &&
-                       (sizeof(T) == 8 || 2 * (r * n2 + n2 * n2) <= P.svd_elems);
+    const bool svd64 = n2 <= kSmallSvdCols && r <= kMaxVec && (sizeof(T) == 8 || 2 * (r * n2 + n2 * n2) <= P.svd_rule);
     if (svd64) {
-      svd_small<T>(r, n2, X.y, X.v, X.lam, P.cutoff, S.jbuf, S.uvec, S.red);
+      const int elems = n2 * (r | 1) * dscale;
+      if (elems + r * dscale <= P.svd_elems)
+        svd_small<T, true>(r, n2, X.y, X.v, X.lam, P.cutoff, S.jbuf, S.jbuf + elems, S.red);
+      else  // X.t is free in the right sweep and holds it: r n2 <= 4 c^2 numbers of 16 bytes
+        svd_small<T, false>(r, n2, X.y, X.v, X.lam, P.cutoff, X.t, S.jbuf, S.red);
       Vc = X.v;
     } else if (sizeof(T) == 4 && P.svd64_all) {
       // Complex64 contractions with every SVD in double precision: the large
@@ -2426,8 +2469,11 @@ static __device__ void set_meas_spec(const Smem<T> &S, int bit) {
 }
 
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(kThreads, 1) round_kernel(EngineParams P) {
+// B: resident CTAs per SM the registers are allotted for.  With 256 threads and
+// one CTA per SM (a batch of up to one shot per SM) the 255 registers a thread
+// may then use save spills: 5 % of a d = 5 round against B = 2.
+template <typename T, int B>
+__global__ void __launch_bounds__(kThreads, B) round_kernel(EngineParams P) {
   extern __shared__ __align__(16) char smem_raw[];
   const int n = P.n, W = P.W;
   Smem<T> S = carve<T>(smem_raw, n, W, P.svd_elems);
@@ -2436,7 +2482,7 @@ __global__ void __launch_bounds__(kThreads, 1) round_kernel(EngineParams P) {
   // contractions run on the tensor cores, staged in the shared SVD buffer
   // (free whenever a GEMM runs)
   bool tc_alloc = false;
-  if constexpr (sizeof(T) == 4) tc_alloc = P.use_tc && static_cast<int64_t>(P.svd_elems) * 2 >= kTcStageFloats;
+  if constexpr (sizeof(T) == 4 && !kLight) tc_alloc = P.use_tc && static_cast<int64_t>(P.svd_elems) * 2 >= kTcStageFloats;
   if (tc_alloc) tc_setup(reinterpret_cast<float *>(S.jbuf));
   else tc_disable();
   bool tc_live = tc_alloc;  // CTA-uniform
@@ -2741,7 +2787,7 @@ static __device__ void svd_bond(int m, int n, const cplx<T> *A, cplx<T> *work, c
                                 cplx<T> *uv, double *red, double *dm, int *flag, float *rv_wrk) {
   if constexpr (sizeof(T) == 8) {
     if (n <= kSmallSvdCols && n * (m | 1) <= SvdSmem<T>::elems) {
-      const int rank = svd_small<T>(m, n, A, V, sig2, 0.0, buf, uv, red);
+      const int rank = svd_small<T, true>(m, n, A, V, sig2, 0.0, buf, uv, red);
       for (int e = tid() + rank * n; e < n * n; e += kThreads) V[e] = cmake<T>(0, 0);
       return;
     }
@@ -2774,7 +2820,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
   extern __shared__ __align__(16) char smem_raw[];
   tc_disable();
   double *red = reinterpret_cast<double *>(smem_raw);
-  double *dm = red + kThreads;
+  double *dm = red + kRedDoubles;
   int *flag = reinterpret_cast<int *>(dm + 16);
   cplx<T> *uv = reinterpret_cast<cplx<T> *>(flag + 16);
   cplx<T> *buf = uv + kMaxVec;
@@ -2818,7 +2864,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
 template <typename T>
 cudaError_t launch_dense_check_t(int what, int m, int n, void *A, void *V, void *sig2, int use_smem,
                                         cudaStream_t s) {
-  size_t smem = sizeof(double) * (kThreads + 16) + sizeof(int) * 16 + sizeof(cplx<T>) * kMaxVec;
+  size_t smem = sizeof(double) * (kRedDoubles + 16) + sizeof(int) * 16 + sizeof(cplx<T>) * kMaxVec;
   smem += sizeof(cplx<T>) * SvdSmem<T>::elems;  // QR panel, SVD matrix or staged column blocks
   smem += sizeof(float) * kRvWrkFloats;           // register-visit reductions
   cudaError_t e = cudaFuncSetAttribute(dense_check_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2840,7 +2886,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_gemm_kernel(int ta, int tb,
                                                                  int *status) {
   extern __shared__ __align__(16) char smem_raw[];
   cplx<T> *tile = reinterpret_cast<cplx<T> *>(smem_raw);
-  float *stage = reinterpret_cast<float *>(tile + kBK * (kBM + kPad + kBN + kPad));
+  float *stage = reinterpret_cast<float *>(tile + kTileElems);
   bool tc = false;
   if constexpr (sizeof(T) == 4) tc = use_tc != 0;
   if (tc) tc_setup(stage);
@@ -2859,7 +2905,7 @@ template <typename T>
 cudaError_t launch_dense_gemm_t(int ta, int tb, int m, int n, int k, const double *alpha, const void *A, int lda,
                                 const void *B, int ldb, const double *beta, void *C, int ldc, int use_tc, int *status,
                                 cudaStream_t s) {
-  size_t smem = sizeof(cplx<T>) * kBK * (kBM + kPad + kBN + kPad);
+  size_t smem = sizeof(cplx<T>) * kTileElems;
   if (sizeof(T) == 4 && use_tc) smem += sizeof(float) * kTcStageFloats;
   cudaError_t e = cudaFuncSetAttribute(dense_gemm_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
@@ -3054,7 +3100,7 @@ static __device__ cplx<double> mps_overlap(const EngineParams &P, const Smem<T> 
 // U |v><0|_j; every application is followed by the truncating sweep.
 // Clifford gates and Paulis only changed the frame and leave mu alone.
 template <typename T>
-__global__ void __launch_bounds__(kThreads, 1) adjoint_kernel(EngineParams P, double *grad) {
+__global__ void __launch_bounds__(kThreads, kLight ? 2 : 1) adjoint_kernel(EngineParams P, double *grad) {
   extern __shared__ __align__(16) char smem_raw[];
   tc_disable();
   const int n = P.n, W = P.W;
@@ -3161,14 +3207,22 @@ cudaError_t launch_diag_t(const EngineParams &p, int what, int target, int cut, 
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_round_t(const EngineParams &p, int grid, cudaStream_t s) {
+template <typename T, int B>
+cudaError_t launch_round_b(const EngineParams &p, int grid, cudaStream_t s) {
   size_t smem = smem_bytes<T>(p.n, p.W, p.svd_elems);
-  cudaError_t e = cudaFuncSetAttribute(round_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(round_kernel<T, B>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  round_kernel<T><<<grid, kThreads, smem, s>>>(p);
+  round_kernel<T, B><<<grid, kThreads, smem, s>>>(p);
   return cudaGetLastError();
 }
 
-}  // namespace stn
+template <typename T>
+cudaError_t launch_round_t(const EngineParams &p, int grid, int sms, cudaStream_t s) {
+  if constexpr (kLight) {
+    if (grid > sms) return launch_round_b<T, 2>(p, grid, s);
+  }
+  return launch_round_b<T, 1>(p, grid, s);
+}
+
+STN_END

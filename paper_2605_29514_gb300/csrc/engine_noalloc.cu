@@ -25,7 +25,7 @@ __global__ void __launch_bounds__(kThreads, 1) svd_noalloc_kernel(int m, int n, 
   extern __shared__ __align__(16) char smem_raw[];
   tc_disable();
   double *red = reinterpret_cast<double *>(smem_raw);
-  double *dm = red + kThreads;
+  double *dm = red + kRedDoubles;
   int *flag = reinterpret_cast<int *>(dm + 16);
   cplx<T> *uv = reinterpret_cast<cplx<T> *>(flag + 16), *buf = uv + kMaxVec;
   float *rv_wrk = reinterpret_cast<float *>(buf + SvdSmem<T>::elems);
@@ -62,7 +62,7 @@ static cudaError_t launch_svd_noalloc_t(int m, int n, const void *C, void *V, vo
   void *work = nullptr;
   cudaError_t e = noalloc_scratch_ptr(&work);
   if (e != cudaSuccess) return e;
-  size_t smem = sizeof(double) * (kThreads + 16) + sizeof(int) * 16 + sizeof(cplx<T>) * kMaxVec +
+  size_t smem = sizeof(double) * (kRedDoubles + 16) + sizeof(int) * 16 + sizeof(cplx<T>) * kMaxVec +
                 sizeof(cplx<T>) * SvdSmem<T>::elems + sizeof(float) * kRvWrkFloats;
   e = cudaFuncSetAttribute(svd_noalloc_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(smem));

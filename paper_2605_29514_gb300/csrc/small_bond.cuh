@@ -14,7 +14,7 @@
 // has to be better than single precision in pairs of floats (ff, 48 bits): the
 // SVD it used to run in double, and the norms and scalars of its reflectors.
 
-namespace stn {
+STN_BEGIN
 
 constexpr int kGroup = 8;                       // lanes that share a column
 constexpr int kGroups = kThreads / kGroup;      // columns in flight
@@ -553,16 +553,21 @@ __device__ __forceinline__ void rotate_pair(cplx<ff> &x, cplx<ff> &y, const Rota
 // rotating them against each other was slower: it leaves the sweeps converging
 // linearly.)
 //
-// buf: n (m | 1) 16-byte complex numbers; u: m of them; nr: n doubles (all
-// shared memory); n <= kSmallSvdCols.  CTA-wide.
-template <typename T>
+// buf: n (m | 1) 16-byte complex numbers in shared memory, or (SM false) n m of
+// them in global memory, for the few bonds that are too large for a CTA that has
+// half of an SM: the same arithmetic, so a result does not depend on where the
+// matrix was; u: m of them; nr: n doubles (both shared memory); n <=
+// kSmallSvdCols.  CTA-wide.
+template <typename T, bool SM>
 static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cplx<T> *V, T *lam, double cutoff_,
                                              void *buf_, void *u_, void *nr_) {
   using S = std::conditional_t<sizeof(T) == 8, double, ff>;
   using K = Work<S>;
   using R = decltype(K::value(S()));  // double or float
-  const int ld = m | 1, steps = min(m, n);
-  cplx<S> *Bm = in_smem<cplx<S>>(buf_), *u = in_smem<cplx<S>>(u_);
+  const int ld = SM ? m | 1 : m, steps = min(m, n);
+  cplx<S> *Bm, *u = in_smem<cplx<S>>(u_);
+  if constexpr (SM) Bm = in_smem<cplx<S>>(buf_);
+  else Bm = static_cast<cplx<S> *>(buf_);
   S *nr = in_smem<S>(nr_);
   const int gl = lane_id() & (kGroup - 1), g = tid() / kGroup;
   float down = 1.f, up = 1.f;  // ff: the matrix scaled by a power of two to entries up to 1
@@ -760,4 +765,4 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   return rank;
 }
 
-}  // namespace stn
+STN_END
