@@ -335,21 +335,21 @@ stn_status stn_create(const stn_config *cfg, int64_t max_shots, void *cuda_strea
   A(dalloc(c, &c->d_obs, static_cast<size_t>(S)));
   A(dalloc(c, &c->d_det_table, sizeof(int32_t) * c->prog.det.size()));
   A(dalloc(c, &c->d_logical, sizeof(int32_t) * c->prog.logical.size()));
-  {
-    const size_t per_cta = c->elem * static_cast<size_t>(c->plan.total);
-    bool got = c->light && dalloc(c, &c->d_scratch, per_cta * c->light_grid) == cudaSuccess;
-    if (c->light && !got) {  // one CTA per SM where the scratch of two does not fit
-      cudaGetLastError();
-      c->light_grid = c->grid;
-    }
-    if (!got) A(dalloc(c, &c->d_scratch, per_cta * c->grid));
-  }
   A(dalloc(c, &c->d_err, sizeof(int)));
   A(dalloc(c, &c->d_offset, sizeof(uint64_t)));
   A(dalloc(c, &c->d_ticket, sizeof(int)));
   A(dalloc(c, &c->d_diag, sizeof(double) * std::max<int64_t>(S, 512)));
   A(dalloc(c, &c->d_diag_count, sizeof(int)));
   A(dalloc(c, &c->d_diag_q, sizeof(int32_t) * n));
+  {  // last, so that the second CTA's share takes nothing that the context cannot do without
+    const size_t per_cta = c->elem * static_cast<size_t>(c->plan.total);
+    bool got = ok && c->light && dalloc(c, &c->d_scratch, per_cta * c->light_grid) == cudaSuccess;
+    if (c->light && !got) {  // one CTA per SM where the scratch of two does not fit
+      cudaGetLastError();
+      c->light_grid = c->grid;
+    }
+    if (!got) A(dalloc(c, &c->d_scratch, per_cta * c->grid));
+  }
   if (!ok) {
     stn_destroy(c);
     cudaGetLastError();
@@ -758,6 +758,21 @@ stn_status stn_sample_shots(stn_ctx *c, int64_t shots, uint64_t shot_offset, con
   return stn_read_records(c, h_records, h_born, h_stats);
 }
 
+// Gives back the scratch of the second CTA per SM, for a call that needs the
+// memory; a captured graph holds its address, so then it stays.
+static bool drop_second_scratch(stn_ctx *c) {
+  if (c->light_grid <= c->grid || !c->light || c->graph) return false;
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
+  void *old = c->d_scratch;
+  if (dalloc(c, &c->d_scratch, c->elem * static_cast<size_t>(c->plan.total) * c->grid) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  c->light_grid = c->grid;
+  c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), old));
+  cudaFree(old);
+  return true;
+}
 
 stn_status stn_logprob_grad(stn_ctx *c, uint64_t shot_offset, int64_t n_rec, const uint8_t *h_records,
                             const double *h_theta, double *h_logp, double *h_grad) {
@@ -774,6 +789,8 @@ stn_status stn_logprob_grad(stn_ctx *c, uint64_t shot_offset, int64_t n_rec, con
   const size_t phi_bytes = c->elem * static_cast<size_t>(n_rec) * std::max(1, n_rot) * c->slab_elems;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return cuda_fail(c, cudaGetLastError(), "memory info");
+  if (phi_bytes > free_b / 10 * 8 && drop_second_scratch(c) && cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
+    return cuda_fail(c, cudaGetLastError(), "memory info");
   if (phi_bytes > free_b / 10 * 8)
     return fail(c, STN_ENOMEM, "stn_logprob_grad: the states after every rotation do not fit device memory");
   AdjointBuffers buf;
