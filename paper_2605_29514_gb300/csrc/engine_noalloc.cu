@@ -24,12 +24,9 @@ __global__ void __launch_bounds__(kThreads, 1) svd_noalloc_kernel(int m, int n, 
                                                                   cplx<T> *work, cplx<T> *V, T *sig2) {
   extern __shared__ __align__(16) char smem_raw[];
   tc_disable();
-  double *red = reinterpret_cast<double *>(smem_raw);
-  double *dm = red + kRedDoubles;
-  int *flag = reinterpret_cast<int *>(dm + 16);
-  cplx<T> *uv = reinterpret_cast<cplx<T> *>(flag + 16), *buf = uv + kMaxVec;
-  float *rv_wrk = reinterpret_cast<float *>(buf + SvdSmem<T>::elems);
-  svd_bond<T>(m, n, C, work, V, sig2, buf, uv, red, dm, flag, rv_wrk);
+  const DenseSmem s = dense_smem<T>(smem_raw);
+  svd_bond<T, false>(m, n, C, work, V, sig2, reinterpret_cast<cplx<T> *>(s.buf), reinterpret_cast<cplx<T> *>(s.uv), s.red,
+                     s.flag, s.rv_wrk);
 }
 
 size_t noalloc_scratch_bytes() { return kNoAllocScratchBytes; }
@@ -62,8 +59,10 @@ static cudaError_t launch_svd_noalloc_t(int m, int n, const void *C, void *V, vo
   void *work = nullptr;
   cudaError_t e = noalloc_scratch_ptr(&work);
   if (e != cudaSuccess) return e;
-  size_t smem = sizeof(double) * (kRedDoubles + 16) + sizeof(int) * 16 + sizeof(cplx<T>) * kMaxVec +
-                sizeof(cplx<T>) * SvdSmem<T>::elems + sizeof(float) * kRvWrkFloats;
+  if (shares_svd<T>(m, n))
+    return launch_dense_shared<T>(true, m, n, const_cast<cplx<T> *>(static_cast<const cplx<T> *>(C)),
+                                  static_cast<cplx<T> *>(work), static_cast<cplx<T> *>(V), static_cast<T *>(sig2), s);
+  const size_t smem = dense_smem_bytes<T>();
   e = cudaFuncSetAttribute(svd_noalloc_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(smem));
   if (e != cudaSuccess) return e;

@@ -115,3 +115,32 @@ def test_pivoted_svd_zero_and_non_finite():
             assert torch.all(ds == 0) and torch.all(dv == 0)
         else:
             assert not torch.any(torch.isfinite(ds))
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("cutoff,cap,theta,basis", [(1e-12, 64, 0.05, "Z"), (1e-12, 64, 0.0225, "X"), (5e-6, 64, 0.05, "X"),
+                                                    (1e-3, 64, 0.05, "X"), (1e-3, 3, 0.1, "Z"), (5e-6, 1, 0.1, "X")])
+def test_truncations_against_oracle(precision, cutoff, cap, theta, basis):
+    """Truncations whose Jacobi ends without a sweep that finds nothing: full and
+    capped ranks, cutoffs inside and below the spectrum.  Born probabilities and
+    the largest bond against the oracle: rounding, 1e-9 in complex128 and 5e-5 in
+    complex64 for states of a few hundred truncations."""
+    if precision == 1 and cutoff < 5e-6:
+        pytest.skip("below the rounding of complex64")
+    from oracle.shot import make_program, run_shot
+    from workloads import D3_EXACT, theta_table
+
+    w = D3_EXACT.with_(rounds=1, p=0.0, theta=theta, memory_basis=basis, precision=precision, chi_cap=cap,
+                       svd_cutoff=cutoff, degeneracy_tol=cutoff)
+    sim = stn.Simulator(w, max_shots=3)
+    angles = theta_table(w, sim.n_pairs)
+    out = sim.sample_shots(3, 11, angles)
+    prog = make_program(w)
+    for s in range(3):
+        ref = run_shot(w, 11 + s, angles, prog)
+        assert list(out["bits"][s]) == list(ref.record)
+        rb = np.array(ref.born)
+        assert (np.abs(out["born"][s] - rb) / np.maximum(rb, 1e-4)).max() < (1e-9 if precision == 0 else 5e-5)
+        if precision == 0:
+            assert out["max_chi"][s] == ref.max_chi
+    sim.close()
