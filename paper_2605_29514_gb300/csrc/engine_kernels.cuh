@@ -687,6 +687,58 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+constexpr int kMaxSweepsF = 15, kMaxSweepsD = 20;  // Jacobi
+
+STN_END
+
+#include "small_bond.cuh"
+
+STN_BEGIN
+
+// A dense problem that is called alone may be shared by the CTAs of a cluster
+// (CL): its matrix lies in global memory, and phases that write it end in
+// share_sync, whose release and acquire order that memory over the cluster.
+template <bool CL>
+__device__ __forceinline__ int share_rank() {
+  int r = 0;
+  if constexpr (CL) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+template <bool CL>
+__device__ __forceinline__ int share_size() {
+  int r = 1;
+  if constexpr (CL) asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+template <bool CL>
+__device__ __forceinline__ void share_sync() {
+  if constexpr (CL) {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  } else {
+    __syncthreads();
+  }
+}
+// An int of the shared memory of CTA `rank` of the cluster, at this CTA's address p.
+template <bool CL>
+__device__ __forceinline__ int share_load(const int *p, int rank) {
+  if constexpr (!CL) return *p;
+  uint32_t a;
+  int v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+template <bool CL>
+__device__ __forceinline__ void share_store(int *p, int rank, int v) {
+  if constexpr (!CL) {
+    *p = v;
+  } else {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+  }
+}
+
 // Householder QR of B (m x n, row-major, leading dimension ld), in place: on
 // return rows 0..min(m,n)-1 hold R (upper trapezoidal) and the rest is zero.
 // Each step uses the Hermitian reflector P = I - 2 u u^dag with
@@ -697,7 +749,9 @@ __device__ __forceinline__ T warp_sum(T v) {
 // T_kk = 2, T[0:k, k] = -2 T[0:k, 0:k] V[:, 0:k]^dag u_k) is applied to the
 // trailing columns at once, one thread per column, so the trailing matrix is
 // read and written twice per panel rather than per column.  pbuf needs
-// m (nb + 1) + 2 nb^2 complex elements (nb is reduced to fit).  CTA-wide.
+// m (nb + 1) + 2 nb^2 complex elements (nb is reduced to fit).  CTA-wide, or over
+// a cluster: every CTA factors the panel for itself, the first one writes it back,
+// and the trailing columns are split.
 constexpr int kQrPanel = 16;
 
 static __device__ __forceinline__ int qr_panel_width(int m, int pbuf_elems) {
@@ -725,14 +779,14 @@ static __device__ void wy_t_factor(int mr, int jb, int nb, int ldv, const cplx<T
     if (lane_id() == 0) G[a * nb + b] = cmake<T>(gr, gi);
   }
   __syncthreads();
-  if (tid() == 0) {
+  if (warp_id() == 0) {  // a lane owns a row of T
+    const int a = lane_id();
     for (int k = 0; k < jb; ++k) {
-      Tm[k * nb + k] = cmake<T>(2, 0);
-      for (int a = 0; a < k; ++a) {
-        cplx<T> acc = cmake<T>(0, 0);
+      cplx<T> acc = cmake<T>(0, 0);
+      if (a < k)
         for (int b = a; b < k; ++b) cfma(acc, Tm[a * nb + b], G[b * nb + k]);
-        Tm[a * nb + k] = cscale(acc, T(-2));
-      }
+      if (a < k) Tm[a * nb + k] = cscale(acc, T(-2));
+      if (a == k) Tm[k * nb + k] = cmake<T>(2, 0);
     }
   }
   __syncthreads();
@@ -741,11 +795,10 @@ static __device__ void wy_t_factor(int mr, int jb, int nb, int ldv, const cplx<T
 // With vstore (row-major m x min(m,n)), the reflectors are also kept there
 // (column j holds u_j in rows j..m-1; rows above are not written) so that
 // form_q can build Q explicitly.
-template <typename T>
+template <typename T, bool CL = false>
 static __device__ __noinline__ void qr_r_inplace(int m, int n, cplx<T> *B, int ld, cplx<T> *pbuf_, int pbuf_elems,
-                                                 double *red_, double *dm_, cplx<T> *vstore = nullptr) {
+                                                 cplx<T> *vstore = nullptr) {
   cplx<T> *pbuf = in_smem<cplx<T>>(pbuf_);
-  double *red = in_smem<double>(red_), *dm = in_smem<double>(dm_);
   const int steps = min(m, n);
   const int nb = qr_panel_width(m, pbuf_elems);
   // rows of the panel padded to an odd number of elements, so that a column
@@ -761,70 +814,61 @@ static __device__ __noinline__ void qr_r_inplace(int m, int n, cplx<T> *B, int l
       const int i = e / jb, c = e % jb;
       Vp[i * ldv + c] = B[static_cast<int64_t>(j0 + i) * ld + j0 + c];
     }
+    share_sync<CL>();
+    // Panel: a warp owns a column (two of a 256-thread CTA's).  The warp that has
+    // brought column jj + 1 up to date forms its reflector at once, in place, while
+    // the others still update theirs, so a column takes one barrier.  (Norm by the
+    // whole CTA, scalars by one thread in double, four barriers: about 12,000
+    // cycles a column.)
+    const bool writes = share_rank<CL>() == 0;
+    auto reflect = [&](int jj) {
+      const Reflector<T> h = column_reflector(Vp + jj, ldv, jj, mr, true);
+      cplx<T> *out = B + static_cast<int64_t>(j0) * ld + j0 + jj;
+      for (int i = lane_id(); i < mr; i += 32) {
+        cplx<T> &x = Vp[i * ldv + jj];
+        if (i < jj) {  // rows above the diagonal are final R entries
+          if (writes) out[static_cast<int64_t>(i) * ld] = x;
+          x = cmake<T>(0, 0);
+        } else {
+          x = h.vector(x, i == jj);
+          if (writes) out[static_cast<int64_t>(i) * ld] = i == jj ? h.diagonal() : cmake<T>(0, 0);
+        }
+      }
+      __syncwarp();
+    };
+    if (warp_id() == 0) reflect(0);
     __syncthreads();
-    for (int jj = 0; jj < jb; ++jj) {
-      double nx2 = 0;
-      for (int i = jj + tid(); i < mr; i += kThreads) nx2 += cabs2d(Vp[i * ldv + jj]);
-      nx2 = block_sum(nx2, red);
-      // rows above the diagonal of this column are final R entries
-      for (int i = tid(); i < jj; i += kThreads) B[static_cast<int64_t>(j0 + i) * ld + j0 + jj] = Vp[i * ldv + jj];
-      if (!(nx2 > 1e-60)) {  // (numerically) zero column: no reflector, R row jj is final
-        for (int i = tid(); i < mr; i += kThreads) {
-          if (i >= jj) B[static_cast<int64_t>(j0 + i) * ld + j0 + jj] = cmake<T>(0, 0);
-          Vp[i * ldv + jj] = cmake<T>(0, 0);
-        }
-        __syncthreads();
-        continue;
-      }
-      if (tid() == 0) {
-        cplx<T> al = Vp[jj * ldv + jj];
-        double aa = sqrt(cabs2d(al));
-        double nx = sqrt(nx2);
-        double pr = aa > 0 ? al.re / aa : 1.0, pi = aa > 0 ? al.im / aa : 0.0;
-        dm[0] = -pr * nx;  // gamma
-        dm[1] = -pi * nx;
-        dm[2] = 1.0 / sqrt(2.0 * nx * (nx + aa));  // 1 / ||x - gamma e_1||
-      }
-      __syncthreads();
-      const cplx<T> gam = cmake<T>(static_cast<T>(dm[0]), static_cast<T>(dm[1]));
-      const T sc = static_cast<T>(dm[2]);
-      for (int i = tid(); i < mr; i += kThreads) {
-        cplx<T> u = cmake<T>(0, 0);
-        if (i >= jj) {
-          cplx<T> x = Vp[i * ldv + jj];
-          if (i == jj) x = cmake<T>(x.re - gam.re, x.im - gam.im);
-          u = cscale(x, sc);
-          B[static_cast<int64_t>(j0 + i) * ld + j0 + jj] = i == jj ? gam : cmake<T>(0, 0);
-        }
-        Vp[i * ldv + jj] = u;
-      }
-      __syncthreads();
-      // the rest of the panel: b <- b - 2 u (u^dag b), one warp per column
-      for (int c = jj + 1 + warp_id(); c < jb; c += kWarps) {
+    for (int jj = 0; jj + 1 < jb; ++jj) {
+      for (int c = warp_id(); c < jb; c += kWarps) {
+        if (c <= jj) continue;  // b <- b - 2 u (u^dag b)
         T sr = 0, si = 0;
+#pragma unroll 4
         for (int i = jj + lane_id(); i < mr; i += 32) {
           const cplx<T> u = Vp[i * ldv + jj], b = Vp[i * ldv + c];
           sr += u.re * b.re + u.im * b.im;
           si += u.re * b.im - u.im * b.re;
         }
-        sr = __shfl_sync(0xffffffffu, warp_sum(sr), 0);
-        si = __shfl_sync(0xffffffffu, warp_sum(si), 0);
+        sr = warp_sum(sr);
+        si = warp_sum(si);
         const cplx<T> s2 = cmake<T>(T(2) * sr, T(2) * si);
+#pragma unroll 4
         for (int i = jj + lane_id(); i < mr; i += 32) {
           const cplx<T> t = cmul(Vp[i * ldv + jj], s2);
           cplx<T> &b = Vp[i * ldv + c];
           b = cmake<T>(b.re - t.re, b.im - t.im);
         }
+        __syncwarp();
+        if (c == jj + 1) reflect(c);
       }
       __syncthreads();
     }
-    if (vstore != nullptr)
+    if (vstore != nullptr && writes)
       for (int e = tid(); e < mr * jb; e += kThreads) {
         const int i = e / jb, c = e % jb;
         vstore[static_cast<int64_t>(j0 + i) * steps + j0 + c] = Vp[i * ldv + c];
       }
     if (j0 + jb >= n) {  // no trailing columns
-      __syncthreads();
+      share_sync<CL>();
       continue;
     }
     wy_t_factor<T>(mr, jb, nb, ldv, Vp, Tm, G);
@@ -838,9 +882,11 @@ static __device__ __noinline__ void qr_r_inplace(int m, int n, cplx<T> *B, int l
     {
       const int nt = n - j0 - jb;
       int ns = 1;
-      while (ns < 8 && nt * 2 * ns <= kThreads) ns *= 2;
+      const int ranks = share_size<CL>();
+      while (ns < 8 && nt * 2 * ns <= kThreads * ranks) ns *= 2;
       const int cpw = 32 / ns, s = lane_id() / cpw;
-      for (int cb = j0 + jb + warp_id() * cpw; cb < n; cb += kWarps * cpw) {  // warp-uniform trip count
+      for (int cb = j0 + jb + (warp_id() * ranks + share_rank<CL>()) * cpw; cb < n;
+           cb += kWarps * ranks * cpw) {  // warp-uniform trip count
         const int c = cb + lane_id() % cpw;
         const bool valid = c < n;
         cplx<T> w[kQrPanel];
@@ -912,7 +958,7 @@ static __device__ __noinline__ void qr_r_inplace(int m, int n, cplx<T> *B, int l
         }
       }
     }
-    __syncthreads();
+    share_sync<CL>();
   }
 }
 
@@ -1075,23 +1121,19 @@ static __device__ T onesided_prologue(int m, int n, const cplx<T> *C, cplx<T> *V
   return static_cast<T>(static_cast<double>(Eps<T>::v) * static_cast<double>(Eps<T>::v) * fro2);
 }
 
-template <typename T>
+template <typename T, bool CL = false>
 static __device__ void onesided_epilogue(int m, int n, const cplx<T> *C, T *sig2) {
-  for (int j = warp_id(); j < n; j += kWarps) {
+  for (int j = warp_id() + kWarps * share_rank<CL>(); j < n; j += kWarps * share_size<CL>()) {
     double a = 0;
     for (int i = lane_id(); i < m; i += 32) a += cabs2d(C[static_cast<int64_t>(j) * m + i]);
     a = warp_sum(a);
     if (lane_id() == 0) sig2[j] = static_cast<T>(a);
   }
-  __syncthreads();
+  share_sync<CL>();
 }
 
-constexpr int kMaxSweepsF = 15, kMaxSweepsD = 20;
 constexpr int kMaxBlockedSweepsF = 30, kMaxBlockedSweepsD = 40;
 
-STN_END
-#include "small_bond.cuh"
-STN_BEGIN
 
 // Unblocked: C and V wherever they are (shared memory for small problems).
 template <typename T>
@@ -1371,7 +1413,11 @@ static __device__ bool cross_visit_dispatch(int m, cplx<T> *C, int c0, int wI, i
 // complex64 problem without V and with m <= kThreads visits block pairs
 // with cross_visit_regs (blocks of 16 columns); the blocks alone are still
 // staged in shared memory.
-template <typename T>
+//
+// Over a cluster (CL, without V) the blocks, and then the disjoint block pairs of a
+// round, go to its CTAs in turn; the stamps live in the first one's shared memory,
+// read and written in place.  The arithmetic is that of one CTA.
+template <typename T, bool CL = false>
 static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C, cplx<T> *V, T *sig2, int *flag,
                                      double *red, cplx<T> *sbuf, int sbuf_elems, float *rv_wrk = nullptr) {
   const T negligible = onesided_prologue<T>(m, n, C, V, red);
@@ -1385,6 +1431,7 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
   while (bw > 1 && static_cast<int64_t>(m) * 2 * bw + (withV ? 4 * bw * bw : 0) + 2 * bw > sbuf_elems) --bw;
   if (bw > 2 * kWarps) bw -= bw % (2 * kWarps);  // whole waves of half warps per step
   if (regs) bw = 16;
+  else if (CL) bw = min(bw, max(4, (n + 2 * share_size<CL>() - 1) / (2 * share_size<CL>())));  // a pair per CTA
   const int nb = (n + bw - 1) / bw, nbe = nb + (nb & 1);
   const int max_sweeps = sizeof(T) == 4 ? kMaxBlockedSweepsF : kMaxBlockedSweepsD;
   int *any = flag + 1;
@@ -1400,11 +1447,17 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
   const bool skipping = nb <= static_cast<int>(kRedDoubles * sizeof(double) / sizeof(int));
   if (skipping) {
     for (int i = tid(); i < nb; i += kThreads) last_mod[i] = -1;
-    __syncthreads();
+    share_sync<CL>();
   }
+  const int ranks = share_size<CL>(), rank = share_rank<CL>();
+  auto mark = [&](int I, int J, int stamp) {  // thread 0
+    share_store<CL>(&last_mod[I], 0, stamp);
+    share_store<CL>(&last_mod[J], 0, stamp);
+  };
 
   auto visit = [&](int I, int J, int stamp) {
-    if (skipping && stamp >= per_sweep && last_mod[I] < stamp - per_sweep && last_mod[J] < stamp - per_sweep)
+    if (skipping && stamp >= per_sweep && share_load<CL>(&last_mod[I], 0) < stamp - per_sweep &&
+        share_load<CL>(&last_mod[J], 0) < stamp - per_sweep)
       return;
     const bool self = I == J;
     const int c0 = I * bw, wI = min(bw, n - c0);
@@ -1412,7 +1465,7 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
     const int w = wI + wJ;
     if (regs && !self) {
       if (cross_visit_dispatch<T>(m, C, c0, wI, c1, wJ, tol, negligible, rv_wrk)) {
-        if (skipping && tid() == 0) last_mod[I] = last_mod[J] = stamp;
+        if (skipping && tid() == 0) mark(I, J, stamp);
         if (tid() == 0) *any = 1;
       }
       __syncthreads();
@@ -1467,7 +1520,7 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
     const int rotated = *flag;
     __syncthreads();
     if (!rotated) return;
-    if (skipping && tid() == 0) last_mod[I] = last_mod[J] = stamp;
+    if (skipping && tid() == 0) mark(I, J, stamp);
     for (int e = tid(); e < m * w; e += kThreads) {
       const int c = e / m, i = e % m;
       C[static_cast<int64_t>(gcol(c)) * m + i] = Cb[e];
@@ -1510,9 +1563,10 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
     if (tid() == 0) *any = 0;
     __syncthreads();
     const int base = sweep * per_sweep;
-    for (int I = 0; I < nb; ++I) visit(I, I, base + I);
+    for (int I = rank; I < nb; I += ranks) visit(I, I, base + I);
+    if (CL) share_sync<CL>();
     for (int round = 0; round < nbe - 1; ++round) {
-      for (int bp = 0; bp < nbe / 2; ++bp) {
+      for (int bp = rank; bp < nbe / 2; bp += ranks) {
         int I, J;
         if (bp == 0) { I = nbe - 1; J = round; }
         else { I = (round + bp) % (nbe - 1); J = (round - bp + (nbe - 1)) % (nbe - 1); }
@@ -1520,13 +1574,15 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
         if (J >= nb) continue;
         visit(I, J, base + nb + round * (nbe / 2) + bp);
       }
+      if (CL) share_sync<CL>();
     }
-    __syncthreads();
-    const int f = *any;
-    __syncthreads();
+    share_sync<CL>();
+    int f = 0;
+    for (int r = 0; r < ranks; ++r) f |= share_load<CL>(any, r);
+    share_sync<CL>();
     if (!f) break;
   }
-  onesided_epilogue<T>(m, n, C, sig2);
+  onesided_epilogue<T, CL>(m, n, C, sig2);
   return sweeps;
 }
 
@@ -1901,7 +1957,7 @@ static __device__ __noinline__ void mps_move_center(const EngineParams &P, const
     } else {
       for (int e = tid(); e < m * r; e += kThreads) X.t[e] = A[e];
       __syncthreads();
-      qr_r_inplace<T>(m, r, X.t, r, S.jbuf, P.svd_elems, S.red, S.dmisc + 4, X.h);
+      qr_r_inplace<T>(m, r, X.t, r, S.jbuf, P.svd_elems, X.h);
       form_q<T>(m, steps, X.h, X.y, S.jbuf, P.svd_elems);
       cgemm<T, 0, 0>(steps, 2 * r2, r, one, X.t, r, Bn, 2 * r2, zero, X.w, 2 * r2, S.tile);
       for (int e = tid(); e < m * steps; e += kThreads) A[e] = X.y[e];
@@ -1933,7 +1989,7 @@ static __device__ __noinline__ void mps_move_center(const EngineParams &P, const
         X.t[e] = cconj(A[static_cast<int64_t>(i) * m + j]);
       }
       __syncthreads();
-      qr_r_inplace<T>(m, l, X.t, l, S.jbuf, P.svd_elems, S.red, S.dmisc + 4, X.h);
+      qr_r_inplace<T>(m, l, X.t, l, S.jbuf, P.svd_elems, X.h);
       form_q<T>(m, steps, X.h, X.y, S.jbuf, P.svd_elems);
       cgemm<T, 0, 1>(2 * ll, steps, l, one, Am, l, X.t, l, zero, X.w, steps, S.tile);
       for (int e = tid(); e < steps * m; e += kThreads) {
@@ -2048,7 +2104,7 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
         for (int e = tid(); e < m * Dr; e += kThreads) X.t[e] = src[e];
         __syncthreads();
       }
-      qr_r_inplace<T>(m, Dr, X.t, Dr, S.jbuf, P.svd_elems, S.red, S.dmisc + 4);
+      qr_r_inplace<T>(m, Dr, X.t, Dr, S.jbuf, P.svd_elems);
       for (int e = tid(); e < rn * Dr; e += kThreads) Rout[e] = X.t[e];
     }
     if (tid() == 0) S.rdim[k + 1 - a] = rn;
@@ -2140,7 +2196,7 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
         Cd[e] = cmake<double>(static_cast<double>(X.y[e].re), static_cast<double>(X.y[e].im));
       __syncthreads();
       const long long tqr = clock64();
-      qr_r_inplace<double>(r, n2, Cd, n2, jd, P.svd_elems / 2, S.red, S.dmisc + 4);
+      qr_r_inplace<double>(r, n2, Cd, n2, jd, P.svd_elems / 2);
       if (tid() == 0) S.dmisc[D_PROF + 1 + PROF_SVD_QR] += static_cast<double>(clock64() - tqr);
       const int kx = min(r, n2);
       for (int e = tid(); e < n2 * kx; e += kThreads) Cd[e] = cconj(Cd[e]);
@@ -2181,7 +2237,7 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
         return;
       }
       const long long tqr = clock64();
-      qr_r_inplace<T>(r, n2, X.y, n2, S.jbuf, P.svd_elems, S.red, S.dmisc + 4);
+      qr_r_inplace<T>(r, n2, X.y, n2, S.jbuf, P.svd_elems);
       if (tid() == 0) S.dmisc[D_PROF + 1 + PROF_SVD_QR] += static_cast<double>(clock64() - tqr);
       const int kx = min(r, n2);
       // complex64 with more than one block of 16 columns: blocked Jacobi
@@ -2781,35 +2837,139 @@ __global__ void init_kernel(EngineParams P) {
 // squared singular values of the row-major m x n matrix A.  complex128 whose
 // matrix fits shared memory: svd_small on A.  Else, on the copy in `work`
 // (work may be A): R factor, Jacobi on X = R^dag (n x k), V = normalised
-// columns of X.
+// columns of X; with CL by the CTAs of a cluster.
 template <typename T>
+__host__ __device__ __forceinline__ bool svd_bond_small(int m, int n) {
+  return sizeof(T) == 8 && n <= kSmallSvdCols && n * (m | 1) <= SvdSmem<T>::elems;
+}
+
+template <typename T, bool CL>
 static __device__ void svd_bond(int m, int n, const cplx<T> *A, cplx<T> *work, cplx<T> *V, T *sig2, cplx<T> *buf,
-                                cplx<T> *uv, double *red, double *dm, int *flag, float *rv_wrk) {
-  if constexpr (sizeof(T) == 8) {
-    if (n <= kSmallSvdCols && n * (m | 1) <= SvdSmem<T>::elems) {
+                                cplx<T> *uv, double *red, int *flag, float *rv_wrk) {
+  if constexpr (sizeof(T) == 8 && !CL) {
+    if (svd_bond_small<T>(m, n)) {
       const int rank = svd_small<T, true>(m, n, A, V, sig2, 0.0, buf, uv, red);
       for (int e = tid() + rank * n; e < n * n; e += kThreads) V[e] = cmake<T>(0, 0);
       return;
     }
   }
-  if (work != A)
-    for (int e = tid(); e < m * n; e += kThreads) work[e] = A[e];
-  __syncthreads();
-  qr_r_inplace<T>(m, n, work, n, buf, SvdSmem<T>::elems, red, dm);
+  const int t0 = tid() + kThreads * share_rank<CL>(), step = kThreads * share_size<CL>();
+  // complex128 matrices that svd_small would take whatever their scale: to entries
+  // around 1, by a power of two that every CTA finds for itself
+  T down = 1, up = 1;
+  if constexpr (sizeof(T) == 8 && CL) {
+    int *top = reinterpret_cast<int *>(red);
+    if (tid() == 0) *top = 0;
+    __syncthreads();
+    int hi = 0;
+    for (int e = tid(); e < m * n; e += kThreads)
+      hi = max(hi, max(__double2hiint(A[e].re) & 0x7fffffff, __double2hiint(A[e].im) & 0x7fffffff));
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane_id() == 0) atomicMax(top, hi);
+    __syncthreads();
+    const int ex = min(2045, max(1, *top >> 20));
+    down = __hiloint2double((2046 - ex) << 20, 0);
+    up = __hiloint2double(ex << 20, 0);
+    share_sync<CL>();  // A may be work
+  }
+  if (work != A || CL)
+    for (int e = t0; e < m * n; e += step) work[e] = cscale(A[e], down);
+  share_sync<CL>();
+  qr_r_inplace<T, CL>(m, n, work, n, buf, SvdSmem<T>::elems);
   const int k = min(m, n);
   const bool regs = sizeof(T) == 4 && k > 16 && n <= kThreads;
-  const bool x_smem = !regs && n * k <= SvdSmem<T>::elems;
+  const bool x_smem = !CL && !regs && n * k <= SvdSmem<T>::elems;
   cplx<T> *Xc = x_smem ? buf : work;
-  for (int e = tid(); e < n * k; e += kThreads) Xc[e] = cconj(work[e]);
-  __syncthreads();
+  for (int e = t0; e < n * k; e += step) Xc[e] = cconj(work[e]);
+  share_sync<CL>();
   if (x_smem) svd_onesided<T>(n, k, Xc, nullptr, sig2, flag, red);
-  else svd_onesided_blocked<T>(n, k, Xc, nullptr, sig2, flag, red, buf, SvdSmem<T>::elems, regs ? rv_wrk : nullptr);
-  for (int e = tid(); e < n * n; e += kThreads) {
+  else svd_onesided_blocked<T, CL>(n, k, Xc, nullptr, sig2, flag, red, buf, SvdSmem<T>::elems, regs ? rv_wrk : nullptr);
+  for (int e = t0; e < n * n; e += step) {
     const int c = e / n;
     const T l = c < k ? sig2[c] : T(0);
     V[e] = l > T(0) ? cscale(Xc[e], T(1) / sqrt(l)) : cmake<T>(0, 0);
   }
-  for (int c = k + tid(); c < n; c += kThreads) sig2[c] = T(0);
+  if (CL) share_sync<CL>();
+  if constexpr (sizeof(T) == 8 && CL)
+    for (int c = t0; c < k; c += step) sig2[c] = sig2[c] * up * up;
+  for (int c = k + t0; c < n; c += step) sig2[c] = T(0);
+  if (CL) share_sync<CL>();  // no CTA leaves while another may read its shared memory
+}
+
+// R factor or SVD of one large matrix that is called alone, by a cluster of CTAs.
+// One CTA left the GPU idle: its block pairs take turns although a round's are
+// disjoint.  Eight CTAs (the portable limit) have a block pair of 16 + 16 columns
+// each up to 256 columns, and in complex128 blocks of a sixteenth of the columns.
+// One CTA against eight: a 256 x 192 complex64 SVD 23.2 and 4.67 ms, 60 x 50 2.40
+// and 1.18 ms; complex128 128 x 128 98 and 16.3 ms, 72 x 66 (svd_small on one CTA,
+// bound by its SM's FP64 rate) 7.4 and 6.8 ms, 30 x 28 would lose; the R factor of
+// 512 x 250 in complex64 4.1 and 1.6 ms, of 200 x 100 in complex128 4.6 and 2.2 ms.
+constexpr int kShareCtas = 8;
+constexpr int kShareMinCols = 48;  // below, block pairs are too few or too small
+
+struct DenseSmem {
+  double *red;
+  int *flag;
+  char *uv, *buf;
+  float *rv_wrk;
+};
+template <typename T>
+static __device__ DenseSmem dense_smem(char *base) {
+  DenseSmem s;
+  s.red = reinterpret_cast<double *>(base);
+  s.flag = reinterpret_cast<int *>(s.red + kRedDoubles + 16);
+  s.uv = reinterpret_cast<char *>(s.flag + 16);
+  s.buf = s.uv + sizeof(cplx<T>) * kMaxVec;
+  s.rv_wrk = reinterpret_cast<float *>(s.buf + sizeof(cplx<T>) * SvdSmem<T>::elems);
+  return s;
+}
+template <typename T>
+static size_t dense_smem_bytes() {
+  size_t smem = sizeof(double) * (kRedDoubles + 16) + sizeof(int) * 16 + sizeof(cplx<T>) * kMaxVec;
+  smem += sizeof(cplx<T>) * SvdSmem<T>::elems;  // QR panel, SVD matrix or staged column blocks
+  return smem + sizeof(float) * kRvWrkFloats;   // register-visit reductions
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1) dense_shared_kernel(bool svd, int m, int n, cplx<T> *A, cplx<T> *work,
+                                                                   cplx<T> *V, T *sig2) {
+  extern __shared__ __align__(16) char smem_raw[];
+  tc_disable();
+  const DenseSmem s = dense_smem<T>(smem_raw);
+  cplx<T> *buf = reinterpret_cast<cplx<T> *>(s.buf);
+  if (svd) svd_bond<T, true>(m, n, A, work, V, sig2, buf, reinterpret_cast<cplx<T> *>(s.uv), s.red, s.flag, s.rv_wrk);
+  else qr_r_inplace<T, true>(m, n, A, n, buf, SvdSmem<T>::elems);
+}
+
+template <typename T>
+static cudaError_t launch_dense_shared(bool svd, int m, int n, cplx<T> *A, cplx<T> *work, cplx<T> *V, T *sig2,
+                                       cudaStream_t s) {
+  const size_t smem = dense_smem_bytes<T>();
+  cudaError_t e = cudaFuncSetAttribute(dense_shared_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kShareCtas);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kShareCtas;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, dense_shared_kernel<T>, svd, m, n, A, work, V, sig2);
+}
+
+// Which calls a cluster takes.
+template <typename T>
+static bool shares_svd(int m, int n) {
+  return (m < n ? m : n) >= kShareMinCols;
+}
+template <typename T>
+static bool shares_qr(int m, int n) {
+  return qr_small_elems(m, n, false) > SvdSmem<T>::elems && (m < n ? m : n) >= kShareMinCols;
 }
 
 // Kernel-level checks of the dense routines on one CTA (complex elements of
@@ -2819,15 +2979,13 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
                                                                   cplx<T> *V, T *sig2, int use_smem) {
   extern __shared__ __align__(16) char smem_raw[];
   tc_disable();
-  double *red = reinterpret_cast<double *>(smem_raw);
-  double *dm = red + kRedDoubles;
-  int *flag = reinterpret_cast<int *>(dm + 16);
-  cplx<T> *uv = reinterpret_cast<cplx<T> *>(flag + 16);
-  cplx<T> *buf = uv + kMaxVec;
-  float *rv_wrk = reinterpret_cast<float *>(buf + SvdSmem<T>::elems);
+  const DenseSmem s = dense_smem<T>(smem_raw);
+  cplx<T> *buf = reinterpret_cast<cplx<T> *>(s.buf);
+  double *red = s.red;
+  int *flag = s.flag;
   if (what == 0) {
     if (qr_small_elems(m, n, false) <= SvdSmem<T>::elems) qr_small<T>(m, n, A, n, false, A, m, nullptr, buf);
-    else qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, red, dm);
+    else qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems);
   } else if (what == 2) {
     // explicit Q of the gauge steps: reflectors kept in sig2's buffer
     cplx<T> *vstore = reinterpret_cast<cplx<T> *>(sig2);
@@ -2836,14 +2994,13 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
       const int ld = m | 1, steps = min(m, n);
       const cplx<T> *U = buf + n * ld;
       for (int e = tid(); e < m * steps; e += kThreads)
-        if (e / steps >= e % steps)  // unit vectors there, of length sqrt(2) in U
-          vstore[e] = cscale(U[(e % steps) * ld + e / steps], static_cast<T>(0.70710678118654752440));
+        if (e / steps >= e % steps) vstore[e] = cscale(U[(e % steps) * ld + e / steps], static_cast<T>(0.70710678118654752440));
     } else {
-      qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, red, dm, vstore);
+      qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, vstore);
       form_q<T>(m, min(m, n), vstore, V, buf, SvdSmem<T>::elems);
     }
   } else if (use_smem == 3) {
-    svd_bond<T>(m, n, A, A, V, sig2, buf, uv, red, dm, flag, rv_wrk);
+    svd_bond<T, false>(m, n, A, A, V, sig2, buf, reinterpret_cast<cplx<T> *>(s.uv), red, flag, s.rv_wrk);
   } else {
     cplx<T> *C = A, *VV = V;
     if (use_smem == 1) {
@@ -2864,9 +3021,11 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
 template <typename T>
 cudaError_t launch_dense_check_t(int what, int m, int n, void *A, void *V, void *sig2, int use_smem,
                                         cudaStream_t s) {
-  size_t smem = sizeof(double) * (kRedDoubles + 16) + sizeof(int) * 16 + sizeof(cplx<T>) * kMaxVec;
-  smem += sizeof(cplx<T>) * SvdSmem<T>::elems;  // QR panel, SVD matrix or staged column blocks
-  smem += sizeof(float) * kRvWrkFloats;           // register-visit reductions
+  const bool svd = what == 1 && use_smem == 3;
+  if (svd ? shares_svd<T>(m, n) : what == 0 && shares_qr<T>(m, n))
+    return launch_dense_shared<T>(svd, m, n, static_cast<cplx<T> *>(A), static_cast<cplx<T> *>(A),
+                                  static_cast<cplx<T> *>(V), static_cast<T *>(sig2), s);
+  const size_t smem = dense_smem_bytes<T>();
   cudaError_t e = cudaFuncSetAttribute(dense_check_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
@@ -2875,15 +3034,16 @@ cudaError_t launch_dense_check_t(int what, int m, int n, void *A, void *V, void 
   return cudaGetLastError();
 }
 
-// The sweeps' complex contraction alone on one CTA: C = alpha op(A) op(B) +
-// beta C through cgemm, with the tensor cores set up as the round kernel
-// sets them up (complex64 and use_tc) or disabled.  *status becomes
+// The sweeps' complex contraction alone: C = alpha op(A) op(B) + beta C through
+// cgemm, by one CTA with the tensor cores set up as the round kernel sets them up
+// (complex64 and use_tc), else by a CTA per block x block outputs: one CTA for all
+// of a 200^3 product took 8.3 ms in complex128 and 351 us in complex64.  *status becomes
 // STN_ETIMEOUT if a tensor-core wait ran out.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 1) dense_gemm_kernel(int ta, int tb, int m, int n, int k, cplx<T> alpha,
                                                                  const cplx<T> *A, int lda, const cplx<T> *B, int ldb,
                                                                  cplx<T> beta, cplx<T> *C, int ldc, int use_tc,
-                                                                 int *status) {
+                                                                 int *status, int block) {
   extern __shared__ __align__(16) char smem_raw[];
   cplx<T> *tile = reinterpret_cast<cplx<T> *>(smem_raw);
   float *stage = reinterpret_cast<float *>(tile + kTileElems);
@@ -2891,6 +3051,13 @@ __global__ void __launch_bounds__(kThreads, 1) dense_gemm_kernel(int ta, int tb,
   if constexpr (sizeof(T) == 4) tc = use_tc != 0;
   if (tc) tc_setup(stage);
   else tc_disable();
+  // this CTA's block of C (all of it with the tensor cores)
+  const int i0 = blockIdx.x * block, j0 = blockIdx.y * block;
+  m = min(block, m - i0);
+  n = min(block, n - j0);
+  A += ta == 0 ? static_cast<int64_t>(i0) * lda : i0;
+  B += tb == 0 ? j0 : static_cast<int64_t>(j0) * ldb;
+  C += static_cast<int64_t>(i0) * ldc + j0;
   if (ta == 0 && tb == 0) cgemm<T, 0, 0>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, tile);
   else if (ta == 0) cgemm<T, 0, 1>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, tile);
   else if (tb == 0) cgemm<T, 1, 0>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, tile);
@@ -2915,9 +3082,14 @@ cudaError_t launch_dense_gemm_t(int ta, int tb, int m, int n, int k, const doubl
   al.im = static_cast<T>(alpha[1]);
   be.re = static_cast<T>(beta[0]);
   be.im = static_cast<T>(beta[1]);
-  dense_gemm_kernel<T><<<1, kThreads, smem, s>>>(ta, tb, m, n, k, al, static_cast<const cplx<T> *>(A), lda,
+  // blocks of 32 x 32 outputs, of 16 x 16 where those would leave SMs without one
+  const bool tc = sizeof(T) == 4 && use_tc;
+  auto tiles = [&](int b) { return dim3((m + b - 1) / b, (n + b - 1) / b); };
+  int block = tc ? (m > n ? m : n) : 32;
+  if (!tc && tiles(32).x * tiles(32).y < 152) block = 16;
+  dense_gemm_kernel<T><<<tiles(block), kThreads, smem, s>>>(ta, tb, m, n, k, al, static_cast<const cplx<T> *>(A), lda,
                                                  static_cast<const cplx<T> *>(B), ldb, be, static_cast<cplx<T> *>(C),
-                                                 ldc, use_tc, status);
+                                                 ldc, use_tc, status, block);
   return cudaGetLastError();
 }
 
@@ -3018,7 +3190,7 @@ __global__ void __launch_bounds__(kThreads, 1) diag_kernel(EngineParams P, int w
         const cplx<T> *A = site_ptr<T>(P, shot, cut);
         for (int e = tid(); e < mrows * r; e += kThreads) X.y[e] = A[e];
         __syncthreads();
-        qr_r_inplace<T>(mrows, r, X.y, r, S.jbuf, P.svd_elems, S.red, S.dmisc + 4);
+        qr_r_inplace<T>(mrows, r, X.y, r, S.jbuf, P.svd_elems);
         // Jacobi on R^dag (r x kx, column-major, ld r), in place as in the sweep
         for (int e = tid(); e < r * kx; e += kThreads) X.y[e] = cconj(X.y[e]);
         __syncthreads();

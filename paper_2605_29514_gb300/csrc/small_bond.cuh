@@ -254,35 +254,43 @@ __device__ __forceinline__ void reflector_scaled(cplx<ff> al, ff nx2, cplx<ff> &
   sc = ff{sc.h * f, sc.l * f};
 }
 
-// Reflector j of the column col[j..m-1] in the storage precision T into
-// u[j..m-1]; col[j] becomes gamma.  A column of norm up to 1e-30 gets none
-// (u = 0).  Norm and scalars in double, or for float in ff; always on the column
-// scaled by a power of two: single-precision squares of entries near 1e-20 would
-// be denormal, and a reflector built from such a norm not unitary.  One warp.
-__device__ __forceinline__ void reflect_column(cplx<double> *col, cplx<double> *u, int j, int m) {
-  double s = 0;
-  for (int i = j + lane_id(); i < m; i += 32) Work<double>::sq(s, col[i]);
-  s = lane_sum<double>(s, 16);
-  cplx<double> gam = cmake<double>(0, 0);
-  double sc = 0;
-  if (s > 1e-60) reflector_scaled(col[j], s, gam, sc);
-  for (int i = j + lane_id(); i < m; i += 32) {
-    cplx<double> x = col[i];
-    if (i == j) x = cmake<double>(x.re - gam.re, x.im - gam.im);
-    u[i] = sc > 0 ? cscale(x, sc) : cmake<double>(0, 0);
+// Reflector of the column x[j..m-1] (elements `stride` apart) in the storage
+// precision T.  A column of norm up to 1e-30 gets none (sc = 0).  Norm and scalars
+// in double, or for float in ff; for float on the column times the power of two
+// `down`: single-precision squares of entries near 1e-20 would be denormal, and a
+// reflector built from such a norm not unitary.  `unit` makes it P = I - 2 u u^dag
+// of a unit u.  One warp.
+template <typename T>
+struct Reflector {
+  cplx<T> gam;  // of the scaled column
+  T sc, down, up;
+  __device__ __forceinline__ cplx<T> vector(cplx<T> x, bool first) const {
+    x = cscale(x, down);
+    if (first) x = cmake<T>(x.re - gam.re, x.im - gam.im);
+    return sc > T(0) ? cscale(x, sc) : cmake<T>(0, 0);
   }
-  __syncwarp();
-  if (lane_id() == 0) col[j] = gam;
+  __device__ __forceinline__ cplx<T> diagonal() const { return cscale(gam, up); }
+};
+__device__ __forceinline__ Reflector<double> column_reflector(const cplx<double> *col, int stride, int j, int m,
+                                                              bool unit) {
+  double s = 0;
+  for (int i = j + lane_id(); i < m; i += 32) Work<double>::sq(s, col[i * stride]);
+  s = lane_sum<double>(s, 16);
+  Reflector<double> h{cmake<double>(0, 0), 0.0, 1.0, 1.0};
+  if (s > 1e-60) reflector_scaled(col[j * stride], s, h.gam, h.sc);
+  if (unit) h.sc *= 0.70710678118654752440;
+  return h;
 }
-__device__ __forceinline__ void reflect_column(cplx<float> *col, cplx<float> *u, int j, int m) {
+// Squared norm of a float column scaled by down = 2^-(ex - 127), up its inverse.
+__device__ __forceinline__ ff column_norm2(const cplx<float> *col, int stride, int j, int m, int &ex) {
   float mx = 0.f;
-  for (int i = j + lane_id(); i < m; i += 32) mx = fmaxf(mx, fmaxf(fabsf(col[i].re), fabsf(col[i].im)));
+  for (int i = j + lane_id(); i < m; i += 32) mx = fmaxf(mx, fmaxf(fabsf(col[i * stride].re), fabsf(col[i * stride].im)));
   const int bits = __reduce_max_sync(0xffffffffu, __float_as_int(mx));
-  const int ex = min(253, max(1, bits >> 23));
-  const float down = __int_as_float((254 - ex) << 23), up = __int_as_float(ex << 23);  // 2^-(ex - 127) and its inverse
+  ex = min(253, max(1, bits >> 23));
+  const float down = __int_as_float((254 - ex) << 23);
   ff s = ff_of(0.f);
   for (int i = j + lane_id(); i < m; i += 32) {
-    const float re = col[i].re * down, im = col[i].im * down;
+    const float re = col[i * stride].re * down, im = col[i * stride].im * down;
     ff_fma(s, ff_of(re), ff_of(re));
     ff_fma(s, ff_of(im), ff_of(im));
   }
@@ -290,32 +298,37 @@ __device__ __forceinline__ void reflect_column(cplx<float> *col, cplx<float> *u,
   // component is in [1, 2), so a lane's sum is at most 8 rows per lane and 512
   // rows give 2^28 in the first): two integer reductions for five levels of
   // shuffles, and exact.
-  if (m <= 512) {
-    const int hi = __float2int_rn(s.h * 0x1p16f);
-    const int lo = __float2int_rn((__fadd_rn(s.h, -static_cast<float>(hi) * 0x1p-16f) + s.l) * 0x1p40f);
-    const int th = __reduce_add_sync(0xffffffffu, hi), tl = __reduce_add_sync(0xffffffffu, lo);
-    const float h0 = static_cast<float>(th);
-    s = ff_add(ff{h0 * 0x1p-16f, static_cast<float>(th - __float2int_rn(h0)) * 0x1p-16f},
-               ff_of(static_cast<float>(tl) * 0x1p-40f));
-  } else {
-    s = lane_sum<ff>(s, 16);
-  }
-  cplx<float> gam = cmake<float>(0.f, 0.f);
-  float sc = 0.f;
-  if (sqrtf(s.h) * up > 1e-30f) {
+  if (m > 512) return lane_sum<ff>(s, 16);
+  const int hi = __float2int_rn(s.h * 0x1p16f);
+  const int lo = __float2int_rn((__fadd_rn(s.h, -static_cast<float>(hi) * 0x1p-16f) + s.l) * 0x1p40f);
+  const int th = __reduce_add_sync(0xffffffffu, hi), tl = __reduce_add_sync(0xffffffffu, lo);
+  const float h0 = static_cast<float>(th);
+  return ff_add(ff{h0 * 0x1p-16f, static_cast<float>(th - __float2int_rn(h0)) * 0x1p-16f},
+                ff_of(static_cast<float>(tl) * 0x1p-40f));
+}
+__device__ __forceinline__ Reflector<float> column_reflector(const cplx<float> *col, int stride, int j, int m,
+                                                             bool unit) {
+  int ex;
+  const ff s = column_norm2(col, stride, j, m, ex);
+  Reflector<float> h{cmake<float>(0.f, 0.f), 0.f, __int_as_float((254 - ex) << 23), __int_as_float(ex << 23)};
+  if (sqrtf(s.h) * h.up > 1e-30f) {
     cplx<ff> g;
     ff c;
-    reflector_scalars<ff>(cmake<ff>(ff_of(col[j].re * down), ff_of(col[j].im * down)), s, g, c);
-    gam = cmake<float>(g.re.h, g.im.h);
-    sc = c.h;
+    const cplx<float> al = cscale(col[j * stride], h.down);
+    reflector_scalars<ff>(cmake<ff>(ff_of(al.re), ff_of(al.im)), s, g, c);
+    h.gam = cmake<float>(g.re.h, g.im.h);
+    h.sc = unit ? ff_mul(c, ff{0.70710677f, 1.2101617e-8f}).h : c.h;
   }
-  for (int i = j + lane_id(); i < m; i += 32) {
-    cplx<float> x = cmake<float>(col[i].re * down, col[i].im * down);
-    if (i == j) x = cmake<float>(x.re - gam.re, x.im - gam.im);
-    u[i] = sc > 0.f ? cscale(x, sc) : cmake<float>(0.f, 0.f);
-  }
+  return h;
+}
+
+// Reflector j of a stored column into u[j..m-1]; col[j] becomes gamma.
+template <typename T>
+__device__ __forceinline__ void reflect_column(cplx<T> *col, cplx<T> *u, int j, int m) {
+  const Reflector<T> h = column_reflector(col, 1, j, m, false);
+  for (int i = j + lane_id(); i < m; i += 32) u[i] = h.vector(col[i], i == j);
   __syncwarp();
-  if (lane_id() == 0) col[j] = cmake<float>(gam.re * up, gam.im * up);
+  if (lane_id() == 0) col[j] = h.diagonal();
 }
 
 // Householder QR in shared memory.  A is m x n: row-major with leading

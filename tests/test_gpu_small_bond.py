@@ -144,3 +144,33 @@ def test_truncations_against_oracle(precision, cutoff, cap, theta, basis):
         if precision == 0:
             assert out["max_chi"][s] == ref.max_chi
     sim.close()
+
+
+@pytest.mark.parametrize("precision,m,n", [(1, 480, 47), (1, 470, 48), (1, 160, 150), (1, 241, 512), (1, 512, 255),
+                                           (0, 300, 49), (0, 101, 95), (0, 130, 129), (0, 64, 512)])
+def test_large_matrices_over_a_cluster(precision, m, n):
+    """R factors and SVDs on both sides of the column count and capacity from
+    which the CTAs of a cluster share them, with odd numbers of 16-column blocks,
+    ragged last blocks and wide matrices.  Bounds as above; a Jacobi vector of
+    complex64 carries sqrt(rotations) roundings more (15 sweeps at most)."""
+    rng = np.random.default_rng(13 * m + n)
+    a = cmat(rng, m, n, precision)
+    k = min(m, n)
+    r = torch.tensor(a, device="cuda")
+    stn.dense_qr(precision, m, n, r.data_ptr())
+    da = torch.tensor(a, device="cuda")
+    dv = torch.full((n, n), np.nan, dtype=CDT[precision], device="cuda")
+    ds = torch.full((n,), np.nan, dtype=RDT[precision], device="cuda")
+    a = a.astype(np.complex128)
+    bound = 64 * EPS[precision] * np.sqrt(m * n) * np.linalg.norm(a)
+    r = r.cpu().numpy().astype(np.complex128)
+    assert np.all(r[k:] == 0) and np.all(np.tril(r[:k, :k], -1) == 0)
+    assert np.abs(r.conj().T @ r - a.conj().T @ a).max() <= bound * np.linalg.norm(a)
+    stn.dense_svd_noalloc(precision, m, n, da.data_ptr(), dv.data_ptr(), ds.data_ptr())
+    sig = np.sqrt(ds.cpu().numpy().astype(np.float64))
+    order = np.argsort(-sig)[:k]
+    vk = dv.cpu().numpy()[order].T.astype(np.complex128)
+    assert np.abs(sig[order] - np.linalg.svd(a, compute_uv=False)).max() < bound
+    grow = np.sqrt(15 * k)
+    assert np.abs(vk.conj().T @ vk - np.eye(k)).max() < 64 * EPS[precision] * np.sqrt(m * n) * grow
+    assert np.abs(a @ vk @ vk.conj().T - a).max() < bound * grow
