@@ -2992,9 +2992,11 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
     if (qr_small_elems(m, n, true) <= SvdSmem<T>::elems) {
       qr_small<T>(m, n, A, n, false, A, m, V, buf);
       const int ld = m | 1, steps = min(m, n);
-      const cplx<T> *U = buf + n * ld;
-      for (int e = tid(); e < m * steps; e += kThreads)
-        if (e / steps >= e % steps) vstore[e] = cscale(U[(e % steps) * ld + e / steps], static_cast<T>(0.70710678118654752440));
+      const ColumnHead<T> *head = reinterpret_cast<const ColumnHead<T> *>(buf + n * ld);
+      for (int e = tid(); e < m * steps; e += kThreads) {  // unit vectors there, v with beta here
+        const int i = e / steps, c = e % steps;
+        if (i >= c) vstore[e] = cscale(i == c ? head[c].v0 : buf[c * ld + i], sqrt(head[c].beta * T(0.5)));
+      }
     } else {
       qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems, vstore);
       form_q<T>(m, min(m, n), vstore, V, buf, SvdSmem<T>::elems);
