@@ -1761,12 +1761,15 @@ enum { M_LO = 0, M_HI, M_A, M_B, M_CENTER, M_FAIL, M_KEEP, M_MAXCHI, M_CASEB, M_
 // dmisc slots
 enum { D_DISC = 0, D_LOGP, D_E, D_NORM, D_FLOPS = 8, D_PROF = 8 };  // D_PROF + 1 + ProfSlot
 
+// The slots from D_FLOPS on hold integers.
+__device__ __forceinline__ long long &tally(double *dmisc, int slot) { return reinterpret_cast<long long *>(dmisc)[slot]; }
+
 // Adds the cycles since `t` to a phase slot and restarts `t` (thread 0 only;
 // callers sit just after a CTA barrier so the CTA is in step).
 __device__ __forceinline__ void prof_mark(double *dmisc, int slot, long long &t) {
   if (threadIdx.x == 0) {
     const long long now = clock64();
-    dmisc[D_PROF + 1 + slot] += static_cast<double>(now - t);
+    tally(dmisc, D_PROF + 1 + slot) += now - t;
     t = now;
   }
 }
@@ -1804,14 +1807,16 @@ static __device__ Scratch<T> scratch_for(const EngineParams &P, int cap) {
 // factor of an m x n matrix 4 (2 m n^2 - 2 n^3 / 3) with m >= n, the
 // singular values and the vectors of the smaller side of an m x n matrix
 // 4 (4 m n^2 + 8 n^3) with m >= n (roles swapped otherwise in both).
-static __device__ __forceinline__ double gemm_flops(int M, int N, int K) { return 8.0 * M * N * K; }
-static __device__ __forceinline__ double qr_flops(int m, int n) {
-  double a = m >= n ? m : n, b = m >= n ? n : m;
-  return 4.0 * (2.0 * a * b * b - 2.0 * b * b * b / 3.0);
+// In thirds of a flop: thread 0 counts in integers, since a double-precision
+// operation takes 64 cycles and these were 40 a bond, of about 70,000 cycles.
+static __device__ __forceinline__ long long gemm_flops(int M, int N, int K) { return 24ll * M * N * K; }
+static __device__ __forceinline__ long long qr_flops(int m, int n) {
+  const long long a = max(m, n), b = min(m, n);
+  return (24 * a - 8 * b) * b * b;
 }
-static __device__ __forceinline__ double svd_flops(int m, int n) {
-  double a = m >= n ? m : n, b = m >= n ? n : m;
-  return 4.0 * (4.0 * a * b * b + 8.0 * b * b * b);
+static __device__ __forceinline__ long long svd_flops(int m, int n) {
+  const long long a = max(m, n), b = min(m, n);
+  return (48 * a + 96 * b) * b * b;
 }
 
 // ---------------------------------------------------------------------------
@@ -1877,56 +1882,6 @@ static __device__ __noinline__ void materialize(const MpoSpec<T> &sp, const uint
   }
 }
 
-// Keep count at one bond from its eigenvalues lam (>= 0) in the decreasing order
-// perm, by one warp.  The cutoff is compared in squares, lam_i > cutoff^2 lam_1:
-// square roots (of double, by one thread) were most of the 11,000 cycles the
-// keep decision of a bond took.
-template <typename T>
-static __device__ int keep_count(const T *lam, const int *perm, int n, int cap, double cutoff, double delta) {
-  auto at = [&](int i) { return static_cast<double>(lam[perm[i]]); };
-  auto above = [&](int m, double thr2) {
-    int k = 0;
-    for (int i = 0; i < m; i += 32)
-      k += __popc(__ballot_sync(0xffffffffu, i + lane_id() < m && at(min(i + lane_id(), m - 1)) > thr2));
-    return k;
-  };
-  const double l1 = at(0);
-  if (!(l1 > 0.0)) return 1;
-  int k = max(1, above(n, cutoff * cutoff * l1));
-  if (k > cap) {
-    const double thr = sqrt(at(cap)) + delta * sqrt(l1);
-    k = max(1, above(cap, thr * thr));
-  }
-  return k;
-}
-
-// Discarded over total weight of a bond, by one warp (lane 0's value counts).
-static __device__ __forceinline__ double discarded_weight(const double *lam, const int *perm, int n, int keep) {
-  double tot = 0, drop = 0;
-  for (int i = lane_id(); i < n; i += 32) {
-    const double l = lam[perm[i]];
-    tot += l;
-    if (i >= keep) drop += l;
-  }
-  tot = warp_sum(tot);
-  drop = warp_sum(drop);
-  return tot > 0 ? drop / tot : 0.0;
-}
-static __device__ __forceinline__ double discarded_weight(const float *lam, const int *perm, int n, int keep) {
-  ff tot = ff_of(0.f), drop = ff_of(0.f);
-  for (int i = lane_id(); i < n; i += 32) {
-    const float l = lam[perm[i]];
-    ff_push(tot, l, 0.f);
-    if (i >= keep) ff_push(drop, l, 0.f);
-  }
-  tot = lane_sum<ff>(tot, 16);
-  drop = lane_sum<ff>(drop, 16);
-  if (!(tot.h > 0.f)) return 0.0;
-  const float q = drop.h / tot.h;
-  ff_fma(drop, ff_of(-q), tot);  // the remainder: a second quotient digit of single precision
-  return static_cast<double>(q) + static_cast<double>((drop.h + drop.l) / tot.h);
-}
-
 // Exact gauge steps (no truncation) moving the orthogonality centre of a
 // shot's MPS from its current site to `target`, so that the sites left of an
 // operator's support are left-canonical and those right of it
@@ -1965,8 +1920,8 @@ static __device__ __noinline__ void mps_move_center(const EngineParams &P, const
     for (int e = tid(); e < steps * 2 * r2; e += kThreads) Bn[e] = X.w[e];
     if (tid() == 0) {
       chi[c + 1] = steps;
-      S.dmisc[D_FLOPS] += 2.0 * qr_flops(m, r) + gemm_flops(steps, 2 * r2, r);
-      S.dmisc[D_PROF + 1 + PROF_NGAUGE] += 1.0;
+      tally(S.dmisc, D_FLOPS) += 2 * qr_flops(m, r) + gemm_flops(steps, 2 * r2, r);
+      tally(S.dmisc, D_PROF + 1 + PROF_NGAUGE) += 1;
     }
     __syncthreads();
     ++c;
@@ -2000,8 +1955,8 @@ static __device__ __noinline__ void mps_move_center(const EngineParams &P, const
     for (int e = tid(); e < 2 * ll * steps; e += kThreads) Am[e] = X.w[e];
     if (tid() == 0) {
       chi[c] = steps;
-      S.dmisc[D_FLOPS] += 2.0 * qr_flops(m, l) + gemm_flops(2 * ll, steps, l);
-      S.dmisc[D_PROF + 1 + PROF_NGAUGE] += 1.0;
+      tally(S.dmisc, D_FLOPS) += 2 * qr_flops(m, l) + gemm_flops(2 * ll, steps, l);
+      tally(S.dmisc, D_PROF + 1 + PROF_NGAUGE) += 1;
     }
     __syncthreads();
     --c;
@@ -2086,7 +2041,7 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
       const int r = S.rdim[k - a];
       const cplx<T> *Rk = X.g + S.goff[k - a];
       cgemm<T, 0, 0>(r, 2 * Dr, Dl, one, Rk, Dl, Ak, 2 * Dr, zero, X.t, 2 * Dr, S.tile);
-      if (tid() == 0) S.dmisc[D_FLOPS] += gemm_flops(r, 2 * Dr, Dl);
+      if (tid() == 0) tally(S.dmisc, D_FLOPS) += gemm_flops(r, 2 * Dr, Dl);
       m = 2 * r;
     }
     if (m > kMaxVec) {
@@ -2094,7 +2049,7 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
       __syncthreads();
       return 0.0;
     }
-    if (tid() == 0) S.dmisc[D_FLOPS] += qr_flops(m, Dr);
+    if (tid() == 0) tally(S.dmisc, D_FLOPS) += qr_flops(m, Dr);
     const int rn = min(m, Dr);
     cplx<T> *Rout = X.g + S.goff[k + 1 - a];
     if (qr_small_elems(m, Dr, false) <= P.svd_elems) {
@@ -2169,15 +2124,18 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
     // every sweep.  In complex128, every bond of up to
     // kSmallSvdCols columns takes this path.
     bool vec_from_columns = false;
+    int keep = 0;
+    cplx<T> *Bk = site_ptr<T>(P, shot, k);
+    const int kmax = min(cap, P.chimax[k]);
     const int dscale = static_cast<int>(sizeof(double) / sizeof(T));
     const bool svd64 = n2 <= kSmallSvdCols && r <= kMaxVec && (sizeof(T) == 8 || 2 * (r * n2 + n2 * n2) <= P.svd_rule);
     if (svd64) {
       const int elems = n2 * (r | 1) * dscale;
-      if (elems + r * dscale <= P.svd_elems)
-        svd_small<T, true>(r, n2, X.y, X.v, X.lam, P.cutoff, S.jbuf, S.jbuf + elems, S.red);
+      const Truncation<T> tr{S.perm, kmax, P.delta, &S.misc[M_FAIL], &S.misc[M_KEEP], &S.dmisc[D_DISC], X.vs, Bk};
+      if (elems + 3 * dscale <= P.svd_elems)
+        keep = svd_small<T, true>(r, n2, X.y, nullptr, S.lam, P.cutoff, S.jbuf, S.jbuf + elems, S.red, &tr);
       else  // X.t is free in the right sweep and holds it: r n2 <= 4 c^2 numbers of 16 bytes
-        svd_small<T, false>(r, n2, X.y, X.v, X.lam, P.cutoff, X.t, S.jbuf, S.red);
-      Vc = X.v;
+        keep = svd_small<T, false>(r, n2, X.y, nullptr, S.lam, P.cutoff, X.t, S.jbuf, S.red, &tr);
     } else if (sizeof(T) == 4 && P.svd64_all) {
       // Complex64 contractions with every SVD in double precision: the large
       // path (Householder R factor, Jacobi on R^dag) on a complex128 copy of
@@ -2197,7 +2155,7 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       __syncthreads();
       const long long tqr = clock64();
       qr_r_inplace<double>(r, n2, Cd, n2, jd, P.svd_elems / 2);
-      if (tid() == 0) S.dmisc[D_PROF + 1 + PROF_SVD_QR] += static_cast<double>(clock64() - tqr);
+      if (tid() == 0) tally(S.dmisc, D_PROF + 1 + PROF_SVD_QR) += clock64() - tqr;
       const int kx = min(r, n2);
       for (int e = tid(); e < n2 * kx; e += kThreads) Cd[e] = cconj(Cd[e]);
       __syncthreads();
@@ -2205,10 +2163,10 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       const int sweeps = svd_onesided_blocked<double>(n2, kx, Cd, nullptr, sd, &S.misc[M_JFLAG], S.red, jd,
                                                       P.svd_elems / 2);
       if (tid() == 0) {
-        S.dmisc[D_PROF + 1 + PROF_JSWEEPS] += sweeps;
-        S.dmisc[D_PROF + 1 + PROF_JROWS] += n2;
-        S.dmisc[D_PROF + 1 + PROF_JCOLS] += kx;
-        if (n2 <= kThreads / 2) S.dmisc[D_PROF + 1 + PROF_JAC_ROWS256] += static_cast<double>(clock64() - tj);
+        tally(S.dmisc, D_PROF + 1 + PROF_JSWEEPS) += sweeps;
+        tally(S.dmisc, D_PROF + 1 + PROF_JROWS) += n2;
+        tally(S.dmisc, D_PROF + 1 + PROF_JCOLS) += kx;
+        if (n2 <= kThreads / 2) tally(S.dmisc, D_PROF + 1 + PROF_JAC_ROWS256) += clock64() - tj;
       }
       for (int e = tid(); e < n2 * kx; e += kThreads)
         X.y[e] = cmake<T>(static_cast<T>(Cd[e].re), static_cast<T>(Cd[e].im));
@@ -2238,7 +2196,7 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       }
       const long long tqr = clock64();
       qr_r_inplace<T>(r, n2, X.y, n2, S.jbuf, P.svd_elems);
-      if (tid() == 0) S.dmisc[D_PROF + 1 + PROF_SVD_QR] += static_cast<double>(clock64() - tqr);
+      if (tid() == 0) tally(S.dmisc, D_PROF + 1 + PROF_SVD_QR) += clock64() - tqr;
       const int kx = min(r, n2);
       // complex64 with more than one block of 16 columns: blocked Jacobi
       // with register-resident block pairs, X in global scratch (L2)
@@ -2253,10 +2211,10 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
                  : svd_onesided_blocked<T>(n2, kx, Xc, nullptr, X.lam, &S.misc[M_JFLAG], S.red, S.jbuf,
                                            P.svd_elems, regs ? reinterpret_cast<float *>(S.lam) : nullptr);
       if (tid() == 0) {
-        S.dmisc[D_PROF + 1 + PROF_JSWEEPS] += sweeps;
-        S.dmisc[D_PROF + 1 + PROF_JROWS] += n2;
-        S.dmisc[D_PROF + 1 + PROF_JCOLS] += kx;
-        if (n2 <= kThreads / 2) S.dmisc[D_PROF + 1 + PROF_JAC_ROWS256] += static_cast<double>(clock64() - tj);
+        tally(S.dmisc, D_PROF + 1 + PROF_JSWEEPS) += sweeps;
+        tally(S.dmisc, D_PROF + 1 + PROF_JROWS) += n2;
+        tally(S.dmisc, D_PROF + 1 + PROF_JCOLS) += kx;
+        if (n2 <= kThreads / 2) tally(S.dmisc, D_PROF + 1 + PROF_JAC_ROWS256) += clock64() - tj;
       }
       for (int i = kx + tid(); i < n2; i += kThreads) X.lam[i] = T(0);
       __syncthreads();
@@ -2264,51 +2222,52 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       vec_from_columns = true;
     }
     __syncthreads();
-    if (tid() == 0 && !vec_from_columns) S.dmisc[D_PROF + 1 + PROF_SVD_SMALL] += static_cast<double>(clock64() - tp);
+    if (tid() == 0 && !vec_from_columns) tally(S.dmisc, D_PROF + 1 + PROF_SVD_SMALL) += clock64() - tp;
     prof_mark(S.dmisc, PROF_SVD, tp);
     if (tid() == 0) {
-      S.dmisc[D_FLOPS] += gemm_flops(r, n2, Dl) + svd_flops(r, n2);
-      S.dmisc[D_PROF + 1 + (vec_from_columns ? PROF_NSVD_LARGE : PROF_NSVD_SMALL)] += 1.0;
+      tally(S.dmisc, D_FLOPS) += gemm_flops(r, n2, Dl) + svd_flops(r, n2);
+      tally(S.dmisc, D_PROF + 1 + (vec_from_columns ? PROF_NSVD_LARGE : PROF_NSVD_SMALL)) += 1;
     }
-    // S.lam holds the squared values, S.perm their order
-    for (int i = tid(); i < n2; i += kThreads) {
-      const T l = X.lam[i];
-      const bool bad = !isfinite(l);
-      if (bad) S.misc[M_FAIL] = STN_ENUMERIC;
-      S.lam[i] = bad ? T(0) : l;
-    }
-    __syncthreads();
     if (S.misc[M_FAIL]) return;
-    sort_desc<T>(n2, S.lam, S.perm);
-    if (warp_id() == 0) {
-      const int kmax = min(cap, P.chimax[k]);
-      const int keep = min(keep_count<T>(S.lam, S.perm, n2, kmax, P.cutoff, P.delta), kmax);
-      if (tid() == 0) S.misc[M_KEEP] = keep;
-    }
-    __syncthreads();
-    const int keep = S.misc[M_KEEP];
-    if (warp_id() == kWarps - 1) {  // the others go on meanwhile
-      const double w = discarded_weight(S.lam, S.perm, n2, keep);
-      if (lane_id() == 0) S.dmisc[D_DISC] += w;
-    }
-    // sorted, kept right singular vectors: Vs[:, c] = V[:, perm[c]], c < keep
-    // (or the rotated column of X over its norm), and the new right-canonical
-    // site k: B[c][s][r] = conj(Vs[(s*kappa + r)][c]).  Vectors rounded from pairs
-    // of floats to float are orthonormal to rounding; the others take one
-    // Newton-Schulz step in between.
-    cplx<T> *Bk = site_ptr<T>(P, shot, k);
     const bool orthonormal = sizeof(T) == 4 && svd64;
-    for (int e = tid(); e < n2 * keep; e += kThreads) {
-      int i = e / keep, c = e % keep;
-      cplx<T> v = Vc[static_cast<int64_t>(S.perm[c]) * n2 + i];
-      if (vec_from_columns) {
-        T l = S.lam[S.perm[c]];
-        v = l > T(0) ? cscale(v, T(1) / sqrt(l)) : cmake<T>(i == c ? T(1) : T(0), 0);
+    if (!svd64) {
+      // S.lam holds the squared values, S.perm their order
+      for (int i = tid(); i < n2; i += kThreads) {
+        const T l = X.lam[i];
+        const bool bad = !isfinite(l);
+        if (bad) S.misc[M_FAIL] = STN_ENUMERIC;
+        S.lam[i] = bad ? T(0) : l;
       }
-      X.vs[i * keep + c] = v;
-      if (orthonormal) Bk[c * n2 + i] = cconj(v);
+      __syncthreads();
+      if (S.misc[M_FAIL]) return;
+      sort_desc<T>(n2, S.lam, S.perm);
+      if (warp_id() == 0) {
+        const int count = min(keep_count<T>(S.lam, S.perm, n2, kmax, P.cutoff, P.delta), kmax);
+        if (tid() == 0) S.misc[M_KEEP] = count;
+      }
+      __syncthreads();
+      keep = S.misc[M_KEEP];
+      if (warp_id() == kWarps - 1) {  // the others go on meanwhile
+        const double w = discarded_weight(S.lam, S.perm, n2, keep);
+        if (lane_id() == 0) S.dmisc[D_DISC] += w;
+      }
+      // sorted, kept right singular vectors: Vs[:, c] = V[:, perm[c]], c < keep
+      // (or the rotated column of X over its norm)
+      for (int e = tid(); e < n2 * keep; e += kThreads) {
+        int i = e / keep, c = e % keep;
+        cplx<T> v = Vc[static_cast<int64_t>(S.perm[c]) * n2 + i];
+        if (vec_from_columns) {
+          T l = S.lam[S.perm[c]];
+          v = l > T(0) ? cscale(v, T(1) / sqrt(l)) : cmake<T>(i == c ? T(1) : T(0), 0);
+        }
+        X.vs[i * keep + c] = v;
+      }
+      __syncthreads();
     }
-    __syncthreads();
+    // and the new right-canonical site k: B[c][s][r] = conj(Vs[(s*kappa + r)][c]).
+    // Vectors rounded from pairs of floats to float are orthonormal to rounding
+    // (svd_small has stored that site); the others take one Newton-Schulz step
+    // before.
     if (!orthonormal) {
       reorthonormalize<T>(n2, keep, X.vs, X.e, X.y, S.tile);
       for (int e = tid(); e < keep * n2; e += kThreads) {
@@ -2324,7 +2283,7 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
     cgemm<T, 0, 0>(2 * Dll, keep, Dl, one, Akm1, Dl, X.w, keep, zero, X.mbuf, keep, S.tile);
     if (tid() == 0) {
       chi[k] = keep;
-      S.dmisc[D_FLOPS] += gemm_flops(Dl, keep, n2) + gemm_flops(2 * Dll, keep, Dl);
+      tally(S.dmisc, D_FLOPS) += gemm_flops(Dl, keep, n2) + gemm_flops(2 * Dll, keep, Dl);
     }
     __syncthreads();
     M = X.mbuf;
@@ -2377,11 +2336,11 @@ static __device__ __noinline__ double mps_expect(const EngineParams &P, const Sm
     __syncthreads();
     if (k == a) {
       cgemm<T, 1, 0>(cr, cr, 2 * cl, one, A, cr, X.sa, cr, zero, X.e, cr, S.tile);
-      if (tid() == 0) S.dmisc[D_FLOPS] += gemm_flops(cr, cr, 2 * cl);
+      if (tid() == 0) tally(S.dmisc, D_FLOPS) += gemm_flops(cr, cr, 2 * cl);
     } else {
       cgemm<T, 0, 0>(cl, 2 * cr, cl, one, X.e, cl, X.sa, 2 * cr, zero, X.te, 2 * cr, S.tile);
       cgemm<T, 1, 0>(cr, cr, 2 * cl, one, A, cr, X.te, cr, zero, X.e, cr, S.tile);
-      if (tid() == 0) S.dmisc[D_FLOPS] += gemm_flops(cl, 2 * cr, cl) + gemm_flops(cr, cr, 2 * cl);
+      if (tid() == 0) tally(S.dmisc, D_FLOPS) += gemm_flops(cl, 2 * cr, cl) + gemm_flops(cr, cr, 2 * cl);
     }
   }
   const int cb = chi[b + 1];
@@ -2567,8 +2526,8 @@ __global__ void __launch_bounds__(kThreads, B) round_kernel(EngineParams P) {
       S.misc[M_MAXCHI] = P.maxchi[shot];
       S.dmisc[D_DISC] = P.disc[shot];
       S.dmisc[D_LOGP] = P.logp[shot];
-      S.dmisc[D_FLOPS] = 0.0;
-      for (int i = 0; i < kProfSlots; ++i) S.dmisc[D_PROF + 1 + i] = 0.0;
+      tally(S.dmisc, D_FLOPS) = 0;
+      for (int i = 0; i < kProfSlots; ++i) tally(S.dmisc, D_PROF + 1 + i) = 0;
     }
     __syncthreads();
     long long t_ops = clock64();
@@ -2789,9 +2748,10 @@ __global__ void __launch_bounds__(kThreads, B) round_kernel(EngineParams P) {
       P.maxchi[shot] = S.misc[M_MAXCHI];
       P.disc[shot] = S.dmisc[D_DISC];
       P.logp[shot] = S.dmisc[D_LOGP];
-      P.flops[shot] += S.dmisc[D_FLOPS];
-      S.dmisc[D_PROF + 1 + PROF_OPS] = static_cast<double>(clock64() - t_ops);
-      for (int i = 0; i < kProfSlots; ++i) P.prof[shot * kProfSlots + i] += S.dmisc[D_PROF + 1 + i];
+      P.flops[shot] += static_cast<double>(tally(S.dmisc, D_FLOPS)) / 3.0;
+      tally(S.dmisc, D_PROF + 1 + PROF_OPS) = clock64() - t_ops;
+      for (int i = 0; i < kProfSlots; ++i)
+        P.prof[shot * kProfSlots + i] += static_cast<double>(tally(S.dmisc, D_PROF + 1 + i));
       if (S.misc[M_FAIL]) atomicCAS(P.err, 0, S.misc[M_FAIL]);
     }
     __syncthreads();
@@ -3287,7 +3247,7 @@ __global__ void __launch_bounds__(kThreads, kLight ? 2 : 1) adjoint_kernel(Engin
       S.misc[M_FAIL] = P.status[shot];
       S.misc[M_MAXCHI] = P.maxchi[shot];
       S.dmisc[D_DISC] = 0.0;
-      S.dmisc[D_FLOPS] = 0.0;
+      tally(S.dmisc, D_FLOPS) = 0;
     }
     __syncthreads();
     for (int oi = P.n_ops_total - 1; oi >= 0 && !S.misc[M_FAIL]; --oi) {

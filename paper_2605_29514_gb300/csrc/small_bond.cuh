@@ -99,10 +99,9 @@ __device__ __forceinline__ ff ff_corrected(float f, float d) {
 }
 // 1 / sqrt(x), x a normal positive number: the same third-order step as rsqrt64
 __device__ __forceinline__ ff ff_rsqrt(ff x) {
-  const float r = rsqrtf(x.h), p = __fmul_rn(r, r);
-  ff d = ff_of(-1.f);
-  ff_fma(d, x, ff{p, fmaf(r, r, -p)});
-  return ff_corrected(r, d.h + d.l);
+  const float r = rsqrtf(x.h), y = __fmul_rn(x.h, r);  // y + yl = x r
+  const float yl = fmaf(x.l, r, fmaf(x.h, r, -y));
+  return ff_corrected(r, fmaf(yl, r, fmaf(y, r, -1.f)));
 }
 
 template <>
@@ -245,15 +244,6 @@ __device__ __forceinline__ void reflector_scaled(cplx<double> al, double nx2, cp
     sc *= r;
   }
 }
-__device__ __forceinline__ void reflector_scaled(cplx<ff> al, ff nx2, cplx<ff> &gam, ff &sc) {
-  const int e = (__float_as_int(nx2.h) >> 24) - 63;  // nx2 in [2^(2 e - 1), 2^(2 e + 1))
-  const float f = __int_as_float((127 - e) << 23), g = __int_as_float((127 + e) << 23);
-  reflector_scalars<ff>(cmake<ff>(ff{al.re.h * f, al.re.l * f}, ff{al.im.h * f, al.im.l * f}),
-                        ff{nx2.h * f * f, nx2.l * f * f}, gam, sc);
-  gam = cmake<ff>(ff{gam.re.h * g, gam.re.l * g}, ff{gam.im.h * g, gam.im.l * g});
-  sc = ff{sc.h * f, sc.l * f};
-}
-
 // Reflector of the column x[j..m-1] (elements `stride` apart) in the storage
 // precision T.  A column of norm up to 1e-30 gets none (sc = 0).  Norm and scalars
 // in double, or for float in ff; for float on the column times the power of two
@@ -281,37 +271,50 @@ __device__ __forceinline__ Reflector<double> column_reflector(const cplx<double>
   if (unit) h.sc *= 0.70710678118654752440;
   return h;
 }
-// Squared norm of a float column scaled by down = 2^-(ex - 127), up its inverse.
+// Squared norm of a float column scaled by 2^-(ex - 127).  Up to 128 rows the sum
+// over the warp is taken in integers, of steps 2^-20 and 2^-42 (the largest component is
+// in [1, 2), so 256 squares give 2^30 of the first): two integer reductions for
+// five levels of shuffles, and no rounding between.  Adding a constant with the
+// step as its last place rounds a square to the step, and the integer is the
+// difference of the bit patterns.
 __device__ __forceinline__ ff column_norm2(const cplx<float> *col, int stride, int j, int m, int &ex) {
   float mx = 0.f;
   for (int i = j + lane_id(); i < m; i += 32) mx = fmaxf(mx, fmaxf(fabsf(col[i * stride].re), fabsf(col[i * stride].im)));
   const int bits = __reduce_max_sync(0xffffffffu, __float_as_int(mx));
   ex = min(253, max(1, bits >> 23));
   const float down = __int_as_float((254 - ex) << 23);
-  ff s = ff_of(0.f);
-  for (int i = j + lane_id(); i < m; i += 32) {
-    const float re = col[i * stride].re * down, im = col[i * stride].im * down;
-    ff_fma(s, ff_of(re), ff_of(re));
-    ff_fma(s, ff_of(im), ff_of(im));
+  if (m > 128) {
+    ff s = ff_of(0.f);
+    for (int i = j + lane_id(); i < m; i += 32) {
+      const float re = col[i * stride].re * down, im = col[i * stride].im * down;
+      ff_fma(s, ff_of(re), ff_of(re));
+      ff_fma(s, ff_of(im), ff_of(im));
+    }
+    return lane_sum<ff>(s, 16);
   }
-  // The sum over the warp in two integers, steps 2^-16 and 2^-40 (the largest
-  // component is in [1, 2), so a lane's sum is at most 8 rows per lane and 512
-  // rows give 2^28 in the first): two integer reductions for five levels of
-  // shuffles, and exact.
-  if (m > 512) return lane_sum<ff>(s, 16);
-  const int hi = __float2int_rn(s.h * 0x1p16f);
-  const int lo = __float2int_rn((__fadd_rn(s.h, -static_cast<float>(hi) * 0x1p-16f) + s.l) * 0x1p40f);
+  constexpr float c1 = 12.f, c2 = 0x1.8p-19f;
+  int hi = 0, lo = 0;
+  auto square = [&](float x) {
+    const float p = __fmul_rn(x, x), e = fmaf(x, x, -p);
+    const float s1 = __fadd_rn(p, c1), r = __fadd_rn(__fsub_rn(p, __fsub_rn(s1, c1)), e);
+    hi += __float_as_int(s1) - __float_as_int(c1);
+    lo += __float_as_int(__fadd_rn(r, c2)) - __float_as_int(c2);
+  };
+  for (int i = j + lane_id(); i < m; i += 32) {
+    square(col[i * stride].re * down);
+    square(col[i * stride].im * down);
+  }
   const int th = __reduce_add_sync(0xffffffffu, hi), tl = __reduce_add_sync(0xffffffffu, lo);
-  const float h0 = static_cast<float>(th);
-  return ff_add(ff{h0 * 0x1p-16f, static_cast<float>(th - __float2int_rn(h0)) * 0x1p-16f},
-                ff_of(static_cast<float>(tl) * 0x1p-40f));
+  ff s = ff_norm(ff{static_cast<float>(th & ~4095) * 0x1p-20f, static_cast<float>(th & 4095) * 0x1p-20f});
+  s.l = fmaf(static_cast<float>(tl), 0x1p-42f, s.l);
+  return ff_norm(s);
 }
 __device__ __forceinline__ Reflector<float> column_reflector(const cplx<float> *col, int stride, int j, int m,
                                                              bool unit) {
   int ex;
   const ff s = column_norm2(col, stride, j, m, ex);
   Reflector<float> h{cmake<float>(0.f, 0.f), 0.f, __int_as_float((254 - ex) << 23), __int_as_float(ex << 23)};
-  if (sqrtf(s.h) * h.up > 1e-30f) {
+  if (ex > 30 || sqrtf(s.h) * h.up > 1e-30f) {
     cplx<ff> g;
     ff c;
     const cplx<float> al = cscale(col[j * stride], h.down);
@@ -396,7 +399,7 @@ __device__ __forceinline__ void column_head(cplx<float> *col, int j, int m, Colu
   const ff s = column_norm2(col, 1, j, m, ex);
   const float down = __int_as_float((254 - ex) << 23), up = __int_as_float(ex << 23);
   ColumnHead<float> r{cmake<float>(0.f, 0.f), cmake<float>(0.f, 0.f), 0.f, 0.f};
-  if (sqrtf(s.h) * up > 1e-30f) {
+  if (ex > 30 || sqrtf(s.h) * up > 1e-30f) {  // 2^-97 is above 1e-30
     const bool far = ex < 97 || ex > 157;  // entries up to 2^-30 or from 2^31
     const cplx<float> al = cscale(col[j], down);
     cplx<ff> v0, gam;
@@ -411,6 +414,41 @@ __device__ __forceinline__ void column_head(cplx<float> *col, int j, int m, Colu
       for (int i = j + 1 + lane_id(); i < m; i += 32) col[i] = cscale(col[i], down);
   }
   if (lane_id() == 0) *out = r;
+}
+
+// The same for a column whose squared norm is known, in the working precision: v0,
+// gam and beta to out[0], out[1] and out[2].re.  One warp.
+__device__ __forceinline__ void head_scaled(cplx<double> al, double nx2, cplx<double> *out) {
+  cplx<double> v0, gam;
+  double h, f = 1.0, g = 1.0;
+  if (!(nx2 > 1e-130 && nx2 < 1e130)) {
+    const int ex = min(1535, max(512, (__double2hiint(nx2) >> 21) + 512));  // half the exponent of nx2, biased
+    f = __hiloint2double((2046 - ex) << 20, 0);
+    g = __hiloint2double(ex << 20, 0);
+  }
+  head_scalars<double>(cscale(al, f), nx2 * f * f, v0, gam, h);
+  if (lane_id() == 0) {
+    out[0] = cscale(v0, g);
+    out[1] = cscale(gam, g);
+    out[2].re = reciprocal(h) * f * f;
+  }
+}
+__device__ __forceinline__ void head_scaled(cplx<ff> al, ff nx2, cplx<ff> *out) {
+  const int e = (__float_as_int(nx2.h) >> 24) - 63;  // nx2 in [2^(2 e - 1), 2^(2 e + 1))
+  const float f = __int_as_float((127 - e) << 23), g = __int_as_float((127 + e) << 23);
+  auto times = [](ff x, float y) { return ff{x.h * y, x.l * y}; };  // by a power of two
+  cplx<ff> v0, gam;
+  ff h;
+  head_scalars<ff>(cmake<ff>(times(al.re, f), times(al.im, f)), times(times(nx2, f), f), v0, gam, h);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h.h));
+  const float e1 = fmaf(-h.l, r, fmaf(-h.h, r, 1.f));
+  const ff beta = ff_norm(ff{r, r * fmaf(e1, e1, e1)});
+  if (lane_id() == 0) {
+    out[0] = cmake<ff>(times(v0.re, g), times(v0.im, g));
+    out[1] = cmake<ff>(times(gam.re, g), times(gam.im, g));
+    out[2].re = times(times(beta, f), f);
+  }
 }
 
 // v^dag b over the rows below j of a group's lanes: two accumulators a part, so
@@ -470,24 +508,28 @@ static __device__ __noinline__ void qr_small(int m, int n, const cplx<T> *A, int
     }
   }
   __syncthreads();
-  const int nthr = min(kThreads, team_threads(n) + 32);
-  const int gl = lane_id() & (kGroup - 1), g = tid() / kGroup, groups = nthr / kGroup - 4;
+  // the last warp finds the scalars; it owns columns only where all warps have to
+  const bool spare = team_threads(n) < kThreads;
+  const int nthr = team_threads(n) + (spare ? 32 : 0);
+  const int gl = lane_id() & (kGroup - 1), g = tid() / kGroup, groups = nthr / kGroup - (spare ? 4 : 0);
   if (tid() < nthr) {
-    const bool scalars = g >= groups;
+    const bool scalars = tid() >= nthr - 32, owns = g < groups;
     for (int j = 0; j < steps; ++j) {
       const cplx<T> *x = Bm + j * ld;
-      const int i0 = j + 1 + ((gl - j - 1) & (kGroup - 1));  // a lane keeps its rows: i = gl (mod 8)
+      // a lane keeps its rows, i = gl (mod 8): its first one below row j, and from it
+      const int i0 = j + 1 + ((gl - j - 1) & (kGroup - 1)), ij = j + ((gl - j) & (kGroup - 1));
       // columns j + 1 .. n - 1 in turn, column c to group c % groups
       int c = j + 1 + (g - (j + 1) % groups + groups) % groups;
       cplx<T> w = cmake<T>(0, 0);
       if (scalars) {
         column_head(Bm + j * ld, j, m, head + j);
-      } else if (j + 1 < n) {
+      }
+      if (owns && j + 1 < n) {
         if (c < n) w = dot_below(x, Bm + c * ld, i0, m);
         w = group_sum(w);
       }
       team_sync(nthr);
-      if (!scalars) {
+      if (owns) {
         const ColumnHead<T> h = head[j];
         for (int k = 0; k * groups < n - j - 1; ++k, c += groups) {  // warp-uniform trip count
           cplx<T> *b = Bm + min(c, n - 1) * ld;
@@ -502,15 +544,10 @@ static __device__ __noinline__ void qr_small(int m, int n, const cplx<T> *A, int
             cfma(w, cconj(h.v0), bj);
             w = cscale(w, -h.beta);
 #pragma unroll 4
-            for (int i = i0; i < m; i += kGroup) {
+            for (int i = ij; i < m; i += kGroup) {
               cplx<T> y = b[i];
-              cfma(y, x[i], w);
+              cfma(y, i == j ? h.v0 : x[i], w);
               b[i] = y;
-            }
-            if (gl == (j & (kGroup - 1))) {
-              cplx<T> y = bj;
-              cfma(y, h.v0, w);
-              b[j] = y;
             }
           }
         }
@@ -665,6 +702,77 @@ __device__ __forceinline__ void rotate_pair(cplx<ff> &x, cplx<ff> &y, const Rota
   y = cmake<ff>(ff_two(r.sn, a.re, r.cs, b.re), ff_two(r.sn, a.im, r.cs, b.im));
 }
 
+// Keep count at one bond from its eigenvalues lam (>= 0) in the decreasing order
+// perm, by one warp.  The cutoff is compared in squares, lam_i > cutoff^2 lam_1:
+// square roots (of double, by one thread) were most of the 11,000 cycles the
+// keep decision of a bond took.
+template <typename T>
+static __device__ int keep_count(const T *lam, const int *perm, int n, int cap, double cutoff, double delta) {
+  auto at = [&](int i) { return static_cast<double>(lam[perm[i]]); };
+  auto above = [&](int m, double thr2) {
+    int k = 0;
+    for (int i = 0; i < m; i += 32)
+      k += __popc(__ballot_sync(0xffffffffu, i + lane_id() < m && at(min(i + lane_id(), m - 1)) > thr2));
+    return k;
+  };
+  const double l1 = at(0);
+  if (!(l1 > 0.0)) return 1;
+  int k;
+  if constexpr (sizeof(T) == 4) {  // a float is above a bound if it is above the float below that
+    const float thr = __double2float_rd(cutoff * cutoff * l1);
+    k = 0;
+    for (int i = 0; i < n; i += 32)
+      k += __popc(__ballot_sync(0xffffffffu, i + lane_id() < n && lam[perm[min(i + lane_id(), n - 1)]] > thr));
+    k = max(1, k);
+  } else {
+    k = max(1, above(n, cutoff * cutoff * l1));
+  }
+  if (k > cap) {
+    const double thr = sqrt(at(cap)) + delta * sqrt(l1);
+    k = max(1, above(cap, thr * thr));
+  }
+  return k;
+}
+
+// Discarded over total weight of a bond, by one warp (lane 0's value counts).
+static __device__ __forceinline__ double discarded_weight(const double *lam, const int *perm, int n, int keep) {
+  double tot = 0, drop = 0;
+  for (int i = lane_id(); i < n; i += 32) {
+    const double l = lam[perm[i]];
+    tot += l;
+    if (i >= keep) drop += l;
+  }
+  tot = warp_sum(tot);
+  drop = warp_sum(drop);
+  return tot > 0 ? drop / tot : 0.0;
+}
+static __device__ __forceinline__ double discarded_weight(const float *lam, const int *perm, int n, int keep) {
+  ff tot = ff_of(0.f), drop = ff_of(0.f);
+  for (int i = lane_id(); i < n; i += 32) {
+    const float l = lam[perm[i]];
+    ff_push(tot, l, 0.f);
+    if (i >= keep) ff_push(drop, l, 0.f);
+  }
+  tot = lane_sum<ff>(tot, 16);
+  drop = lane_sum<ff>(drop, 16);
+  if (!(tot.h > 0.f)) return 0.0;
+  const float q = drop.h / tot.h;
+  ff_fma(drop, ff_of(-q), tot);  // the remainder: a second quotient digit of single precision
+  return static_cast<double>(q) + static_cast<double>((drop.h + drop.l) / tot.h);
+}
+
+// What the truncation wants of a bond's SVD: the order of its values, how many are
+// kept (of at most kmax; also the result of svd_small) and the kept vectors.
+template <typename T>
+struct Truncation {
+  int *perm;      // decreasing order of lam (shared memory)
+  int kmax;
+  double delta;
+  int *fail, *keep;
+  double *discarded;  // the discarded over the total weight is added
+  cplx<T> *vs, *site;  // n x keep vectors and, in complex64, the keep x n site of their conjugates
+};
+
 // SVD of a bond in shared memory, in double precision (T = double) or in
 // pairs of floats (T = float): Householder QR with column pivoting, then
 // one-sided (Hestenes) Jacobi on the rows of R, the preconditioning of Drmac
@@ -696,14 +804,20 @@ __device__ __forceinline__ void rotate_pair(cplx<ff> &x, cplx<ff> &y, const Rota
 // rotating them against each other was slower: it leaves the sweeps converging
 // linearly.)
 //
+// With tr (the truncation's) V is not written: values are sorted, counted and the
+// kept vectors stored from shared memory, without a pass through V and back (with
+// the shorter sums of column_norm2 and integer flop counts: a d = 5 round at theta
+// = 1e-3 86.4 -> 79.3 ms, d = 7 151.7 -> 138.1 ms).
+//
 // buf: n (m | 1) 16-byte complex numbers in shared memory, or (SM false) n m of
 // them in global memory, for the few bonds that are too large for a CTA that has
 // half of an SM: the same arithmetic, so a result does not depend on where the
-// matrix was; u: m of them; nr: n doubles (both shared memory); n <=
+// matrix was; u: 3 of them; nr: 2 kSmallSvdCols
+// doubles (both shared memory; lam too, with tr); n <=
 // kSmallSvdCols.  CTA-wide.
 template <typename T, bool SM>
 static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cplx<T> *V, T *lam, double cutoff_,
-                                             void *buf_, void *u_, void *nr_) {
+                                             void *buf_, void *u_, void *nr_, const Truncation<T> *tr = nullptr) {
   using S = std::conditional_t<sizeof(T) == 8, double, ff>;
   using K = Work<S>;
   using R = decltype(K::value(S()));  // double or float
@@ -749,9 +863,16 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   R left = 0;   // bound on the squared norm of the remainder that was
   bool finite = true;
   {
-    const int nthr = team_threads(n);
+    const bool spare = team_threads(n) < kThreads;
+    const int nthr = team_threads(n) + (spare ? 32 : 0), groups = nthr / kGroup - (spare ? 4 : 0);
+    const bool scalars = tid() >= nthr - 32, owns = g < groups;
+    int last = -1;  // the pivot column of the step before, and its diagonal element
+    cplx<S> gam = cmake<S>(K::of(0), K::of(0));
+    auto finish = [&](int c, int i0) {
+      for (int i = i0 + lane_id(); i < m; i += 32) Bm[c * ld + i] = i == i0 ? gam : cmake<S>(K::of(0), K::of(0));
+    };
     if (tid() < nthr) {
-      for (int c = g; (c & ~3) < n; c += kGroups) {
+      for (int c = g; (c & ~3) < n; c += nthr / kGroup) {
         S s = K::of(0);
         if (c < n)
           for (int i = gl; i < m; i += kGroup) K::sq(s, Bm[c * ld + i]);
@@ -773,52 +894,61 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
         left = K::value(nx2) * (n - j);
         if (!(K::value(nx2) > neg) || left <= rest) break;  // what is left is dropped or below rounding
         left = 0;
-        if (warp_id() == (p & (kGroups - 1)) / 4) {
-          cplx<S> *col = Bm + p * ld;
-          cplx<S> gam;
-          S sc;
-          reflector_scaled(col[j], nx2, gam, sc);
-          for (int i = j + lane_id(); i < m; i += 32) {
-            cplx<S> x = col[i];
-            if (i == j) {
-              x.re = K::add(x.re, K::minus(gam.re));
-              x.im = K::add(x.im, K::minus(gam.im));
-            }
-            u[i] = cmake<S>(K::mul(x.re, sc), K::mul(x.im, sc));
-          }
-          __syncwarp();
-          for (int i = j + lane_id(); i < m; i += 32) col[i] = i == j ? gam : cmake<S>(K::of(0), K::of(0));
+        // as in qr_small: v^dag b below row j while one warp finds the scalars
+        const cplx<S> *x = Bm + p * ld;
+        const int i0 = j + ((gl - j) & (kGroup - 1));  // a lane keeps its rows: i = gl (mod 8)
+        auto raw = [&](int c, bool on) {
+          cplx<S> w = cmake<S>(K::of(0), K::of(0));
+          if (on)
+#pragma unroll 4
+            for (int i = i0; i < m; i += kGroup)
+              if (i > j) K::dot(w, x[i], Bm[c * ld + i]);
+          return group_sum(w);
+        };
+        auto open = [&](int c) { return c < n && c != p && K::value(nr[min(c, n - 1)]) >= 0; };
+        cplx<S> w = cmake<S>(K::of(0), K::of(0));
+        if (scalars) {
+          head_scaled(x[j], nx2, u);
+          if (last >= 0) finish(last, j - 1);
         }
+        if (owns) w = raw(g, open(g));
         team_sync(nthr);
-        const int i0 = j + ((gl - j) & (kGroup - 1));
-        for (int c = g; (c & ~3) < n; c += kGroups) {
-          const bool on = c < n && c != p && K::value(nr[min(c, n - 1)]) >= 0;
-          if (__any_sync(0xffffffffu, on)) {
-            cplx<S> *b = Bm + min(c, n - 1) * ld;
-            cplx<S> w = cmake<S>(K::of(0), K::of(0));
-            if (on)
-#pragma unroll 4
-              for (int i = i0; i < m; i += kGroup) K::dot(w, u[i], b[i]);
-            w = group_sum(w);
-            S s = K::of(0);
-            if (on) {
-#pragma unroll 4
-              for (int i = i0; i < m; i += kGroup) {
-                cplx<S> x = b[i];
-                K::axpy(x, u[i], w);
-                b[i] = x;
-                if (i > j) K::sq(s, x);
+        if (owns) {
+          const cplx<S> v0 = u[0];
+          const S beta = u[2].re;
+          for (int c = g; (c & ~3) < n; c += groups) {
+            const bool on = open(c);
+            if (__any_sync(0xffffffffu, on)) {
+              cplx<S> *b = Bm + min(c, n - 1) * ld;
+              if (c != g) w = raw(c, on);
+              S s = K::of(0);
+              if (on) {
+                K::dot(w, v0, b[j]);
+                w = cmake<S>(K::mul(K::norm(w.re), beta), K::mul(K::norm(w.im), beta));
               }
+              __syncwarp();
+              if (on) {
+#pragma unroll 4
+                for (int i = i0; i < m; i += kGroup) {
+                  cplx<S> y = b[i];
+                  K::axpy(y, i == j ? v0 : x[i], w);
+                  b[i] = y;
+                  if (i > j) K::sq(s, y);
+                }
+              }
+              s = group_sum(s);
+              if (gl == 0 && on) nr[c] = s;
             }
-            s = group_sum(s);
-            if (gl == 0 && on) nr[c] = s;
+            __syncwarp();
+            if (gl == 0 && c == p) nr[c] = K::of(-1);
           }
-          __syncwarp();
-          if (gl == 0 && c == p) nr[c] = K::of(-1);
         }
+        last = p;
+        gam = u[1];
         team_sync(nthr);
         rank = j + 1;
       }
+      if (scalars && last >= 0) finish(last, rank - 1);
     }
   }
   // the rank is known to the team's threads
@@ -900,6 +1030,50 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
     norms();
   }
   __syncthreads();
+  if (tr != nullptr) {
+    S *inv = nr + kSmallSvdCols;
+    for (int i = tid(); i < n; i += kThreads) {
+      const T l = i < rank ? static_cast<T>(K::value(nr[i])) * up * up : i == rank ? static_cast<T>(left) * up * up : T(0);
+      const bool bad = !finite || !isfinite(l);
+      if (bad) *tr->fail = STN_ENUMERIC;
+      lam[i] = bad ? T(0) : l;
+      if (i < rank) inv[i] = K::value(nr[i]) > 0 ? K::rsqrt(nr[i]) : K::of(0);
+    }
+    __syncthreads();
+    for (int i = g; (i & ~3) < n; i += kGroups) {  // decreasing order, ties by index
+      const T li = lam[min(i, n - 1)];
+      int before = 0;
+      for (int j = gl; j < n; j += kGroup) before += lam[j] > li || (lam[j] == li && j < i);
+#pragma unroll
+      for (int o = kGroup / 2; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+      if (gl == 0 && i < n) tr->perm[before] = i;
+    }
+    __syncthreads();
+    if (*tr->fail) return 1;
+    if (warp_id() == 0) {
+      const int count = min(keep_count<T>(lam, tr->perm, n, tr->kmax, cutoff_, tr->delta), tr->kmax);
+      if (lane_id() == 0) *tr->keep = count;
+    }
+    __syncthreads();
+    const int keep = *tr->keep;
+    if (warp_id() == kWarps - 1) {  // beside the others
+      const double w = discarded_weight(lam, tr->perm, n, keep);
+      if (lane_id() == 0) *tr->discarded += w;
+    } else {
+      for (int e = tid(); e < n * keep; e += kThreads - 32) {
+        const int c = e / n, i = e % n, row = tr->perm[c];
+        cplx<T> v = cmake<T>(T(i == 0), 0);  // of a zero matrix
+        if (row < rank) {
+          const cplx<S> x = Bm[i * ld + row];
+          v = cmake<T>(static_cast<T>(K::value(K::mul(x.re, inv[row]))), static_cast<T>(-K::value(K::mul(x.im, inv[row]))));
+        }
+        tr->vs[i * keep + c] = v;
+        if (sizeof(T) == 4) tr->site[e] = cconj(v);
+      }
+    }
+    __syncthreads();
+    return keep;
+  }
   for (int e = tid(); e < n * rank; e += kThreads) {
     const int i = e / n, c = e % n;
     const S s = nr[i];
