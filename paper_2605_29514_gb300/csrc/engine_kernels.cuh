@@ -1163,9 +1163,8 @@ static __device__ __noinline__ int svd_onesided(int m, int n, cplx<T> *C, cplx<T
 // step t rotates the disjoint column pairs (b, (b + t) mod w_a) over the
 // smaller block's columns b and the larger block's columns, so each cross
 // pair is visited once per sweep.  A visited block (or block pair) is staged
-// in shared memory with its squared column norms, which the warp that rotates
-// a pair recomputes from the rotated columns, so testing a pair costs one dot
-// product.  With V, a w x w unitary Q accumulates the rotations of the visit
+// in shared memory with its squared column norms, which a rotation updates by
+// what it moves between them, so testing a pair costs one dot product.  With V, a w x w unitary Q accumulates the rotations of the visit
 // and is applied to V's matching columns afterwards, a chunk of V's rows at a
 // time through shared memory.  Outer sweeps repeat until one rotates nothing.
 // Sum over the 16 lanes of a half warp (mask: those lanes), the same value
@@ -1187,34 +1186,42 @@ static __device__ void jacobi_rotate_staged(int m, int w, cplx<T> *Cb, cplx<T> *
   const int hl = lane_id() & 15;
   const unsigned mask = 0xFFFFu << (lane_id() & 16);
   cplx<T> *cp = Cb + static_cast<int64_t>(p) * m, *cq = Cb + static_cast<int64_t>(q) * m;
-  T gr = 0, gi = 0;
+  T g0 = 0, g1 = 0, h0 = 0, h1 = 0;  // conj(x) y, two sums a part
   for (int i = hl; i < m; i += 16) {
     cplx<T> x = cp[i], y = cq[i];
-    gr += x.re * y.re + x.im * y.im;  // conj(x) y
-    gi += x.re * y.im - x.im * y.re;
+    g0 = fma(x.re, y.re, g0);
+    g1 = fma(x.im, y.im, g1);
+    h0 = fma(x.re, y.im, h0);
+    h1 = fma(-x.im, y.re, h1);
   }
-  gr = half_sum(gr, mask);
-  gi = half_sum(gi, mask);
-  const T absg = sqrt(gr * gr + gi * gi);
-  if (!(absg > tol * sqrt(al) * sqrt(be))) return;
-  const T zeta = (be - al) / (T(2) * absg);
-  const T az = fabs(zeta);
-  T t = az > T(1e10) ? T(0.5) / az : T(1) / (az + sqrt(T(1) + zeta * zeta));
-  if (zeta < 0) t = -t;
-  const T cs = T(1) / sqrt(T(1) + t * t), sn = t * cs;
-  const cplx<T> uc = cmake<T>(gr / absg, -gi / absg);  // conj(gamma / |gamma|)
-  T np = 0, nq = 0;
+  const T gr = half_sum(g0 + g1, mask), gi = half_sum(h0 + h1, mask);
+  T cs, sn, tg;
+  cplx<T> uc;
+  if constexpr (sizeof(T) == 8) {
+    // angle in single precision: the roots and divisions were 150 operations of 64 cycles
+    Rotation<double> r;
+    if (!make_rotation(al, be, cmake<double>(gr, gi), static_cast<float>(tol), r)) return;
+    cs = r.cs;
+    sn = r.sn;
+    tg = r.tg;
+    uc = r.uc;
+  } else {
+    const T absg = sqrt(gr * gr + gi * gi);
+    if (!(absg > tol * sqrt(al) * sqrt(be))) return;
+    const T zeta = (be - al) / (T(2) * absg);
+    const T az = fabs(zeta);
+    T t = az > T(1e10) ? T(0.5) / az : T(1) / (az + sqrt(T(1) + zeta * zeta));
+    if (zeta < 0) t = -t;
+    cs = T(1) / sqrt(T(1) + t * t);
+    sn = t * cs;
+    tg = t * absg;
+    uc = cmake<T>(gr / absg, -gi / absg);  // conj(gamma / |gamma|)
+  }
   for (int i = hl; i < m; i += 16) {
     cplx<T> x = cp[i], y = cmul(uc, cq[i]);
-    cplx<T> xn = cmake<T>(cs * x.re - sn * y.re, cs * x.im - sn * y.im);
-    cplx<T> yn = cmake<T>(sn * x.re + cs * y.re, sn * x.im + cs * y.im);
-    cp[i] = xn;
-    cq[i] = yn;
-    np += cabs2(xn);
-    nq += cabs2(yn);
+    cp[i] = cmake<T>(cs * x.re - sn * y.re, cs * x.im - sn * y.im);
+    cq[i] = cmake<T>(sn * x.re + cs * y.re, sn * x.im + cs * y.im);
   }
-  np = half_sum(np, mask);
-  nq = half_sum(nq, mask);
   if (Q != nullptr) {
     cplx<T> *qp = Q + static_cast<int64_t>(p) * w, *qq = Q + static_cast<int64_t>(q) * w;
     for (int i = hl; i < w; i += 16) {
@@ -1225,8 +1232,8 @@ static __device__ void jacobi_rotate_staged(int m, int w, cplx<T> *Cb, cplx<T> *
   }
   __syncwarp(mask);
   if (hl == 0) {
-    nr[p] = np;
-    nr[q] = nq;
+    nr[p] = max(al - tg, T(0));
+    nr[q] = max(be + tg, T(0));
     *flag = 1;
   }
 }
@@ -1891,6 +1898,7 @@ static __device__ __noinline__ void materialize(const MpoSpec<T> &sp, const uint
 //   chi_{k+1})) and A_{k+1} <- R A_{k+1}.
 //   Left across site k: A_k^dag as a (2 chi_{k+1}) x chi_k matrix = Q R;
 //   site k becomes Q^dag and A_{k-1} <- A_{k-1} R^dag.
+// A matrix with no more rows than columns is its own R, with Q = 1.
 template <typename T>
 static __device__ __noinline__ void mps_move_center(const EngineParams &P, const Smem<T> &S, int64_t shot, const Scratch<T> &X,
                                 int target) {
@@ -1906,7 +1914,10 @@ static __device__ __noinline__ void mps_move_center(const EngineParams &P, const
       return;
     }
     cplx<T> *A = site_ptr<T>(P, shot, c), *Bn = site_ptr<T>(P, shot, c + 1);
-    if (qr_small_elems(m, r, true) <= P.svd_elems) {
+    if (m <= r) {
+      cgemm<T, 0, 0>(m, 2 * r2, r, one, A, r, Bn, 2 * r2, zero, X.w, 2 * r2, S.tile);
+      for (int e = tid(); e < m * m; e += kThreads) A[e] = cmake<T>(T(e / m == e % m), 0);
+    } else if (qr_small_elems(m, r, true) <= P.svd_elems) {
       qr_small<T>(m, r, A, r, false, X.t, steps, A, S.jbuf);
       cgemm<T, 0, 0>(steps, 2 * r2, r, one, X.t, r, Bn, 2 * r2, zero, X.w, 2 * r2, S.tile);
     } else {
@@ -1935,7 +1946,10 @@ static __device__ __noinline__ void mps_move_center(const EngineParams &P, const
       return;
     }
     cplx<T> *A = site_ptr<T>(P, shot, c), *Am = site_ptr<T>(P, shot, c - 1);
-    if (qr_small_elems(m, l, true) <= P.svd_elems) {
+    if (m <= l) {
+      cgemm<T, 0, 0>(2 * ll, m, l, one, Am, l, A, m, zero, X.w, m, S.tile);
+      for (int e = tid(); e < m * m; e += kThreads) A[e] = cmake<T>(T(e / m == e % m), 0);
+    } else if (qr_small_elems(m, l, true) <= P.svd_elems) {
       qr_small<T>(m, l, A, m, true, X.t, steps, A, S.jbuf);
       cgemm<T, 0, 1>(2 * ll, steps, l, one, Am, l, X.t, l, zero, X.w, steps, S.tile);
     } else {
@@ -2032,17 +2046,27 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
   for (int k = a; k < b; ++k) {
     const int Dl = Dbond(k), Dr = Dbond(k + 1);
     const cplx<T> *Ak = X.ap + S.off[k - a];
+    cplx<T> *Rout = X.g + S.goff[k + 1 - a];
     int m;
     const cplx<T> *src = X.t;
+    // A matrix with no more rows than columns is an R as it stands (any R with the
+    // same R^dag R will do): it goes where R goes.  That is the first site of most
+    // spans: a d = 5 round at theta = 0.05 takes 158 ms instead of 165, two d = 3
+    // rounds in complex128 54.6 instead of 59.8.
+    bool is_r;
     if (k == a) {
       m = 2 * Dl;
       src = Ak;
+      is_r = m <= Dr;
+      if (is_r)
+        for (int e = tid(); e < m * Dr; e += kThreads) Rout[e] = Ak[e];
     } else {
       const int r = S.rdim[k - a];
       const cplx<T> *Rk = X.g + S.goff[k - a];
-      cgemm<T, 0, 0>(r, 2 * Dr, Dl, one, Rk, Dl, Ak, 2 * Dr, zero, X.t, 2 * Dr, S.tile);
-      if (tid() == 0) tally(S.dmisc, D_FLOPS) += gemm_flops(r, 2 * Dr, Dl);
       m = 2 * r;
+      is_r = m <= Dr;
+      cgemm<T, 0, 0>(r, 2 * Dr, Dl, one, Rk, Dl, Ak, 2 * Dr, zero, is_r ? Rout : X.t, 2 * Dr, S.tile);
+      if (tid() == 0) tally(S.dmisc, D_FLOPS) += gemm_flops(r, 2 * Dr, Dl);
     }
     if (m > kMaxVec) {
       if (tid() == 0) S.misc[M_FAIL] = STN_EOVERFLOW;
@@ -2051,10 +2075,9 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
     }
     if (tid() == 0) tally(S.dmisc, D_FLOPS) += qr_flops(m, Dr);
     const int rn = min(m, Dr);
-    cplx<T> *Rout = X.g + S.goff[k + 1 - a];
-    if (qr_small_elems(m, Dr, false) <= P.svd_elems) {
+    if (!is_r && qr_small_elems(m, Dr, false) <= P.svd_elems) {
       qr_small<T>(m, Dr, src, Dr, false, Rout, rn, nullptr, S.jbuf);
-    } else {
+    } else if (!is_r) {
       if (src != X.t) {
         for (int e = tid(); e < m * Dr; e += kThreads) X.t[e] = src[e];
         __syncthreads();
@@ -2861,9 +2884,9 @@ static __device__ void svd_bond(int m, int n, const cplx<T> *A, cplx<T> *work, c
 // disjoint.  Eight CTAs (the portable limit) have a block pair of 16 + 16 columns
 // each up to 256 columns, and in complex128 blocks of a sixteenth of the columns.
 // One CTA against eight: a 256 x 192 complex64 SVD 23.2 and 4.67 ms, 60 x 50 2.40
-// and 1.18 ms; complex128 128 x 128 98 and 16.3 ms, 72 x 66 (svd_small on one CTA,
-// bound by its SM's FP64 rate) 7.4 and 6.8 ms, 30 x 28 would lose; the R factor of
-// 512 x 250 in complex64 4.1 and 1.6 ms, of 200 x 100 in complex128 4.6 and 2.2 ms.
+// and 1.18 ms; complex128 128 x 128 98 and 10.8 ms, 72 x 66 (svd_small on one CTA,
+// bound by its SM's FP64 rate) 7.4 and 4.6 ms; the R factor of
+// 512 x 250 in complex64 4.1 and 1.58 ms, of 200 x 100 in complex128 4.6 and 2.2 ms.
 constexpr int kShareCtas = 8;
 constexpr int kShareMinCols = 48;  // below, block pairs are too few or too small
 

@@ -271,19 +271,19 @@ __device__ __forceinline__ Reflector<double> column_reflector(const cplx<double>
   if (unit) h.sc *= 0.70710678118654752440;
   return h;
 }
-// Squared norm of a float column scaled by 2^-(ex - 127).  Up to 128 rows the sum
-// over the warp is taken in integers, of steps 2^-20 and 2^-42 (the largest component is
-// in [1, 2), so 256 squares give 2^30 of the first): two integer reductions for
-// five levels of shuffles, and no rounding between.  Adding a constant with the
-// step as its last place rounds a square to the step, and the integer is the
-// difference of the bit patterns.
+// Squared norm of a float column scaled by 2^-(ex - 127).  The sum over the warp is
+// taken in integers, of steps 2^-20 and 2^-42 (the largest component is in [1, 2),
+// so 256 squares give 2^30 of the first), or 2^-17 and 2^-36 for 129 to 1024 rows:
+// two integer reductions for five levels of shuffles, and no rounding between.
+// Adding a constant with the step as its last place rounds a square to the step,
+// and the integer is the difference of the bit patterns.
 __device__ __forceinline__ ff column_norm2(const cplx<float> *col, int stride, int j, int m, int &ex) {
   float mx = 0.f;
   for (int i = j + lane_id(); i < m; i += 32) mx = fmaxf(mx, fmaxf(fabsf(col[i * stride].re), fabsf(col[i * stride].im)));
   const int bits = __reduce_max_sync(0xffffffffu, __float_as_int(mx));
   ex = min(253, max(1, bits >> 23));
   const float down = __int_as_float((254 - ex) << 23);
-  if (m > 128) {
+  if (m > 1024) {
     ff s = ff_of(0.f);
     for (int i = j + lane_id(); i < m; i += 32) {
       const float re = col[i * stride].re * down, im = col[i * stride].im * down;
@@ -292,7 +292,9 @@ __device__ __forceinline__ ff column_norm2(const cplx<float> *col, int stride, i
     }
     return lane_sum<ff>(s, 16);
   }
-  constexpr float c1 = 12.f, c2 = 0x1.8p-19f;
+  const bool tall = m > 128;
+  const float c1 = tall ? 0x1.8p6f : 0x1.8p3f, c2 = tall ? 0x1.8p-13f : 0x1.8p-19f;
+  const float step1 = tall ? 0x1p-17f : 0x1p-20f, step2 = tall ? 0x1p-36f : 0x1p-42f;
   int hi = 0, lo = 0;
   auto square = [&](float x) {
     const float p = __fmul_rn(x, x), e = fmaf(x, x, -p);
@@ -305,8 +307,8 @@ __device__ __forceinline__ ff column_norm2(const cplx<float> *col, int stride, i
     square(col[i * stride].im * down);
   }
   const int th = __reduce_add_sync(0xffffffffu, hi), tl = __reduce_add_sync(0xffffffffu, lo);
-  ff s = ff_norm(ff{static_cast<float>(th & ~4095) * 0x1p-20f, static_cast<float>(th & 4095) * 0x1p-20f});
-  s.l = fmaf(static_cast<float>(tl), 0x1p-42f, s.l);
+  ff s = ff_norm(ff{static_cast<float>(th & ~4095) * step1, static_cast<float>(th & 4095) * step1});
+  s.l = fmaf(static_cast<float>(tl), step2, s.l);
   return ff_norm(s);
 }
 __device__ __forceinline__ Reflector<float> column_reflector(const cplx<float> *col, int stride, int j, int m,
@@ -618,8 +620,9 @@ static __device__ __noinline__ void qr_small(int m, int n, const cplx<T> *A, int
 // is found in single precision from numbers scaled by a power of two; cosine,
 // sine and the phase uc = conj(g / |g|) are then brought to the working
 // precision by a third-order correction, so the rotation is unitary to rounding
-// and only its angle is approximate (which costs no sweep: an angle good to
-// 1e-7 leaves 1e-7 of the product).  tg: what |x|^2 loses and |y|^2 gains;
+// and only its angle is approximate (which costs no sweep: an angle good to a few
+// 1e-7 leaves that much of the product).  So the angle and the test whether there
+// is one to rotate by use the hardware's approximate reciprocal and root.  tg: what |x|^2 loses and |y|^2 gains;
 // reach: |tan| sqrt(max / min) of the norms, at least 0.8 of the rows' cosine.
 template <typename S>
 struct Rotation {
@@ -628,25 +631,40 @@ struct Rotation {
   float reach;
 };
 
+__device__ __forceinline__ float fast_reciprocal(float x) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float fast_root(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ void rotation_angle(float diff, float gr, float gi, float &t, float &ur, float &ui,
                                                float &absg) {
-  const float mx = fmaxf(fmaxf(fabsf(gr), fabsf(gi)), 1e-37f), imx = 1.f / mx;
+  const float mx = fmaxf(fmaxf(fabsf(gr), fabsf(gi)), 1e-37f), imx = fast_reciprocal(mx);
   const float a = gr * imx, b = gi * imx, n2 = a * a + b * b, rn = rsqrtf(n2);
   absg = mx * (n2 * rn);
-  const float zeta = diff / (2.f * absg), az = fabsf(zeta);
-  t = az > 1e10f ? 0.5f / az : 1.f / (az + sqrtf(1.f + az * az));
+  const float zeta = 0.5f * diff * fast_reciprocal(absg), az = fabsf(zeta);
+  t = az > 1e10f ? 0.5f * fast_reciprocal(az) : fast_reciprocal(az + fast_root(1.f + az * az));
   if (zeta < 0.f) t = -t;
   ur = a * rn;
   ui = -b * rn;
 }
 
-__device__ __forceinline__ bool make_rotation(double al, double be, cplx<double> g, double tol2, Rotation<double> &r) {
-  if (!(cabs2(g) > tol2 * al * be)) return false;
-  const int ex = min(2045, max(1, __double2hiint(fmax(al, be)) >> 20));  // the larger norm is scaled to [1, 2)
+__device__ __forceinline__ bool make_rotation(double al, double be, cplx<double> g, float tol, Rotation<double> &r) {
+  // the larger norm is scaled to [1, 2) and the rest seen in single precision: a
+  // double-precision comparison of the squares takes five operations of 64 cycles
+  const int ex = min(2045, max(1, max(__double2hiint(al), __double2hiint(be)) >> 20));
   const double sc = __hiloint2double((2046 - ex) << 20, 0);
+  const float af = static_cast<float>(al * sc), bf = static_cast<float>(be * sc);
+  const float gr = static_cast<float>(g.re * sc), gi = static_cast<float>(g.im * sc);
+  const float root = fast_root(af) * fast_root(bf), lim = tol * root;
+  if (!(fmaxf(fabsf(gr), fabsf(gi)) > 0.70711f * lim)) return false;  // max(|re|, |im|) >= |g| / sqrt(2)
   float tf, urf, uif, absg;
-  rotation_angle(static_cast<float>((be - al) * sc), static_cast<float>(g.re * sc), static_cast<float>(g.im * sc), tf,
-                 urf, uif, absg);
+  rotation_angle(static_cast<float>((be - al) * sc), gr, gi, tf, urf, uif, absg);
+  if (!(absg > lim)) return false;
   const double t = static_cast<double>(tf), w = fma(t, t, 1.0);
   const double c0 = static_cast<double>(rsqrtf(fmaf(tf, tf, 1.f)));
   double d = fma(-w * c0, c0, 1.0);
@@ -657,13 +675,12 @@ __device__ __forceinline__ bool make_rotation(double al, double be, cplx<double>
   d = fma(d, fma(0.375, d, 0.5), 1.0);
   r.uc = cmake<double>(ur * d, ui * d);
   r.tg = static_cast<double>(tf * absg) * __hiloint2double(ex << 20, 0);
-  const float af = static_cast<float>(al * sc), bf = static_cast<float>(be * sc);
-  r.reach = fabsf(tf) * fmaxf(af, bf) * rsqrtf(af * bf);
+  r.reach = fabsf(tf) * fmaxf(af, bf) * fast_reciprocal(root);
   return true;
 }
 __device__ __forceinline__ bool make_rotation(ff al, ff be, cplx<ff> g, float tol, Rotation<ff> &r) {
   const float gr = g.re.h, gi = g.im.h;
-  const float lim = tol * sqrtf(al.h) * sqrtf(be.h);
+  const float lim = tol * fast_root(al.h) * fast_root(be.h);
   if (!(fmaxf(fabsf(gr), fabsf(gi)) > 0.70711f * lim)) return false;  // max(|re|, |im|) >= |g| / sqrt(2)
   float tf, ur, ui, absg;
   rotation_angle(ff_add(be, ff_neg(al)).h, gr, gi, tf, ur, ui, absg);
@@ -678,7 +695,7 @@ __device__ __forceinline__ bool make_rotation(ff al, ff be, cplx<ff> g, float to
   ff_fma(d, ff_of(ui), ff_of(ui));
   r.uc = cmake<ff>(ff_corrected(ur, d.h + d.l), ff_corrected(ui, d.h + d.l));
   r.tg = ff_of(tf * absg);
-  r.reach = fabsf(tf) * fmaxf(al.h, be.h) * __fdividef(tol, lim);
+  r.reach = fabsf(tf) * fmaxf(al.h, be.h) * tol * fast_reciprocal(lim);
   return true;
 }
 
@@ -965,7 +982,6 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   const int kk = rank + (rank & 1), half = kk / 2;
   const int nthr = team_threads(max(1, half));
   const R tol = R(4) * K::eps * sqrt(static_cast<R>(n));
-  const R limit = sizeof(T) == 8 ? tol * tol : tol;  // make_rotation takes tol^2 in double
   // A sweep whose rotations all stayed within `near` is the last one, without a
   // sweep that only finds nothing left.  A pair made orthogonal is disturbed by
   // the sweep's later rotations of p or q with another row r, each by |tan_pr|
@@ -1007,7 +1023,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
             for (int c = gl; c < n; c += kGroup) K::dot(dot, Bm[c * ld + p], Bm[c * ld + q]);
           dot = group_sum(dot);
           Rotation<S> rot;
-          if (on && make_rotation(al, be, dot, limit, rot)) {
+          if (on && make_rotation(al, be, dot, static_cast<float>(tol), rot)) {
             again |= rot.reach > near;
 #pragma unroll 2
             for (int c = gl; c < n; c += kGroup) {
