@@ -13,15 +13,16 @@
 //   left sweep   R_{k+1} = R factor of (R_k A'_k), R_a = identity since the
 //                sites left of the span are left-canonical (Householder QR,
 //                no Q formed); ||R_b A'_b||^2 is the squared norm of the new
-//                state, which for a projector is the Born probability;
+//                state, which for a projector is the Born probability; a
+//                matrix with no more rows than columns is its own R;
 //   right sweep  C = R_k M_k = U Sigma V^dag (one-sided Jacobi); the kept
 //                columns of V give the new right-canonical site and
 //                M_{k-1} = A'_{k-1} (M_k V_keep) carries the rest to the left.
 // Sigma holds the Schmidt values of the bond, so keeping the largest ones is
 // the truncation of Eq. 8.  Small bonds are decomposed in shared memory (in
-// double precision on the complex64 path where that fits); large bonds take
-// the Householder R factor of C and run Jacobi on its conjugate transpose,
-// which converges in a few sweeps.  Dense work runs in complex T (float or
+// pairs of floats on the complex64 path); large bonds take the Householder R
+// factor of C and run Jacobi on its conjugate transpose, which converges in a
+// few sweeps.  Dense work runs in complex T (float or
 // double); norms, Born probabilities and log-probabilities in double.
 #include <cuda_runtime.h>
 #include <math.h>
@@ -2151,7 +2152,8 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
     cplx<T> *Bk = site_ptr<T>(P, shot, k);
     const int kmax = min(cap, P.chimax[k]);
     const int dscale = static_cast<int>(sizeof(double) / sizeof(T));
-    const bool svd64 = n2 <= kSmallSvdCols && r <= kMaxVec && (sizeof(T) == 8 || 2 * (r * n2 + n2 * n2) <= P.svd_rule);
+    const bool svd64 = n2 <= kSmallSvdCols && r <= kMaxVec &&
+                       (sizeof(T) == 8 || (!P.svd64_all && 2 * (r * n2 + n2 * n2) <= P.svd_rule));
     if (svd64) {
       const int elems = n2 * (r | 1) * dscale;
       const Truncation<T> tr{S.perm, kmax, P.delta, &S.misc[M_FAIL], &S.misc[M_KEEP], &S.dmisc[D_DISC], X.vs, Bk};
@@ -2176,27 +2178,36 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       for (int e = tid(); e < r * n2; e += kThreads)
         Cd[e] = cmake<double>(static_cast<double>(X.y[e].re), static_cast<double>(X.y[e].im));
       __syncthreads();
-      const long long tqr = clock64();
-      qr_r_inplace<double>(r, n2, Cd, n2, jd, P.svd_elems / 2);
-      if (tid() == 0) tally(S.dmisc, D_PROF + 1 + PROF_SVD_QR) += clock64() - tqr;
-      const int kx = min(r, n2);
-      for (int e = tid(); e < n2 * kx; e += kThreads) Cd[e] = cconj(Cd[e]);
-      __syncthreads();
-      const long long tj = clock64();
-      const int sweeps = svd_onesided_blocked<double>(n2, kx, Cd, nullptr, sd, &S.misc[M_JFLAG], S.red, jd,
-                                                      P.svd_elems / 2);
-      if (tid() == 0) {
-        tally(S.dmisc, D_PROF + 1 + PROF_JSWEEPS) += sweeps;
-        tally(S.dmisc, D_PROF + 1 + PROF_JROWS) += n2;
-        tally(S.dmisc, D_PROF + 1 + PROF_JCOLS) += kx;
-        if (n2 <= kThreads / 2) tally(S.dmisc, D_PROF + 1 + PROF_JAC_ROWS256) += clock64() - tj;
+      if (n2 <= kSmallSvdCols && 2 * (n2 * (r | 1) + 3) <= P.svd_elems) {  // a small bond: svd_small on the copy
+        cplx<double> *Vd = reinterpret_cast<cplx<double> *>(X.t);  // free in the right sweep, 4 c^2 complex128
+        const int cols = max(1, svd_small<double, true>(r, n2, Cd, Vd, sd, P.cutoff, jd, jd + n2 * (r | 1), S.red));
+        for (int e = tid(); e < n2 * cols; e += kThreads)
+          X.y[e] = cmake<T>(static_cast<T>(Vd[e].re), static_cast<T>(Vd[e].im));
+        for (int i = tid(); i < n2; i += kThreads) X.lam[i] = static_cast<T>(sd[i]);
+        Vc = X.y;
+      } else {
+        const long long tqr = clock64();
+        qr_r_inplace<double>(r, n2, Cd, n2, jd, P.svd_elems / 2);
+        if (tid() == 0) tally(S.dmisc, D_PROF + 1 + PROF_SVD_QR) += clock64() - tqr;
+        const int kx = min(r, n2);
+        for (int e = tid(); e < n2 * kx; e += kThreads) Cd[e] = cconj(Cd[e]);
+        __syncthreads();
+        const long long tj = clock64();
+        const int sweeps = svd_onesided_blocked<double>(n2, kx, Cd, nullptr, sd, &S.misc[M_JFLAG], S.red, jd,
+                                                        P.svd_elems / 2);
+        if (tid() == 0) {
+          tally(S.dmisc, D_PROF + 1 + PROF_JSWEEPS) += sweeps;
+          tally(S.dmisc, D_PROF + 1 + PROF_JROWS) += n2;
+          tally(S.dmisc, D_PROF + 1 + PROF_JCOLS) += kx;
+          if (n2 <= kThreads / 2) tally(S.dmisc, D_PROF + 1 + PROF_JAC_ROWS256) += clock64() - tj;
+        }
+        for (int e = tid(); e < n2 * kx; e += kThreads)
+          X.y[e] = cmake<T>(static_cast<T>(Cd[e].re), static_cast<T>(Cd[e].im));
+        for (int i = tid(); i < n2; i += kThreads) X.lam[i] = i < kx ? static_cast<T>(sd[i]) : T(0);
+        __syncthreads();
+        Vc = X.y;
+        vec_from_columns = true;
       }
-      for (int e = tid(); e < n2 * kx; e += kThreads)
-        X.y[e] = cmake<T>(static_cast<T>(Cd[e].re), static_cast<T>(Cd[e].im));
-      for (int i = tid(); i < n2; i += kThreads) X.lam[i] = i < kx ? static_cast<T>(sd[i]) : T(0);
-      __syncthreads();
-      Vc = X.y;
-      vec_from_columns = true;
     } else if (in_smem) {
       for (int e = tid(); e < r * n2; e += kThreads) {
         int i = e / n2, j = e % n2;
@@ -2252,7 +2263,7 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       tally(S.dmisc, D_PROF + 1 + (vec_from_columns ? PROF_NSVD_LARGE : PROF_NSVD_SMALL)) += 1;
     }
     if (S.misc[M_FAIL]) return;
-    const bool orthonormal = sizeof(T) == 4 && svd64;
+    const bool rounded = sizeof(T) == 4 && !vec_from_columns && (svd64 || P.svd64_all);
     if (!svd64) {
       // S.lam holds the squared values, S.perm their order
       for (int i = tid(); i < n2; i += kThreads) {
@@ -2288,11 +2299,11 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       __syncthreads();
     }
     // and the new right-canonical site k: B[c][s][r] = conj(Vs[(s*kappa + r)][c]).
-    // Vectors rounded from pairs of floats to float are orthonormal to rounding
-    // (svd_small has stored that site); the others take one Newton-Schulz step
-    // before.
-    if (!orthonormal) {
-      reorthonormalize<T>(n2, keep, X.vs, X.e, X.y, S.tile);
+    // Vectors rounded to float from a higher precision are orthonormal to rounding
+    // (from pairs of floats, svd_small has stored the site too); the others take one
+    // Newton-Schulz step before.
+    if (!rounded) reorthonormalize<T>(n2, keep, X.vs, X.e, X.y, S.tile);
+    if (!rounded || !svd64) {
       for (int e = tid(); e < keep * n2; e += kThreads) {
         int c = e / n2, sr = e % n2;
         Bk[e] = cconj(X.vs[sr * keep + c]);

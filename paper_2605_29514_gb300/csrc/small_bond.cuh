@@ -9,10 +9,10 @@
 // only the warps that hold columns take part in a step's barrier, and square
 // roots start from the hardware's approximation.
 //
-// An FP64 instruction of a warp holds its quarter of the SM for 64 cycles
-// (measured; a dependent FP32 FMA takes 4), so the complex64 path computes what
-// has to be better than single precision in pairs of floats (ff, 48 bits): the
-// SVD it used to run in double, and the norms and scalars of its reflectors.
+// A double-precision operation takes 64 cycles, and an SM issues a warp's every
+// 19 whatever its active lanes (measured; a dependent FP32 FMA takes 4.6), so the
+// complex64 path computes what has to be better than single precision in pairs of
+// floats (ff, 48 bits): its SVDs, and the norms and scalars of its reflectors.
 
 STN_BEGIN
 
