@@ -1167,7 +1167,7 @@ static __device__ __noinline__ int svd_onesided(int m, int n, cplx<T> *C, cplx<T
 // in shared memory with its squared column norms, which a rotation updates by
 // what it moves between them, so testing a pair costs one dot product.  With V, a w x w unitary Q accumulates the rotations of the visit
 // and is applied to V's matching columns afterwards, a chunk of V's rows at a
-// time through shared memory.  Outer sweeps repeat until one rotates nothing.
+// time through shared memory.  Outer sweeps repeat until one has only small rotations.
 // Sum over the 16 lanes of a half warp (mask: those lanes), the same value
 // broadcast to all of them.
 template <typename T>
@@ -1181,7 +1181,7 @@ __device__ __forceinline__ T half_sum(T v, unsigned mask) {
 // halves of a warp work on two disjoint pairs).
 template <typename T>
 static __device__ void jacobi_rotate_staged(int m, int w, cplx<T> *Cb, cplx<T> *Q, T *nr, int p, int q, T tol,
-                                     T negligible, int *flag) {
+                                     T negligible, float near, int *flag, int *any) {
   const T al = nr[p], be = nr[q];
   if (!(al > negligible) || !(be > negligible)) return;
   const int hl = lane_id() & 15;
@@ -1198,6 +1198,7 @@ static __device__ void jacobi_rotate_staged(int m, int w, cplx<T> *Cb, cplx<T> *
   const T gr = half_sum(g0 + g1, mask), gi = half_sum(h0 + h1, mask);
   T cs, sn, tg;
   cplx<T> uc;
+  float reach;
   if constexpr (sizeof(T) == 8) {
     // angle in single precision: the roots and divisions were 150 operations of 64 cycles
     Rotation<double> r;
@@ -1206,9 +1207,10 @@ static __device__ void jacobi_rotate_staged(int m, int w, cplx<T> *Cb, cplx<T> *
     sn = r.sn;
     tg = r.tg;
     uc = r.uc;
+    reach = r.reach;
   } else {
-    const T absg = sqrt(gr * gr + gi * gi);
-    if (!(absg > tol * sqrt(al) * sqrt(be))) return;
+    const T absg = sqrt(gr * gr + gi * gi), root = sqrt(al) * sqrt(be);
+    if (!(absg > tol * root)) return;
     const T zeta = (be - al) / (T(2) * absg);
     const T az = fabs(zeta);
     T t = az > T(1e10) ? T(0.5) / az : T(1) / (az + sqrt(T(1) + zeta * zeta));
@@ -1216,6 +1218,7 @@ static __device__ void jacobi_rotate_staged(int m, int w, cplx<T> *Cb, cplx<T> *
     cs = T(1) / sqrt(T(1) + t * t);
     sn = t * cs;
     tg = t * absg;
+    reach = fabs(t) * max(al, be) / root;
     uc = cmake<T>(gr / absg, -gi / absg);  // conj(gamma / |gamma|)
   }
   for (int i = hl; i < m; i += 16) {
@@ -1236,6 +1239,7 @@ static __device__ void jacobi_rotate_staged(int m, int w, cplx<T> *Cb, cplx<T> *
     nr[p] = max(al - tg, T(0));
     nr[q] = max(be + tg, T(0));
     *flag = 1;
+    if (reach > near) *any = 1;
   }
 }
 
@@ -1294,7 +1298,7 @@ constexpr int kLamElems = kRvWrkFloats > 512 ? kRvWrkFloats : 512;
 
 template <int R>
 static __device__ bool cross_visit_regs(int m, cplx<float> *C, int c0, int wI, int c1, int wJ, float tol,
-                                        float negligible, float *wrk) {
+                                        float negligible, float near, float *wrk, int *any) {
   float *red = wrk;                   // kWarps * 32
   float4 *prm = reinterpret_cast<float4 *>(wrk + kWarps * 32);  // 16 rotations
   float *nrm = wrk + kWarps * 32 + 64;  // 32 column norms: I then J (in J's column order)
@@ -1350,8 +1354,8 @@ static __device__ bool cross_visit_regs(int m, cplx<float> *C, int c0, int wI, i
         const float gr = s, al = nrm[b], be = nrm[16 + jb];
         float4 p = make_float4(1.f, 0.f, 1.f, 0.f);  // identity: skipped
         if (al > negligible && be > negligible) {
-          const float absg = sqrtf(gr * gr + gi * gi);
-          if (absg > tol * sqrtf(al) * sqrtf(be)) {
+          const float absg = sqrtf(gr * gr + gi * gi), root = sqrtf(al) * sqrtf(be);
+          if (absg > tol * root) {
             const float zeta = (be - al) / (2.f * absg);
             const float az = fabsf(zeta);
             float tt = az > 1e10f ? 0.5f / az : 1.f / (az + sqrtf(1.f + zeta * zeta));
@@ -1361,6 +1365,7 @@ static __device__ bool cross_visit_regs(int m, cplx<float> *C, int c0, int wI, i
             nrm[b] = fmaxf(al - tt * absg, 0.f);
             nrm[16 + jb] = fmaxf(be + tt * absg, 0.f);
             *rot = 1;
+            if (fabsf(tt) * fmaxf(al, be) > near * root) *any = 1;
           }
         }
         prm[b] = p;
@@ -1409,9 +1414,9 @@ static __device__ bool cross_visit_regs(int m, cplx<float> *C, int c0, int wI, i
 
 template <typename T>
 static __device__ bool cross_visit_dispatch(int m, cplx<T> *C, int c0, int wI, int c1, int wJ, T tol, T negligible,
-                                            float *wrk) {
+                                            float near, float *wrk, int *any) {
   if constexpr (sizeof(T) == 4) {
-    return cross_visit_regs<1>(m, C, c0, wI, c1, wJ, tol, negligible, wrk);  // m <= kThreads
+    return cross_visit_regs<1>(m, C, c0, wI, c1, wJ, tol, negligible, near, wrk, any);  // m <= kThreads
   } else {
     return false;
   }
@@ -1430,6 +1435,10 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
                                      double *red, cplx<T> *sbuf, int sbuf_elems, float *rv_wrk = nullptr) {
   const T negligible = onesided_prologue<T>(m, n, C, V, red);
   const T tol = onesided_tol<T>(m);
+  // A sweep whose rotations all reach no further than `near` is the last one: what it
+  // leaves is within tol (svd_small explains the bound), and the sweep that would
+  // find nothing was one of 4.5.
+  const float near = sqrtf(static_cast<float>(tol) / (2.5f * static_cast<float>(n)));
   // staged block pair: Q (w x w, only with V), norms (w complex slots),
   // columns (m x w)
   const bool withV = V != nullptr;
@@ -1472,9 +1481,8 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
     const int c1 = J * bw, wJ = self ? 0 : min(bw, n - c1);
     const int w = wI + wJ;
     if (regs && !self) {
-      if (cross_visit_dispatch<T>(m, C, c0, wI, c1, wJ, tol, negligible, rv_wrk)) {
+      if (cross_visit_dispatch<T>(m, C, c0, wI, c1, wJ, tol, negligible, near, rv_wrk, any)) {
         if (skipping && tid() == 0) mark(I, J, stamp);
-        if (tid() == 0) *any = 1;
       }
       __syncthreads();
       return;
@@ -1508,7 +1516,7 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
           else { p = (round + pi) % (mm - 1); q = (round - pi + (mm - 1)) % (mm - 1); }
           if (p > q) { int tt = p; p = q; q = tt; }
           if (q >= w) continue;
-          jacobi_rotate_staged<T>(m, w, Cb, Q, nr, p, q, tol, negligible, flag);
+          jacobi_rotate_staged<T>(m, w, Cb, Q, nr, p, q, tol, negligible, near, flag, any);
         }
         __syncthreads();
       }
@@ -1520,7 +1528,7 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
         for (int b = hw; b < wb; b += 2 * kWarps) {
           const int a = (b + t) % wa;
           const int p = i_larger ? a : b, q = wI + (i_larger ? b : a);
-          jacobi_rotate_staged<T>(m, w, Cb, Q, nr, p, q, tol, negligible, flag);
+          jacobi_rotate_staged<T>(m, w, Cb, Q, nr, p, q, tol, negligible, near, flag, any);
         }
         __syncthreads();
       }
@@ -1562,7 +1570,6 @@ static __device__ __noinline__ int svd_onesided_blocked(int m, int n, cplx<T> *C
       }
       __syncthreads();
     }
-    if (tid() == 0) *any = 1;
   };
 
   int sweeps = 0;
