@@ -54,8 +54,9 @@ typedef enum {
 enum { STN_PAIRS_ADJACENT_IDLE = 0, STN_PAIRS_ADJACENT_IDLE_DIAG_XX = 1 };
 /* Arithmetic of the MPS path.  C128: complex128 throughout.  C64: complex64
  * contractions; norms, Born probabilities and log P in double; the SVDs of
- * bonds whose complex128 copy fits shared memory (about 75 columns) in double
- * precision, larger bonds by single-precision Jacobi on the R factor.
+ * bonds whose copy in 16-byte numbers fits shared memory (about 75 columns) in
+ * pairs of floats (48 bits), larger bonds by single-precision Jacobi on the R
+ * factor.
  * C64_SVD64: as C64 with every bond SVD (R factor and Jacobi) in double
  * precision, at the FP64 rate of the GPU. */
 enum { STN_PRECISION_C128 = 0, STN_PRECISION_C64 = 1, STN_PRECISION_C64_SVD64 = 2 };
@@ -344,8 +345,9 @@ stn_status stn_philox_uniforms(uint64_t seed, uint64_t shot_offset, int64_t n_sh
                                uint32_t event_offset, int32_t n_events, double *d_out,
                                void *cuda_stream);
 
-/* Dense building blocks of the truncation sweep (Sec. IV B, Eq. 8), run alone
- * on one CTA for checking.  precision: STN_PRECISION_*; complex elements are
+/* Dense building blocks of the truncation sweep (Sec. IV B, Eq. 8), run alone:
+ * on one CTA, or, for R factors past its shared memory and SVDs (in_shared = 3)
+ * of 48 columns and more, on a cluster of eight.  precision: STN_PRECISION_*; complex elements are
  * interleaved (re, im) of that precision, all device memory.
  * stn_dense_qr: Householder QR of d_b (m x n, row-major, m <= 1024), in
  *   place; rows 0..min(m,n)-1 then hold R, the rest is zero.

@@ -323,7 +323,7 @@ def dense_gemm_tc(m, n, k, d_a, d_b, d_c, d_status, stream=0):
 def dense_cgemm(precision, op_a, op_b, m, n, k, d_a, lda, d_b, ldb, d_c, ldc, d_status, alpha=1.0, beta=0.0,
                 gemm_units=GEMM_FMA, stream=0):
     """stn_dense_cgemm: d_c = alpha op(A) op(B) + beta d_c (row-major complex
-    device buffers, op 0 = identity, 1 = conjugate transpose) on one CTA
+    device buffers, op 0 = identity, 1 = conjugate transpose)
     through the sweeps' contraction routine."""
     al = (ctypes.c_double * 2)(complex(alpha).real, complex(alpha).imag)
     be = (ctypes.c_double * 2)(complex(beta).real, complex(beta).imag)
