@@ -174,3 +174,24 @@ def test_large_matrices_over_a_cluster(precision, m, n):
     grow = np.sqrt(15 * k)
     assert np.abs(vk.conj().T @ vk - np.eye(k)).max() < 64 * EPS[precision] * np.sqrt(m * n) * grow
     assert np.abs(a @ vk @ vk.conj().T - a).max() < bound * grow
+
+
+@pytest.mark.parametrize("precision,scales", [(1, (1.0, 1e-12, 1e12, 1e-25)), (1, (1e-20,)), (0, (1.0, 1e70, 1e-25)),
+                                              (0, (1e75,))])
+@pytest.mark.parametrize("m,n", [(3, 2), (40, 20), (100, 70), (128, 30), (129, 30), (400, 40)])
+def test_qr_of_columns_far_from_one(precision, scales, m, n):
+    """Columns whose reflectors are scaled by a power of two, beside ordinary
+    ones; a Householder QR is backward stable column by column, so the bounds hold
+    relative to each column's norm.  128 and 129 rows: both steps of the integer
+    column norm."""
+    rng = np.random.default_rng(m * n)
+    size = np.array([scales[c % len(scales)] for c in range(n)])
+    a = (cmat(rng, m, n, 0) * size).astype([np.complex128, np.complex64][precision])
+    b, q = torch.tensor(a, device="cuda"), torch.zeros(m, n, dtype=CDT[precision], device="cuda")
+    work = torch.zeros(m, n, dtype=CDT[precision], device="cuda")
+    stn.dense_qr_q(precision, m, n, b.data_ptr(), q.data_ptr(), work.data_ptr())
+    b, q = (x.cpu().numpy().astype(np.complex128) for x in (b, q))
+    a = a.astype(np.complex128)
+    bound = 64 * EPS[precision] * np.sqrt(m * n)
+    assert np.abs(q.conj().T @ q - np.eye(n)).max() < bound
+    assert (np.abs(q @ b[:n] - a).max(axis=0) / np.linalg.norm(a, axis=0)).max() < bound
