@@ -350,7 +350,9 @@ stn_status stn_philox_uniforms(uint64_t seed, uint64_t shot_offset, int64_t n_sh
  * of 48 columns and more, on a cluster of eight.  precision: STN_PRECISION_*; complex elements are
  * interleaved (re, im) of that precision, all device memory.
  * stn_dense_qr: Householder QR of d_b (m x n, row-major, m <= 1024), in
- *   place; rows 0..min(m,n)-1 then hold R, the rest is zero.
+ *   place; rows 0..min(m,n)-1 then hold R, the rest is zero.  Row j has the
+ *   phase -x_j / |x_j| of its reflected column x, known to eps ||x|| / |x_j|;
+ *   that it is computed by one CTA or by a cluster changes no bit of R.
  * stn_dense_svd: one-sided Jacobi SVD of d_c (m x n, column-major, n <= 512):
  *   d_c becomes U diag(sigma), d_v (n x n, column-major) the right singular
  *   vectors, d_sig2[n] (real, of the precision) sigma^2, unsorted.

@@ -748,11 +748,13 @@ __device__ __forceinline__ void share_store(int *p, int rank, int v) {
 // its reflectors u_1..u_nb are kept as the columns of V, and the product
 // P_nb ... P_1 = I - V T^dag V^dag (compact WY form, T upper triangular with
 // T_kk = 2, T[0:k, k] = -2 T[0:k, 0:k] V[:, 0:k]^dag u_k) is applied to the
-// trailing columns at once, one thread per column, so the trailing matrix is
+// trailing columns at once (qr_trailing), so the trailing matrix is
 // read and written twice per panel rather than per column.  pbuf needs
 // m (nb + 1) + 2 nb^2 complex elements (nb is reduced to fit).  CTA-wide, or over
 // a cluster: every CTA factors the panel for itself, the first one writes it back,
-// and the trailing columns are split.
+// and the trailing columns are split.  R is the same to the last bit either way:
+// row j of R carries the phase of x_j, known to eps ||x|| / |x_j| only, so sums in
+// another order would move single elements of a large R by 1e-3.
 constexpr int kQrPanel = 16;
 
 static __device__ __forceinline__ int qr_panel_width(int m, int pbuf_elems) {
@@ -791,6 +793,112 @@ static __device__ void wy_t_factor(int mr, int jb, int nb, int ldv, const cplx<T
     }
   }
   __syncthreads();
+}
+
+// Trailing columns of a panel: b <- b - V (T^dag (V^dag b)).  The columns go to
+// the warps in groups of cpw consecutive ones (coalesced row reads).  The ns G
+// lanes that share a column split w = V^dag b: slice s sums over the rows s, s +
+// ns, ..., for the reflectors of one of G groups; the slices' partials are summed
+// by shuffles and the groups' values exchanged, and then the lanes split the rows
+// of the update.  w and the update depend on ns but not on G, which spreads a
+// column over more lanes without another order of summation.  Rows go several at
+// a time so that their loads are in flight together.  A cluster's CTAs have lanes
+// to spare: with G = 4 or 8 the R factor of 512 x 250 in complex64 takes 1.36 ms;
+// more slices instead (ns = 8) took 1.57 ms and gave an R with other phases.
+template <typename T, int G>
+static __device__ __forceinline__ void qr_trailing(int mr, int n, int j0, int jb, int nb, int ldv, const cplx<T> *Vp,
+                                                   const cplx<T> *Tm, cplx<T> *B, int ld, int ns, int warp,
+                                                   int warps) {
+  constexpr int KW = kQrPanel / G;  // reflectors of a lane
+  constexpr int U = G == 1 ? 4 : 64 / static_cast<int>(sizeof(T));  // rows in flight in w
+  const int cpw = 32 / (ns * G), part = lane_id() / cpw, s = part % ns, k0 = part / ns * KW;
+  for (int cb = j0 + jb + warp * cpw; cb < n; cb += warps * cpw) {  // warp-uniform trip count
+    const int c = cb + lane_id() % cpw;
+    const bool valid = c < n;
+    cplx<T> own[KW], all[G == 1 ? 1 : kQrPanel], *const w = G == 1 ? own : all;
+#pragma unroll
+    for (int k = 0; k < KW; ++k) own[k] = cmake<T>(0, 0);
+    if (valid) {
+      int i = s;
+      for (; i + (U - 1) * ns < mr; i += U * ns) {
+        cplx<T> b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) b[u] = B[static_cast<int64_t>(j0 + i + u * ns) * ld + c];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int k = 0; k < KW; ++k)
+            if (k0 + k < jb) cfma(own[k], cconj(Vp[(i + u * ns) * ldv + k0 + k]), b[u]);
+      }
+      for (; i < mr; i += ns) {
+        const cplx<T> b = B[static_cast<int64_t>(j0 + i) * ld + c];
+#pragma unroll
+        for (int k = 0; k < KW; ++k)
+          if (k0 + k < jb) cfma(own[k], cconj(Vp[i * ldv + k0 + k]), b);
+      }
+    }
+    for (int off = cpw; off < cpw * ns; off *= 2)
+#pragma unroll
+      for (int k = 0; k < KW; ++k)
+        if (G > 1 || k < jb) {
+          own[k].re += __shfl_xor_sync(0xffffffffu, own[k].re, off);
+          own[k].im += __shfl_xor_sync(0xffffffffu, own[k].im, off);
+        }
+    // every lane gets the groups' values, in order
+    auto exchange = [&]() {
+      if constexpr (G > 1) {
+        const int first = lane_id() % (cpw * ns);
+#pragma unroll
+        for (int k = 0; k < kQrPanel; ++k) {
+          const int from = first + k / KW * (cpw * ns);
+          w[k] = cmake<T>(__shfl_sync(0xffffffffu, own[k % KW].re, from), __shfl_sync(0xffffffffu, own[k % KW].im, from));
+        }
+      }
+    };
+    exchange();
+    // w <- T^dag w, highest index first: w'[a] = sum_{b<=a} conj(T[b][a]) w[b]
+#pragma unroll
+    for (int k = KW - 1; k >= 0; --k) {
+      const int a = k0 + k;
+      if (a >= jb) continue;
+      cplx<T> acc = cmake<T>(0, 0);
+#pragma unroll
+      for (int b = 0; b < kQrPanel; ++b)
+        if (b <= a) cfma(acc, cconj(Tm[b * nb + a]), w[b]);
+      own[k] = acc;
+    }
+    exchange();
+    if (valid) {
+      const int step = ns * G;
+      int i = part;
+      for (; i + 3 * step < mr; i += 4 * step) {
+        cplx<T> b[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) b[u] = B[static_cast<int64_t>(j0 + i + u * step) * ld + c];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+#pragma unroll
+          for (int k = 0; k < kQrPanel; ++k)
+            if (k < jb) {
+              const cplx<T> t = cmul(Vp[(i + u * step) * ldv + k], w[k]);
+              b[u] = cmake<T>(b[u].re - t.re, b[u].im - t.im);
+            }
+          B[static_cast<int64_t>(j0 + i + u * step) * ld + c] = b[u];
+        }
+      }
+      for (; i < mr; i += step) {
+        cplx<T> &bref = B[static_cast<int64_t>(j0 + i) * ld + c];
+        cplx<T> acc = bref;
+#pragma unroll
+        for (int k = 0; k < kQrPanel; ++k)
+          if (k < jb) {
+            const cplx<T> t = cmul(Vp[i * ldv + k], w[k]);
+            acc = cmake<T>(acc.re - t.re, acc.im - t.im);
+          }
+        bref = acc;
+      }
+    }
+  }
 }
 
 // With vstore (row-major m x min(m,n)), the reflectors are also kept there
@@ -873,90 +981,17 @@ static __device__ __noinline__ void qr_r_inplace(int m, int n, cplx<T> *B, int l
       continue;
     }
     wy_t_factor<T>(mr, jb, nb, ldv, Vp, Tm, G);
-    // trailing columns: b <- b - V (T^dag (V^dag b)).  The nt trailing
-    // columns go to the warps in groups of cpw = 32 / ns consecutive columns
-    // (coalesced row reads), and the ns lanes that share a column split its
-    // rows (rows s, s + ns, s + 2 ns, ... for slice s); their partials of
-    // w = V^dag b are summed by shuffles, so that a trailing matrix of a few
-    // hundred columns still occupies the whole CTA.  Rows go four at a time
-    // so that four loads per thread are in flight.
     {
-      const int nt = n - j0 - jb;
+      // the slices of one CTA whatever the number of CTAs, so that R does not depend on it
+      const int nt = n - j0 - jb, ranks = share_size<CL>();
       int ns = 1;
-      const int ranks = share_size<CL>();
-      while (ns < 8 && nt * 2 * ns <= kThreads * ranks) ns *= 2;
-      const int cpw = 32 / ns, s = lane_id() / cpw;
-      for (int cb = j0 + jb + (warp_id() * ranks + share_rank<CL>()) * cpw; cb < n;
-           cb += kWarps * ranks * cpw) {  // warp-uniform trip count
-        const int c = cb + lane_id() % cpw;
-        const bool valid = c < n;
-        cplx<T> w[kQrPanel];
-#pragma unroll
-        for (int k = 0; k < kQrPanel; ++k) w[k] = cmake<T>(0, 0);
-        if (valid) {
-          int i = s;
-          for (; i + 3 * ns < mr; i += 4 * ns) {
-            cplx<T> b[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) b[u] = B[static_cast<int64_t>(j0 + i + u * ns) * ld + c];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-              for (int k = 0; k < kQrPanel; ++k)
-                if (k < jb) cfma(w[k], cconj(Vp[(i + u * ns) * ldv + k]), b[u]);
-          }
-          for (; i < mr; i += ns) {
-            const cplx<T> b = B[static_cast<int64_t>(j0 + i) * ld + c];
-#pragma unroll
-            for (int k = 0; k < kQrPanel; ++k)
-              if (k < jb) cfma(w[k], cconj(Vp[i * ldv + k]), b);
-          }
-        }
-        for (int off = cpw; off < 32; off *= 2)
-#pragma unroll
-          for (int k = 0; k < kQrPanel; ++k)
-            if (k < jb) {
-              w[k].re += __shfl_xor_sync(0xffffffffu, w[k].re, off);
-              w[k].im += __shfl_xor_sync(0xffffffffu, w[k].im, off);
-            }
-        // w <- T^dag w in place, highest index first: w'[a] = sum_{b<=a} conj(T[b][a]) w[b]
-#pragma unroll
-        for (int a = kQrPanel - 1; a >= 0; --a) {
-          if (a >= jb) continue;
-          cplx<T> acc = cmake<T>(0, 0);
-#pragma unroll
-          for (int b = 0; b <= a; ++b) cfma(acc, cconj(Tm[b * nb + a]), w[b]);
-          w[a] = acc;
-        }
-        if (valid) {
-          int i = s;
-          for (; i + 3 * ns < mr; i += 4 * ns) {
-            cplx<T> b[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) b[u] = B[static_cast<int64_t>(j0 + i + u * ns) * ld + c];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-#pragma unroll
-              for (int k = 0; k < kQrPanel; ++k)
-                if (k < jb) {
-                  const cplx<T> t = cmul(Vp[(i + u * ns) * ldv + k], w[k]);
-                  b[u] = cmake<T>(b[u].re - t.re, b[u].im - t.im);
-                }
-              B[static_cast<int64_t>(j0 + i + u * ns) * ld + c] = b[u];
-            }
-          }
-          for (; i < mr; i += ns) {
-            cplx<T> &bref = B[static_cast<int64_t>(j0 + i) * ld + c];
-            cplx<T> acc = bref;
-#pragma unroll
-            for (int k = 0; k < kQrPanel; ++k)
-              if (k < jb) {
-                const cplx<T> t = cmul(Vp[i * ldv + k], w[k]);
-                acc = cmake<T>(acc.re - t.re, acc.im - t.im);
-              }
-            bref = acc;
-          }
-        }
+      while (ns < 8 && nt * 2 * ns <= kThreads) ns *= 2;
+      const int warp = warp_id() * ranks + share_rank<CL>(), warps = kWarps * ranks;
+      if constexpr (CL) {  // as many lanes as a warp has for its columns
+        if (ns == 8) qr_trailing<T, 4>(mr, n, j0, jb, nb, ldv, Vp, Tm, B, ld, ns, warp, warps);
+        else qr_trailing<T, 8>(mr, n, j0, jb, nb, ldv, Vp, Tm, B, ld, ns, warp, warps);
+      } else {
+        qr_trailing<T, 1>(mr, n, j0, jb, nb, ldv, Vp, Tm, B, ld, ns, warp, warps);
       }
     }
     share_sync<CL>();
@@ -2904,7 +2939,7 @@ static __device__ void svd_bond(int m, int n, const cplx<T> *A, cplx<T> *work, c
 // One CTA against eight: a 256 x 192 complex64 SVD 23.2 and 4.67 ms, 60 x 50 2.40
 // and 1.18 ms; complex128 128 x 128 98 and 10.8 ms, 72 x 66 (svd_small on one CTA,
 // bound by its SM's FP64 rate) 7.4 and 4.6 ms; the R factor of
-// 512 x 250 in complex64 4.1 and 1.58 ms, of 200 x 100 in complex128 4.6 and 2.2 ms.
+// 512 x 250 in complex64 4.0 and 1.36 ms, of 200 x 100 in complex128 4.5 and 1.8 ms.
 constexpr int kShareCtas = 8;
 constexpr int kShareMinCols = 48;  // below, block pairs are too few or too small
 
