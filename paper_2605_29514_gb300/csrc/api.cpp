@@ -269,16 +269,8 @@ stn_status stn_create(const stn_config *cfg, int64_t max_shots, void *cuda_strea
     c->site_off[k + 1] = c->site_off[k] + 2ll * c->chimax[k] * c->chimax[k + 1];
   c->slab_elems = c->site_off[n];
   c->plan = stn::plan_scratch(n, c->chimax.data(), cfg->chi_cap);
-  if (cfg->arena_cap_bytes > 0) {  // shrink the span stacks to the caller's cap
-    const int64_t cap = cfg->arena_cap_bytes / static_cast<int64_t>(c->elem);
-    const int64_t need = c->plan.ap_elems + c->plan.g_elems;
-    if (cap < need) {
-      const double f = static_cast<double>(cap) / static_cast<double>(need);
-      c->plan.ap_elems = static_cast<int64_t>(static_cast<double>(c->plan.ap_elems) * f);
-      c->plan.g_elems = static_cast<int64_t>(static_cast<double>(c->plan.g_elems) * f);
-      c->plan.total = c->plan.ap_elems + c->plan.g_elems + c->plan.work_elems;
-    }
-  }
+  if (cfg->arena_cap_bytes > 0)  // shrink the span stacks to the caller's cap
+    stn::shrink_scratch(c->plan, cfg->arena_cap_bytes / static_cast<int64_t>(c->elem));
   c->svd_elems = stn::round_kernel_svd_elems(cfg->precision, n, c->W);
   if (c->svd_elems < 2 * 4 * c->plan.work_c + 16) {  // the blocked SVD needs two columns
     delete c;

@@ -65,6 +65,8 @@ int svd_smem_elems(int precision) { return precision == 0 ? SvdSmem<double>::ele
 
 // ---------------------------------------------------------------------------
 // host side
+static int64_t align_up(int64_t elems) { return (elems + kScratchAlign - 1) / kScratchAlign * kScratchAlign; }
+
 ScratchPlan plan_scratch(int n, const int *chimax, int chi_cap) {
   ScratchPlan p{};
   int64_t ap = 0, g = 0;
@@ -75,11 +77,21 @@ ScratchPlan plan_scratch(int n, const int *chimax, int chi_cap) {
   (void)chi_cap;
   int64_t c2 = static_cast<int64_t>(cmax) * cmax;
   p.work_c = cmax;
-  p.ap_elems = ap;
-  p.g_elems = g;
-  p.work_elems = 35 * c2 + 4ll * cmax + 1024;
-  p.total = ap + g + p.work_elems;
+  p.ap_elems = align_up(ap);
+  p.g_elems = align_up(g);
+  p.work_elems = align_up(35 * c2 + 4ll * cmax + 1024);
+  p.total = p.ap_elems + p.g_elems + p.work_elems;
   return p;
+}
+
+void shrink_scratch(ScratchPlan &p, int64_t elems) {
+  const int64_t need = p.ap_elems + p.g_elems;
+  if (elems >= need) return;
+  const double f = static_cast<double>(elems) / static_cast<double>(need);
+  auto share = [&](int64_t e) { return static_cast<int64_t>(static_cast<double>(e) * f) / kScratchAlign * kScratchAlign; };
+  p.ap_elems = share(p.ap_elems);
+  p.g_elems = share(p.g_elems);
+  p.total = p.ap_elems + p.g_elems + p.work_elems;
 }
 
 int round_kernel_svd_elems(int precision, int n, int W) {

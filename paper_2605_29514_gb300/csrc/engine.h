@@ -83,7 +83,15 @@ struct ScratchPlan {
   int work_c;
 };
 
+// Per-CTA scratch of complex elements of 8 or 16 bytes.  Every CTA's share and its
+// work area start at multiples of kScratchAlign elements: the complex64 path keeps
+// 16-byte numbers in the work area (svd_small), which an odd bond cap's 35 c^2
+// elements would leave at 8 modulo 16.  Four divides the size of every tensor of a
+// span and of every R factor, so a shrunk stack still holds what it held.
+constexpr int kScratchAlign = 4;
 ScratchPlan plan_scratch(int n, const int *chimax, int chi_cap);
+// Shrinks the span stacks (ap and g together) to at most `elems` elements.
+void shrink_scratch(ScratchPlan &p, int64_t elems);
 size_t round_kernel_smem(int precision, int n, int W, int svd_elems);
 int round_kernel_svd_elems(int precision, int n, int W);
 int jacobi_smem_limit(int precision);
