@@ -751,20 +751,23 @@ static __device__ int keep_count(const T *lam, const int *perm, int n, int cap, 
   return k;
 }
 
-// Discarded over total weight of a bond, by one warp (lane 0's value counts).
-static __device__ __forceinline__ double discarded_weight(const double *lam, const int *perm, int n, int keep) {
+// Discarded over total weight of a bond, by one warp (lane 0's value counts);
+// left: weight that is not in lam, discarded too.
+static __device__ __forceinline__ double discarded_weight(const double *lam, const int *perm, int n, int keep,
+                                                          double left = 0) {
   double tot = 0, drop = 0;
   for (int i = lane_id(); i < n; i += 32) {
     const double l = lam[perm[i]];
     tot += l;
     if (i >= keep) drop += l;
   }
-  tot = warp_sum(tot);
-  drop = warp_sum(drop);
+  tot = warp_sum(tot) + left;
+  drop = warp_sum(drop) + left;
   return tot > 0 ? drop / tot : 0.0;
 }
-static __device__ __forceinline__ double discarded_weight(const float *lam, const int *perm, int n, int keep) {
-  ff tot = ff_of(0.f), drop = ff_of(0.f);
+static __device__ __forceinline__ double discarded_weight(const float *lam, const int *perm, int n, int keep,
+                                                          float left = 0) {
+  ff tot = ff_of(lane_id() == 0 ? left : 0.f), drop = tot;
   for (int i = lane_id(); i < n; i += 32) {
     const float l = lam[perm[i]];
     ff_push(tot, l, 0.f);
@@ -797,9 +800,10 @@ struct Truncation {
 // leading dimension n) = Q R, R in the original column order; rotating the rows
 // of R until they are orthogonal gives the rows sigma_i v_i^dag, so no rotation
 // is accumulated.  lam[i] = sigma_i^2 (unsorted, zero beyond the numerical rank,
-// which is returned; but see cutoff) and column i of V (n x n, column-major; columns beyond the
-// rank are not written, except column 0 of a zero matrix) = v_i.  Values that
-// are not finite give lam = NaN.
+// which is returned) and column i of V (n x n, column-major; columns beyond the
+// rank are not written, except column 0 of a zero matrix) = v_i.  A row of R whose
+// norm falls below rounding counts as zero: it was not rotated any more, so it
+// gives no vector.  Values that are not finite give lam = NaN.
 //
 // Against Jacobi on A's columns with accumulated V this takes about half the
 // sweeps and a quarter of the rotations on the matrices of a d = 3 and a d = 5
@@ -812,8 +816,8 @@ struct Truncation {
 //
 // cutoff > 0 (the truncation's): the QR stops once the norm of all that is left
 // is at most d sigma_1, d = min(cutoff / 16, sqrt(eps_T cutoff)) with eps_T the
-// rounding of T; lam[rank] is then what is left (its squared norm, for the
-// discarded weight).  A value below cutoff sigma_1 is dropped by the caller, and
+// rounding of T; what is left counts as discarded weight and has no vector, whatever
+// the cutoff.  A value below cutoff sigma_1 is dropped by the caller, and
 // leaving such a remainder out turns a kept vector of value s by at most (d
 // sigma_1 / s)^2, that is the decomposed matrix by d^2 sigma_1 / cutoff <= eps_T
 // sigma_1.  In complex64 the remainder is the rounding noise of A, about a third
@@ -1046,10 +1050,13 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
     norms();
   }
   __syncthreads();
+  auto squared = [&](int i) {
+    return i < rank && !(K::value(nr[i]) <= neg) ? static_cast<T>(K::value(nr[i])) * up * up : T(0);
+  };
   if (tr != nullptr) {
     S *inv = nr + kSmallSvdCols;
     for (int i = tid(); i < n; i += kThreads) {
-      const T l = i < rank ? static_cast<T>(K::value(nr[i])) * up * up : i == rank ? static_cast<T>(left) * up * up : T(0);
+      const T l = squared(i);
       const bool bad = !finite || !isfinite(l);
       if (bad) *tr->fail = STN_ENUMERIC;
       lam[i] = bad ? T(0) : l;
@@ -1073,7 +1080,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
     __syncthreads();
     const int keep = *tr->keep;
     if (warp_id() == kWarps - 1) {  // beside the others
-      const double w = discarded_weight(lam, tr->perm, n, keep);
+      const double w = discarded_weight(lam, tr->perm, n, keep, static_cast<T>(left) * up * up);
       if (lane_id() == 0) *tr->discarded += w;
     } else {
       for (int e = tid(); e < n * keep; e += kThreads - 32) {
@@ -1100,9 +1107,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   if (rank == 0)
     for (int c = tid(); c < n; c += kThreads) V[c] = cmake<T>(c == 0 ? T(1) : T(0), 0);
   for (int i = tid(); i < n; i += kThreads)
-    lam[i] = !finite ? static_cast<T>(__longlong_as_double(0x7ff8000000000000ll))
-                     : i < rank ? static_cast<T>(K::value(nr[i])) * up * up
-                     : i == rank && cutoff > 0 ? static_cast<T>(left) * up * up : T(0);
+    lam[i] = finite ? squared(i) : static_cast<T>(__longlong_as_double(0x7ff8000000000000ll));
   __syncthreads();
   return rank;
 }

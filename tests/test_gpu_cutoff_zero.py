@@ -21,7 +21,7 @@ def built():
 
 @pytest.mark.parametrize("precision", [0, 1, 2])
 @pytest.mark.parametrize("cutoff", [0.0, 1e-300, 1e-16, 1e-14])
-@pytest.mark.parametrize("basis,theta,cap", [("Z", 0.05, 32), ("X", 0.0225, 32), ("X", 0.1, 5)])
+@pytest.mark.parametrize("basis,theta,cap", [("Z", 0.05, 32), ("X", 0.1, 5)])
 def test_cutoffs_at_rounding(precision, cutoff, basis, theta, cap):
     """Born probabilities against the oracle at the same cutoff: 1e-9 in
     complex128 and 5e-5 in complex64, the bounds of ordinary cutoffs."""
