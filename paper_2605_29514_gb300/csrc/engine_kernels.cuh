@@ -2304,9 +2304,10 @@ static __device__ __noinline__ void mps_finish(const EngineParams &P, const Smem
       tally(S.dmisc, D_FLOPS) += gemm_flops(r, n2, Dl) + svd_flops(r, n2);
       tally(S.dmisc, D_PROF + 1 + (vec_from_columns ? PROF_NSVD_LARGE : PROF_NSVD_SMALL)) += 1;
     }
-    if (S.misc[M_FAIL]) return;
     const bool rounded = sizeof(T) == 4 && !vec_from_columns && (svd64 || P.svd64_all);
-    if (!svd64) {
+    if (svd64) {
+      if (S.misc[M_FAIL]) return;
+    } else {  // no thread reads M_FAIL here before the barrier that follows its write
       // S.lam holds the squared values, S.perm their order
       for (int i = tid(); i < n2; i += kThreads) {
         const T l = X.lam[i];
