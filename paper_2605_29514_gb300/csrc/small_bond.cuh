@@ -752,22 +752,22 @@ static __device__ int keep_count(const T *lam, const int *perm, int n, int cap, 
 }
 
 // Discarded over total weight of a bond, by one warp (lane 0's value counts);
-// left: weight that is not in lam, discarded too.
+// left: the lane's share of a weight that is not in lam, discarded too.
 static __device__ __forceinline__ double discarded_weight(const double *lam, const int *perm, int n, int keep,
                                                           double left = 0) {
-  double tot = 0, drop = 0;
+  double tot = left, drop = left;
   for (int i = lane_id(); i < n; i += 32) {
     const double l = lam[perm[i]];
     tot += l;
     if (i >= keep) drop += l;
   }
-  tot = warp_sum(tot) + left;
-  drop = warp_sum(drop) + left;
+  tot = warp_sum(tot);
+  drop = warp_sum(drop);
   return tot > 0 ? drop / tot : 0.0;
 }
 static __device__ __forceinline__ double discarded_weight(const float *lam, const int *perm, int n, int keep,
                                                           float left = 0) {
-  ff tot = ff_of(lane_id() == 0 ? left : 0.f), drop = tot;
+  ff tot = ff_of(left), drop = tot;
   for (int i = lane_id(); i < n; i += 32) {
     const float l = lam[perm[i]];
     ff_push(tot, l, 0.f);
@@ -846,7 +846,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   cplx<S> *Bm, *u = in_smem<cplx<S>>(u_);
   if constexpr (SM) Bm = in_smem<cplx<S>>(buf_);
   else Bm = static_cast<cplx<S> *>(buf_);
-  S *nr = in_smem<S>(nr_);
+  S *nr = in_smem<S>(nr_), *rows = nr + kSmallSvdCols;  // squared norms of the columns and of R's rows
   const int gl = lane_id() & (kGroup - 1), g = tid() / kGroup;
   float down = 1.f, up = 1.f;  // ff: the matrix scaled by a power of two to entries up to 1
   if constexpr (sizeof(T) == 4) {
@@ -881,7 +881,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   int rank = 0;
   R neg = 0;    // squared norm of a negligible row
   R rest = 0;   // squared norm of the remainder that may be left out
-  R left = 0;   // bound on the squared norm of the remainder that was
+  R left = 0;   // bound on the squared norm of the remainder that was left out
   bool finite = true;
   {
     const bool spare = team_threads(n) < kThreads;
@@ -1001,7 +1001,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
       if (i < rank)
         for (int c = gl; c < n; c += kGroup) K::sq(s, Bm[c * ld + i]);
       s = group_sum(s);
-      if (gl == 0 && i < rank) nr[i] = s;
+      if (gl == 0 && i < rank) rows[i] = s;
     }
   };
   if (tid() < nthr && finite) {
@@ -1017,7 +1017,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
           if (p > q) { const int t = p; p = q; q = t; }
           bool on = pi < half && q < rank;
           if (!on) p = q = 0;
-          const S al = nr[p], be = nr[q];
+          const S al = rows[p], be = rows[q];
           const R av = K::value(al), bv = K::value(be);
           on = on && av > neg && bv > neg;
           if (!__any_sync(0xffffffffu, on)) continue;
@@ -1038,8 +1038,8 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
             }
             if (gl == 0) {
               const S a1 = K::add(al, K::minus(rot.tg)), b1 = K::add(be, rot.tg);
-              nr[p] = K::value(a1) > 0 ? a1 : K::of(0);
-              nr[q] = K::value(b1) > 0 ? b1 : K::of(0);
+              rows[p] = K::value(a1) > 0 ? a1 : K::of(0);
+              rows[q] = K::value(b1) > 0 ? b1 : K::of(0);
             }
           }
         }
@@ -1051,16 +1051,16 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   }
   __syncthreads();
   auto squared = [&](int i) {
-    return i < rank && !(K::value(nr[i]) <= neg) ? static_cast<T>(K::value(nr[i])) * up * up : T(0);
+    return i < rank && !(K::value(rows[i]) <= neg) ? static_cast<T>(K::value(rows[i])) * up * up : T(0);
   };
   if (tr != nullptr) {
-    S *inv = nr + kSmallSvdCols;
+    S *inv = rows;  // then their reciprocal roots
     for (int i = tid(); i < n; i += kThreads) {
       const T l = squared(i);
       const bool bad = !finite || !isfinite(l);
       if (bad) *tr->fail = STN_ENUMERIC;
       lam[i] = bad ? T(0) : l;
-      if (i < rank) inv[i] = K::value(nr[i]) > 0 ? K::rsqrt(nr[i]) : K::of(0);
+      if (i < rank) inv[i] = K::value(rows[i]) > 0 ? K::rsqrt(rows[i]) : K::of(0);
     }
     __syncthreads();
     for (int i = g; (i & ~3) < n; i += kGroups) {  // decreasing order, ties by index
@@ -1080,7 +1080,10 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
     __syncthreads();
     const int keep = *tr->keep;
     if (warp_id() == kWarps - 1) {  // beside the others
-      const double w = discarded_weight(lam, tr->perm, n, keep, static_cast<T>(left) * up * up);
+      R share = 0;  // what was left: the columns without a pivot, whose norms the Jacobi has not touched
+      if (left > 0)
+        for (int c = lane_id(); c < n; c += 32) share += max(K::value(nr[c]), R(0));
+      const double w = discarded_weight(lam, tr->perm, n, keep, static_cast<T>(share) * up * up);
       if (lane_id() == 0) *tr->discarded += w;
     } else {
       for (int e = tid(); e < n * keep; e += kThreads - 32) {
@@ -1099,7 +1102,7 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   }
   for (int e = tid(); e < n * rank; e += kThreads) {
     const int i = e / n, c = e % n;
-    const S s = nr[i];
+    const S s = rows[i];
     const cplx<S> x = Bm[c * ld + i];
     const S inv = K::value(s) > 0 ? K::rsqrt(s) : K::of(0);
     V[e] = cmake<T>(static_cast<T>(K::value(K::mul(x.re, inv))), static_cast<T>(-K::value(K::mul(x.im, inv))));
