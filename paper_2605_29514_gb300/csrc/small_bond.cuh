@@ -245,7 +245,8 @@ __device__ __forceinline__ void reflector_scaled(cplx<double> al, double nx2, cp
   }
 }
 // Reflector of the column x[j..m-1] (elements `stride` apart) in the storage
-// precision T.  A column of norm up to 1e-30 gets none (sc = 0).  Norm and scalars
+// precision T.  A column of norm up to 1e-30 gets none (sc = 0), one that is not
+// finite gets a NaN on the diagonal.  Norm and scalars
 // in double, or for float in ff; for float on the column times the power of two
 // `down`: single-precision squares of entries near 1e-20 would be denormal, and a
 // reflector built from such a norm not unitary.  `unit` makes it P = I - 2 u u^dag
@@ -267,7 +268,7 @@ __device__ __forceinline__ Reflector<double> column_reflector(const cplx<double>
   for (int i = j + lane_id(); i < m; i += 32) Work<double>::sq(s, col[i * stride]);
   s = lane_sum<double>(s, 16);
   Reflector<double> h{cmake<double>(0, 0), 0.0, 1.0, 1.0};
-  if (s > 1e-60) reflector_scaled(col[j * stride], s, h.gam, h.sc);
+  if (!(s <= 1e-60)) reflector_scaled(col[j * stride], s, h.gam, h.sc);  // a NaN goes on into gam
   if (unit) h.sc *= 0.70710678118654752440;
   return h;
 }
@@ -278,9 +279,10 @@ __device__ __forceinline__ Reflector<double> column_reflector(const cplx<double>
 // Adding a constant with the step as its last place rounds a square to the step,
 // and the integer is the difference of the bit patterns.
 __device__ __forceinline__ ff column_norm2(const cplx<float> *col, int stride, int j, int m, int &ex) {
-  float mx = 0.f;
-  for (int i = j + lane_id(); i < m; i += 32) mx = fmaxf(mx, fmaxf(fabsf(col[i * stride].re), fabsf(col[i * stride].im)));
-  const int bits = __reduce_max_sync(0xffffffffu, __float_as_int(mx));
+  int bits = 0;  // of the largest component: infinity and, above it, NaN among them
+  for (int i = j + lane_id(); i < m; i += 32)
+    bits = max(bits, max(__float_as_int(fabsf(col[i * stride].re)), __float_as_int(fabsf(col[i * stride].im))));
+  bits = __reduce_max_sync(0xffffffffu, bits);
   ex = min(253, max(1, bits >> 23));
   const float down = __int_as_float((254 - ex) << 23);
   if (m > 1024) {
@@ -309,7 +311,9 @@ __device__ __forceinline__ ff column_norm2(const cplx<float> *col, int stride, i
   const int th = __reduce_add_sync(0xffffffffu, hi), tl = __reduce_add_sync(0xffffffffu, lo);
   ff s = ff_norm(ff{static_cast<float>(th & ~4095) * step1, static_cast<float>(th & 4095) * step1});
   s.l = fmaf(static_cast<float>(tl), step2, s.l);
-  return ff_norm(s);
+  s = ff_norm(s);
+  if (bits >= 0x7f800000) s.h = __int_as_float(bits);  // the integers say nothing then
+  return s;
 }
 __device__ __forceinline__ Reflector<float> column_reflector(const cplx<float> *col, int stride, int j, int m,
                                                              bool unit) {
@@ -378,7 +382,7 @@ __device__ __forceinline__ void column_head(cplx<double> *col, int j, int m, Col
   s = __shfl_sync(0xffffffffu, s, 0);
   cplx<double> al = col[j];
   ColumnHead<double> r{cmake<double>(0, 0), cmake<double>(0, 0), 0.0, 0.0};
-  if (s > 1e-60) {
+  if (!(s <= 1e-60)) {
     double up = 1.0;
     if (s > 1e130) {
       const int ex = min(2045, max(1, (__double2hiint(s) >> 21) + 512));  // half the exponent of s, biased
