@@ -65,6 +65,23 @@ cudaError_t launch_gemm(int ta, int tb, int m, int n, int k, const void *A, cons
   return cudaGetLastError();
 }
 
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1) qr_kernel(bool conj_t, int m, int n, const cplx<T> *A, cplx<T> *R,
+                                                         cplx<T> *Q) {
+  extern __shared__ __align__(16) char smem_raw[];
+  qr_small<T>(m, n, A, conj_t ? m : n, conj_t, R, min(m, n), Q, reinterpret_cast<cplx<T> *>(smem_raw));
+}
+
+template <typename T>
+cudaError_t launch_qr(int conj_t, int m, int n, const void *A, void *R, void *Q) {
+  const size_t smem = sizeof(cplx<T>) * qr_small_elems(m, n, Q != nullptr);
+  cudaError_t e = cudaFuncSetAttribute(qr_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  qr_kernel<T><<<1, kThreads, smem>>>(conj_t != 0, m, n, static_cast<const cplx<T> *>(A), static_cast<cplx<T> *>(R),
+                                      static_cast<cplx<T> *>(Q));
+  return cudaGetLastError();
+}
+
 __device__ ff split(double x) {
   const float h = static_cast<float>(x);
   return ff_norm(ff{h, static_cast<float>(x - h)});
@@ -110,6 +127,9 @@ int check_svd(int precision, int shared, int m, int n, const void *A, void *V, v
 int check_gemm(int precision, int ta, int tb, int m, int n, int k, const void *A, const void *B, void *C) {
   return precision == 0 ? stn::launch_gemm<double>(ta, tb, m, n, k, A, B, C)
                         : stn::launch_gemm<float>(ta, tb, m, n, k, A, B, C);
+}
+int check_qr(int precision, int conj_t, int m, int n, const void *A, void *R, void *Q) {
+  return precision == 0 ? stn::launch_qr<double>(conj_t, m, n, A, R, Q) : stn::launch_qr<float>(conj_t, m, n, A, R, Q);
 }
 int check_math(int what, int count, const double *x, double *y) {
   stn::math_kernel<<<(count + 255) / 256, 256>>>(what, count, x, y);

@@ -66,3 +66,14 @@ def test_rows_have_householder_phases(precision, m, n):
         ref[j:, j:] -= 2 * np.outer(x, x.conj() @ ref[j:, j:])
         ref[j + 1:, j] = 0
     assert np.all(np.abs(r[:n] - ref[:n]).max(axis=1) < bound)
+
+
+@pytest.mark.parametrize("m,n", [(5, 3), (40, 20), (60, 50), (100, 70), (140, 100), (160, 150)])
+def test_r_without_q_is_r_with_q(m, n):
+    """Complex64: the same R to the last bit with and without Q, at sizes whose
+    columns fit shared memory with Q, without it only, or not at all."""
+    a = graded(np.random.default_rng(m + n), m, n, 1)
+    k = min(m, n)
+    b, q, work = torch.tensor(a, device="cuda"), *(torch.zeros(m, k, dtype=CDT[1], device="cuda") for _ in "qw")
+    stn.dense_qr_q(1, m, n, b.data_ptr(), q.data_ptr(), work.data_ptr())
+    assert np.array_equal(r_factor(1, a), b.cpu().numpy())

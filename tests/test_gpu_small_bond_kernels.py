@@ -1,6 +1,6 @@
 """The routines of small bonds alone, for both CTA sizes: the SVD of the
 truncation in double precision and in pairs of floats, with its matrix in shared
-and in global memory; the contraction by one CTA; the roots and reciprocals.
+and in global memory; the QR; the contraction by one CTA; the roots and reciprocals.
 References are numpy in float64.
 
 Bounds: 64 eps sqrt(m n) of the working precision (1.1e-16; 1.4e-14 for pairs of
@@ -173,6 +173,37 @@ def test_zero_and_non_finite(libs, precision, shared, value):
         assert np.array_equal(v[:, 0], np.eye(6)[0])
     else:
         assert not np.any(np.isfinite(lam)) and fail != 0
+
+
+@pytest.mark.parametrize("threads", [256, 512])
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("conj_t", [False, True])
+@pytest.mark.parametrize("m,n", [(1, 1), (1, 5), (5, 1), (2, 3), (4, 5), (16, 63), (40, 20), (66, 64), (63, 65), (128, 30),
+                                 (129, 30), (60, 70), (2, 400)])
+@pytest.mark.parametrize("scales", [(1.0,), (1.0, 1e-12, 1e12, 1e-25)])
+def test_qr(libs, threads, precision, conj_t, m, n, scales):
+    """R and Q of the shared-memory QR, of the matrix or its conjugate transpose as
+    stored, with a zero column and with columns far from one: relative to the
+    columns' norms, 64 roundings of the precision times sqrt(size)."""
+    rng = np.random.default_rng(31 * m + n)
+    size = np.array([scales[c % len(scales)] for c in range(n)])
+    a = ((rng.normal(size=(m, n)) + 1j * rng.normal(size=(m, n))) * size).astype(NP[precision])
+    a[:, n // 2] = 0
+    k = min(m, n)
+    given = torch.tensor(np.ascontiguousarray(a.conj().T) if conj_t else a, device="cuda")
+    r, r2 = (torch.full((k, n), 7.0, dtype=CDT[precision], device="cuda") for _ in range(2))
+    q = torch.full((k, m) if conj_t else (m, k), 7.0, dtype=CDT[precision], device="cuda")
+    assert libs[threads].check_qr(precision, int(conj_t), m, n, ptr(given), ptr(r), ptr(q)) == 0
+    assert libs[threads].check_qr(precision, int(conj_t), m, n, ptr(given), ptr(r2), None) == 0
+    assert torch.equal(r, r2)
+    r, q = (x.cpu().numpy().astype(np.complex128) for x in (r, q))
+    q = q.conj().T if conj_t else q
+    unit = a.astype(np.complex128) / size
+    norm = np.maximum(np.linalg.norm(unit, axis=0), 1e-3)
+    bound = 64 * (1.1e-16 if precision == 0 else 6e-8) * np.sqrt(m * n)
+    assert np.all(np.tril(r, -1) == 0)
+    assert np.abs(q.conj().T @ q - np.eye(k)).max() < bound
+    assert (np.abs(q @ (r / size) - unit).max(axis=0) / norm).max() < bound
 
 
 @pytest.mark.parametrize("threads", [256, 512])
