@@ -3009,6 +3009,16 @@ __host__ __device__ __forceinline__ bool qr_alone_small(int m, int n, bool with_
   return sizeof(T) == 8 && qr_small_elems(m, n, with_q) <= SvdSmem<T>::elems;
 }
 
+// Whether qr_small takes the entries of a caller's complex128 matrix.  CTA-wide.
+template <typename T>
+static __device__ __forceinline__ bool in_small_range(int count, const cplx<T> *A) {
+  bool large = false;
+  if constexpr (sizeof(T) == 8)
+    for (int e = tid(); e < count; e += kThreads)
+      large |= max(__double2hiint(A[e].re) & 0x7fffffff, __double2hiint(A[e].im) & 0x7fffffff) >= (1023 + 300) << 20;
+  return !__syncthreads_or(large);
+}
+
 // Which calls a cluster takes.
 template <typename T>
 static bool shares_svd(int m, int n) {
@@ -3031,12 +3041,12 @@ __global__ void __launch_bounds__(kThreads, 1) dense_check_kernel(int what, int 
   double *red = s.red;
   int *flag = s.flag;
   if (what == 0) {
-    if (qr_alone_small<T>(m, n, false)) qr_small<T>(m, n, A, n, false, A, m, nullptr, buf);
+    if (qr_alone_small<T>(m, n, false) && in_small_range(m * n, A)) qr_small<T>(m, n, A, n, false, A, m, nullptr, buf);
     else qr_r_inplace<T>(m, n, A, n, buf, SvdSmem<T>::elems);
   } else if (what == 2) {
     // explicit Q of the gauge steps: reflectors kept in sig2's buffer
     cplx<T> *vstore = reinterpret_cast<cplx<T> *>(sig2);
-    if (qr_alone_small<T>(m, n, true)) {
+    if (qr_alone_small<T>(m, n, true) && in_small_range(m * n, A)) {
       qr_small<T>(m, n, A, n, false, A, m, V, buf);
       const int ld = m | 1, steps = min(m, n);
       const ColumnHead<T> *head = reinterpret_cast<const ColumnHead<T> *>(buf + n * ld);

@@ -483,6 +483,10 @@ __device__ __forceinline__ cplx<T> dot_below(const cplx<T> *x, const cplx<T> *b,
 // (which keep the reflectors' rows below the diagonal), the reflectors' heads,
 // then Q.  CTA-wide.
 //
+// The vectors are not normalised, so v^dag b is a product of two columns' sizes:
+// entries have to stay below 2^60 in complex64 and 2^300 in complex128, as those of
+// a state do.
+//
 // What bounds a column is a chain: its norm, a root and a reciprocal (about 600
 // cycles for ff, 1400 for double, whose operations take 64 each), then the
 // update.  One warp that owns no column runs the chain while the others form

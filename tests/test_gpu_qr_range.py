@@ -54,3 +54,18 @@ def test_columns_that_would_overflow_together(precision, scales, m, n):
     assert (np.abs(q @ (b[:k] / size) - unit).max(axis=0) / norm).max() < bound
     for x in (r / size, b / size):
         assert (np.abs(x.conj().T @ x - unit.conj().T @ unit) / np.outer(norm, norm)).max() < bound
+
+
+@pytest.mark.parametrize("m,n", [(1, 2), (2, 5), (20, 41), (60, 130)])
+def test_wide_columns_of_another_size(m, n):
+    """Complex128: columns that get no reflector may have squares out of range."""
+    rng = np.random.default_rng(m)
+    size = np.where(np.arange(n) < m, 1e60, 1e250)
+    unit = rng.normal(size=(m, n)) + 1j * rng.normal(size=(m, n))
+    b = torch.tensor(unit * size, device="cuda")
+    r, q, work = b.clone(), *(torch.zeros(m, m, dtype=CDT[0], device="cuda") for _ in "qw")
+    stn.dense_qr(0, m, n, r.data_ptr())
+    stn.dense_qr_q(0, m, n, b.data_ptr(), q.data_ptr(), work.data_ptr())
+    bound = 64 * 2.2e-16 * np.sqrt(m * n) * np.linalg.norm(unit, axis=0)
+    for x in (r, b):
+        assert np.all(np.abs(q.cpu().numpy() @ (x.cpu().numpy() / size) - unit).max(axis=0) < bound)
