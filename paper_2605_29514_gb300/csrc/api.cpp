@@ -23,6 +23,7 @@ struct stn_ctx {
   int n = 0, W = 0, rec_bytes = 0, K = 0, grid = 1, svd_elems = 0;
   bool light = false;                 // the round and adjoint kernels of 256 threads
   int sms = 1, light_grid = 0, light_elems = 0;
+  int scratch_ctas = 0;               // CTAs whose scratch stn_create allocated
   std::vector<int> chimax;
   std::vector<int64_t> site_off;
   int64_t slab_elems = 0;
@@ -341,6 +342,7 @@ stn_status stn_create(const stn_config *cfg, int64_t max_shots, void *cuda_strea
       c->light_grid = c->grid;
     }
     if (!got) A(dalloc(c, &c->d_scratch, per_cta * c->grid));
+    c->scratch_ctas = c->light ? c->light_grid : c->grid;
   }
   if (!ok) {
     stn_destroy(c);
@@ -750,25 +752,24 @@ stn_status stn_sample_shots(stn_ctx *c, int64_t shots, uint64_t shot_offset, con
   return stn_read_records(c, h_records, h_born, h_stats);
 }
 
-// Gives back the scratch of the second CTA per SM, for a call that needs the
-// memory; a captured graph holds its address, so then it stays.
-static bool drop_second_scratch(stn_ctx *c) {
-  if (c->light_grid <= c->grid || !c->light || c->graph) return false;
+// Replaces the scratch by that of `ctas` CTAs.  A captured graph holds its
+// address, so then it stays, as it does where the new one cannot be allocated.
+static bool resize_scratch(stn_ctx *c, int ctas) {
+  if (!c->light || c->graph || c->light_grid == ctas) return false;
   if (cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
   void *old = c->d_scratch;
-  if (dalloc(c, &c->d_scratch, c->elem * static_cast<size_t>(c->plan.total) * c->grid) != cudaSuccess) {
+  if (dalloc(c, &c->d_scratch, c->elem * static_cast<size_t>(c->plan.total) * ctas) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  c->light_grid = c->grid;
+  c->light_grid = ctas;
   c->allocs.erase(std::find(c->allocs.begin(), c->allocs.end(), old));
   cudaFree(old);
   return true;
 }
 
-stn_status stn_logprob_grad(stn_ctx *c, uint64_t shot_offset, int64_t n_rec, const uint8_t *h_records,
-                            const double *h_theta, double *h_logp, double *h_grad) {
-  if (!c) return STN_EINVAL;
+static stn_status logprob_grad(stn_ctx *c, uint64_t shot_offset, int64_t n_rec, const uint8_t *h_records,
+                               const double *h_theta, double *h_logp, double *h_grad) {
   if (n_rec < 1 || n_rec > c->max_shots || !h_records || !h_logp || !h_grad || (!h_theta && c->K > 0))
     return fail(c, STN_EINVAL, "stn_logprob_grad: bad argument");
   for (int k = 0; k < c->K; ++k)
@@ -781,7 +782,9 @@ stn_status stn_logprob_grad(stn_ctx *c, uint64_t shot_offset, int64_t n_rec, con
   const size_t phi_bytes = c->elem * static_cast<size_t>(n_rec) * std::max(1, n_rot) * c->slab_elems;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return cuda_fail(c, cudaGetLastError(), "memory info");
-  if (phi_bytes > free_b / 10 * 8 && drop_second_scratch(c) && cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
+  // without the second CTA's scratch per SM, where the call needs the memory
+  if (phi_bytes > free_b / 10 * 8 && c->light_grid > c->grid && resize_scratch(c, c->grid) &&
+      cudaMemGetInfo(&free_b, &total_b) != cudaSuccess)
     return cuda_fail(c, cudaGetLastError(), "memory info");
   if (phi_bytes > free_b / 10 * 8)
     return fail(c, STN_ENOMEM, "stn_logprob_grad: the states after every rotation do not fit device memory");
@@ -834,6 +837,14 @@ stn_status stn_logprob_grad(stn_ctx *c, uint64_t shot_offset, int64_t n_rec, con
   e = cudaMemcpy(h_grad, d_grad, sizeof(double) * c->K, cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(c, e, "stn_logprob_grad grad");
   return STN_OK;
+}
+
+stn_status stn_logprob_grad(stn_ctx *c, uint64_t shot_offset, int64_t n_rec, const uint8_t *h_records,
+                            const double *h_theta, double *h_logp, double *h_grad) {
+  if (!c) return STN_EINVAL;
+  const stn_status st = logprob_grad(c, shot_offset, n_rec, h_records, h_theta, h_logp, h_grad);
+  if (c->light) resize_scratch(c, c->scratch_ctas);  // two CTAs per SM again for the batches that follow
+  return st;
 }
 
 stn_status stn_dense_qr_q(int32_t precision, int32_t m, int32_t n, void *d_b, void *d_q, void *d_work,
