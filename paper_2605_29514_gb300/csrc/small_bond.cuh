@@ -753,8 +753,8 @@ static __device__ int keep_count(const T *lam, const int *perm, int n, int cap, 
     k = max(1, above(n, cutoff * cutoff * l1));
   }
   if (k > cap) {
-    const double thr = sqrt(at(cap)) + delta * sqrt(l1);
-    k = max(1, above(cap, thr * thr));
+    const double c = at(cap);  // (sqrt(c) + delta sqrt(l1))^2, and c itself at delta = 0
+    k = max(1, above(cap, c + delta * (2.0 * sqrt(c * l1) + delta * l1)));
   }
   return k;
 }

@@ -1,7 +1,7 @@
 // Kernels that call the routines of small bonds alone (small_bond.cuh and the
 // contraction of engine_kernels.cuh), compiled by test_gpu_small_bond_kernels.py
 // for either CTA size (STN_CTA_THREADS).  All pointers are device memory; every
-// launch is one CTA (check_heads: a warp per element).
+// launch is one CTA (check_keep: a warp, check_heads: one per element).
 #include "engine_kernels.cuh"
 
 STN_BEGIN
@@ -82,6 +82,12 @@ cudaError_t launch_qr(int conj_t, int m, int n, const void *A, void *R, void *Q)
   return cudaGetLastError();
 }
 
+template <typename T>
+__global__ void keep_kernel(const T *lam, const int *perm, int n, int cap, double cutoff, double delta, int *out) {
+  const int k = keep_count<T>(lam, perm, n, cap, cutoff, delta);
+  if (threadIdx.x == 0) *out = k;
+}
+
 __device__ ff split(double x) {
   const float h = static_cast<float>(x);
   return ff_norm(ff{h, static_cast<float>(x - h)});
@@ -130,6 +136,11 @@ int check_gemm(int precision, int ta, int tb, int m, int n, int k, const void *A
 }
 int check_qr(int precision, int conj_t, int m, int n, const void *A, void *R, void *Q) {
   return precision == 0 ? stn::launch_qr<double>(conj_t, m, n, A, R, Q) : stn::launch_qr<float>(conj_t, m, n, A, R, Q);
+}
+int check_keep(int precision, const void *lam, const int *perm, int n, int cap, double cutoff, double delta, int *out) {
+  if (precision == 0) stn::keep_kernel<double><<<1, 32>>>(static_cast<const double *>(lam), perm, n, cap, cutoff, delta, out);
+  else stn::keep_kernel<float><<<1, 32>>>(static_cast<const float *>(lam), perm, n, cap, cutoff, delta, out);
+  return cudaGetLastError();
 }
 int check_math(int what, int count, const double *x, double *y) {
   stn::math_kernel<<<(count + 255) / 256, 256>>>(what, count, x, y);

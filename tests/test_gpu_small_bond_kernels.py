@@ -1,6 +1,6 @@
 """The routines of small bonds alone, for both CTA sizes: the SVD of the
 truncation in double precision and in pairs of floats, with its matrix in shared
-and in global memory; the QR; the contraction by one CTA; the roots and reciprocals.
+and in global memory; the QR; the keep rule; the contraction by one CTA; the roots and reciprocals.
 References are numpy in float64.
 
 Bounds: 64 eps sqrt(m n) of the working precision (1.1e-16; 1.4e-14 for pairs of
@@ -158,6 +158,24 @@ def test_weight_of_the_remainder(libs, threads, precision, small, kept, m, n):
     _, _, _, keep, disc, fail = svd(libs[threads], precision, True, a, 1e-3, n)
     assert fail == 0 and keep == kept
     assert disc == pytest.approx(weight / (kept + weight), rel=1e-5, abs=0)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("delta", [0.0, 1e-3])
+def test_keep_count(libs, precision, delta):
+    """The keep rule on squared values: those above the cutoff, and at most the cap
+    of them that exceed the first dropped one by more than delta sigma_1.  Of equal
+    values on both sides of the cap none is kept, whatever their size."""
+    rng = np.random.default_rng(3)
+    for trial in range(200):
+        s = rng.uniform(0.1, 0.9)
+        lam = np.array([1.0, s, s, s, s * s, 1e-12] + [0.0] * (trial % 60)).astype([np.float64, np.float32][precision])
+        dl, out = torch.tensor(lam, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+        perm = torch.arange(len(lam), dtype=torch.int32, device="cuda")
+        for cap, want in ((1, 1), (2, 1), (3, 1), (4, 4), (5, 5), (6, 5), (len(lam) + 1, 5)):
+            assert libs[512].check_keep(precision, ptr(dl), ptr(perm), len(lam), cap, ctypes.c_double(1e-5),
+                                        ctypes.c_double(delta), ptr(out)) == 0
+            assert out.item() == want
 
 
 @pytest.mark.parametrize("precision", [0, 1])
