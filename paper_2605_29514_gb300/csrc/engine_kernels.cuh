@@ -2050,6 +2050,7 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
   }
   // doubled bond dimensions D[k] for bonds a..b+1
   auto Dbond = [&](int k) { return (k > sp.lo && k <= sp.hi) ? 2 * chi[k] : chi[k]; };
+  __syncthreads();  // the callers have read M_FAIL, which may be written here
   if (tid() == 0) {
     int64_t o = 0;
     for (int k = a; k <= b; ++k) {

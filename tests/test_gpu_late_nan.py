@@ -38,3 +38,18 @@ def test_non_finite_bond_is_reported(precision, cap, cutoff):
     again = sim.sample_shots(2, 0, theta)
     assert np.array_equal(again["records"], want["records"]) and np.array_equal(again["born"], want["born"])
     sim.close()
+
+
+@pytest.mark.parametrize("arena", [1, 4096, 16384, 65536])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_arena_that_is_too_small_is_reported(precision, arena):
+    """Sweeps that outgrow the span stacks at different points of the program."""
+    w = D3_EXACT.with_(rounds=1, p=0.0, theta=0.1, memory_basis="X", precision=precision, svd_cutoff=5e-6,
+                       degeneracy_tol=5e-6)
+    sim = stn.Simulator(w, max_shots=200, arena_cap_bytes=arena)
+    theta = theta_table(w, sim.n_pairs)
+    with pytest.raises(stn.StnError) as e:
+        sim.sample_shots(200, 0, theta)
+    assert e.value.status == stn.STN_EOVERFLOW
+    assert np.all(sim.sample_shots(200, 0, np.zeros_like(theta))["max_chi"] == 1) if arena > 4096 else True
+    sim.close()
