@@ -346,9 +346,10 @@ stn_status stn_philox_uniforms(uint64_t seed, uint64_t shot_offset, int64_t n_sh
                                void *cuda_stream);
 
 /* Dense building blocks of the truncation sweep (Sec. IV B, Eq. 8), run alone:
- * on one CTA, or, for R factors past its shared memory and SVDs (in_shared = 3)
- * of 48 columns and more, on a cluster of eight.  precision: STN_PRECISION_*; complex elements are
- * interleaved (re, im) of that precision, all device memory.
+ * on one CTA, or, from 48 columns (the smaller of m and n) on, SVDs with
+ * in_shared = 3, complex64 R factors and those complex128 ones that do not fit
+ * its shared memory on a cluster of eight.  precision: STN_PRECISION_*; complex
+ * elements are interleaved (re, im) of that precision, all device memory.
  * stn_dense_qr: Householder QR of d_b (m x n, row-major, m <= 1024), in
  *   place; rows 0..min(m,n)-1 then hold R, the rest is zero.  Row j has the
  *   phase -x_j / |x_j| of its reflected column x, known to eps ||x|| / |x_j|;
@@ -416,8 +417,9 @@ stn_status stn_dense_gemm_tc(int32_t m, int32_t n, int32_t k, const float *d_a, 
                              int32_t *d_status, void *cuda_stream);
 
 /* The complex contraction of the MPS sweeps (R_k A'_k, C = R_k M_k,
- * M_k V_keep, A'_{k-1} W, the transfer products; Sec. IV A-B) alone on one
- * CTA, through the same device routine the round kernel calls:
+ * M_k V_keep, A'_{k-1} W, the transfer products; Sec. IV A-B) alone, through the
+ * same device routine the round kernel calls (on the CUDA cores a CTA per block of
+ * the output, so C must not overlap A or B):
  *   C = alpha op(A) op(B) + beta C
  * row-major complex of the precision (0: complex128, 1: complex64; device
  * memory), op = identity (0) or conjugate transpose (1), op(A) m x k, op(B)

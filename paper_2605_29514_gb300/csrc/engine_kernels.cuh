@@ -515,8 +515,8 @@ static __device__ __noinline__ void cgemm_tc(int M, int N, int K, cplx<float> al
 // / N), so a row of B is read once for U products and nothing is padded.  The
 // shared-memory tiles below round every product up to 64 x 64 x 16.  For an
 // 8 x 8 x 8 complex128 product that is 128 times its arithmetic, on a pipe of
-// two FP64 FMAs a clock: 68 us in tiles, 8 us here (of which 8 the launch);
-// 200^3 takes 13.4 ms in tiles and 8.3 ms here, so complex128 always comes
+// two FP64 FMAs a clock: 68 us in tiles, 8 us here, which is the launch's time;
+// by one CTA 200^3 takes 13.4 ms in tiles and 8.3 ms here, so complex128 always comes
 // here (N <= 512 in a sweep; a wider product runs in tiles).  In complex64 the
 // tiles' arithmetic is cheap but their barriers are not: up to 2^16 products
 // the direct form is faster (one d = 5 round at cap 32: 439 ms in tiles, 406
@@ -1857,6 +1857,8 @@ static __device__ Scratch<T> scratch_for(const EngineParams &P, int cap) {
 // factor of an m x n matrix 4 (2 m n^2 - 2 n^3 / 3) with m >= n, the
 // singular values and the vectors of the smaller side of an m x n matrix
 // 4 (4 m n^2 + 8 n^3) with m >= n (roles swapped otherwise in both).
+// An R factor counts also where the matrix is its own R and none is computed: the
+// count is the algorithm's, and stays comparable.
 // In thirds of a flop: thread 0 counts in integers, since a double-precision
 // operation takes 64 cycles and these were 40 a bond, of about 70,000 cycles.
 static __device__ __forceinline__ long long gemm_flops(int M, int N, int K) { return 24ll * M * N * K; }
@@ -2071,8 +2073,8 @@ static __device__ __noinline__ double mps_prepare(const EngineParams &P, const S
   // Doubled sites: one of up to kWarpSite elements by a warp, the span's sites
   // in parallel (a site's tensor is a chain of index arithmetic and two loads:
   // 5000 cycles, which the whole CTA would spend per site); a larger one by
-  // the CTA.  The span is the operator's support, so a <= lo <= hi <= b hold with
-  // equality.
+  // the CTA.  (With 256 or 4096 elements for 1024 the workloads measured stay within 1 %.)
+  // The span is the operator's support, so a <= lo <= hi <= b hold with equality.
   constexpr int kWarpSite = 1024;
   for (int pass = 0; pass < 2; ++pass) {
     for (int k = pass == 0 ? a + warp_id() : a; k <= b; k += pass == 0 ? kWarps : 1) {
@@ -2938,12 +2940,15 @@ static __device__ void svd_bond(int m, int n, const cplx<T> *A, cplx<T> *work, c
 // One CTA left the GPU idle: its block pairs take turns although a round's are
 // disjoint.  Eight CTAs (the portable limit) have a block pair of 16 + 16 columns
 // each up to 256 columns, and in complex128 blocks of a sixteenth of the columns.
-// One CTA against eight: a 256 x 192 complex64 SVD 23.2 and 4.67 ms, 60 x 50 2.40
-// and 1.18 ms; complex128 128 x 128 98 and 10.8 ms, 72 x 66 (svd_small on one CTA,
-// bound by its SM's FP64 rate) 7.4 and 4.6 ms; the R factor of
-// 512 x 250 in complex64 4.0 and 1.36 ms, of 200 x 100 in complex128 4.5 and 1.8 ms.
+// The same code on one CTA and on eight: a 256 x 192 complex64 SVD 21.8 and 4.57 ms,
+// 60 x 50 2.07 and 1.16 ms; complex128 128 x 128 58 and 10.6 ms, 72 x 66 (svd_small on
+// one CTA, bound by its SM's FP64 rate) 7.3 and 4.3 ms; the R factor of 512 x 250 in
+// complex64 2.76 and 1.37 ms, of 200 x 100 in complex128 3.8 and 1.8 ms.
+// From 48 columns on: 64 x 48 takes 2.65 and 2.33 ms in complex128 and 1.26 and 1.05 ms
+// in complex64; 52 x 40 1.66 and 1.83 ms in complex128 (1.10 and 0.97 ms in complex64,
+// which could start lower: 40 x 32 0.57 and 0.49 ms).
 constexpr int kShareCtas = 8;
-constexpr int kShareMinCols = 48;  // below, block pairs are too few or too small
+constexpr int kShareMinCols = 48;
 
 struct DenseSmem {
   double *red;
@@ -3146,7 +3151,8 @@ cudaError_t launch_dense_gemm_t(int ta, int tb, int m, int n, int k, const doubl
   const bool tc = sizeof(T) == 4 && use_tc;
   auto tiles = [&](int b) { return dim3((m + b - 1) / b, (n + b - 1) / b); };
   int block = tc ? (m > n ? m : n) : 32;
-  if (!tc && tiles(32).x * tiles(32).y < 152) block = 16;
+  constexpr unsigned kSms = 152;
+  if (!tc && tiles(32).x * tiles(32).y < kSms) block = 16;
   dense_gemm_kernel<T><<<tiles(block), kThreads, smem, s>>>(ta, tb, m, n, k, al, static_cast<const cplx<T> *>(A), lda,
                                                  static_cast<const cplx<T> *>(B), ldb, be, static_cast<cplx<T> *>(C),
                                                  ldc, use_tc, status, block);

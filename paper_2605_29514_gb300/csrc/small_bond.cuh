@@ -331,7 +331,9 @@ __device__ __forceinline__ Reflector<float> column_reflector(const cplx<float> *
   return h;
 }
 
-// 1 / x of a normal x to the rounding of T
+// 1 / x of a normal x: the hardware's approximation r and, with e = 1 - x r, the
+// geometric series r (1 + e + ...) to e^2 for double, to e for the float of a pair;
+// within one unit in the last place.
 __device__ __forceinline__ double reciprocal(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -448,7 +450,7 @@ __device__ __forceinline__ void head_scaled(cplx<ff> al, ff nx2, cplx<ff> *out) 
   head_scalars<ff>(cmake<ff>(times(al.re, f), times(al.im, f)), times(times(nx2, f), f), v0, gam, h);
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h.h));
-  const float e1 = fmaf(-h.l, r, fmaf(-h.h, r, 1.f));
+  const float e1 = fmaf(-h.l, r, fmaf(-h.h, r, 1.f));  // the same series, to e^2, as a pair
   const ff beta = ff_norm(ff{r, r * fmaf(e1, e1, e1)});
   if (lane_id() == 0) {
     out[0] = cmake<ff>(times(v0.re, g), times(v0.im, g));
