@@ -117,9 +117,10 @@ struct Work<double> {
   static constexpr double eps = 1.11e-16, tiny2 = 1e-32;
   static __device__ __forceinline__ double minus(double x) { return -x; }
   static __device__ __forceinline__ double scale(double x, float) { return x; }
-  static __device__ __forceinline__ int key(double x, int c) {  // column in the low bits, order of the high words
+  // order of the high words, then (low bits) the lower column first
+  static __device__ __forceinline__ int key(double x, int c) {
     const int hi = __double2hiint(x);
-    return hi < 0 ? -1 : ((hi & ~127) | c);
+    return hi < 0 ? -1 : ((hi & ~127) | (127 - c));
   }
   static constexpr int key_infinite = 0x7ff00000;
   static __device__ __forceinline__ double infinite() { return __longlong_as_double(0x7ff0000000000000ll); }
@@ -151,7 +152,7 @@ struct Work<ff> {
   static __device__ __forceinline__ ff scale(float x, float sc) { return ff_of(x * sc); }
   static __device__ __forceinline__ int key(ff x, int c) {
     const int b = __float_as_int(x.h);
-    return b < 0 ? -1 : ((b & ~127) | c);
+    return b < 0 ? -1 : ((b & ~127) | (127 - c));
   }
   static constexpr int key_infinite = 0x7f800000;
   static __device__ __forceinline__ ff infinite() { return ff_of(__int_as_float(0x7f800000)); }
@@ -881,7 +882,10 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
   }
   __syncthreads();
   // largest of k numbers >= 0 (or -1), column in the low bits; every warp finds
-  // it by itself
+  // it by itself.  Of equal columns the first is the pivot, and of equal values the
+  // first row's is kept: where a cap cuts a cluster of orthogonal columns of equal
+  // norm, the branch that survives is the first one, which is the branch that a
+  // gradient's states share (the last one has no overlap with them).
   auto top_key = [&](int k) {
     int key = -1;
     for (int c = lane_id(); c < k; c += 32) key = max(key, K::key(nr[c], c));
@@ -914,13 +918,14 @@ static __device__ __noinline__ int svd_small(int m, int n, const cplx<T> *A, cpl
     __syncthreads();
     const int k0 = top_key(n);
     finite = k0 < K::key_infinite;
-    neg = K::eps * K::eps * K::value(nr[k0 & 127]);
-    rest = min(cutoff * cutoff / 256, eps_t * cutoff) * K::value(nr[k0 & 127]);
+    const R top = K::value(nr[127 - (k0 & 127)]);
+    neg = K::eps * K::eps * top;
+    rest = min(cutoff * cutoff / 256, eps_t * cutoff) * top;
     __syncthreads();
     if (tid() < nthr && finite) {
       for (int j = 0; j < steps; ++j) {
         const int key = top_key(n);
-        const int p = key & 127;
+        const int p = 127 - (key & 127);
         const S nx2 = key < 0 ? K::of(0) : nr[p];
         left = K::value(nx2) * (n - j);
         if (!(K::value(nx2) > neg) || left <= rest) break;  // what is left is dropped or below rounding

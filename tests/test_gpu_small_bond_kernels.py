@@ -161,6 +161,17 @@ def test_weight_of_the_remainder(libs, threads, precision, small, kept, m, n):
 
 
 @pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("m,n", [(2, 2), (8, 4), (20, 16), (128, 128)])
+def test_first_of_equal_columns_is_kept(libs, precision, m, n):
+    """A cap that cuts a cluster of orthogonal columns of equal norm keeps the first."""
+    a = np.zeros((m, n), dtype=NP[precision])
+    a[np.arange(n) * (m // n), np.arange(n)] = 0.5j
+    _, v, _, keep, _, fail = svd(libs[256], precision, False, a, 1e-6, 1)
+    assert fail == 0 and keep == 1
+    assert np.array_equal(np.abs(v[:, 0]), np.eye(n)[0])
+
+
+@pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("delta", [0.0, 1e-3])
 def test_keep_count(libs, precision, delta):
     """The keep rule on squared values: those above the cutoff, and at most the cap
